@@ -450,8 +450,8 @@ pce_status pce_schedule_lpt(const double* cost, int n, int lanes, int* lane_of, 
  *     column-factor slots: the row pass and the column pass of one slot at a
  *     time, so that one slot's intermediate and the accumulator fit in L2);
  *   - row-pass variant (2D): 0 = block Stockham rows, the adjoint with the
- *     next term's data prefetched into registers (2 CTAs per SM), 1 = block
- *     Stockham rows without prefetch (3 CTAs per SM), 2 = variant 1 with the
+ *     next term's data prefetched into registers (512 threads per SM), 1 = block
+ *     Stockham rows without prefetch (768 threads per SM), 2 = variant 1 with the
  *     forward's windowed R2C run by row pairs (each pair's rows loaded once
  *     for all the terms or slots whose box holds them) and, for rows of 1024
  *     or 512 points, the plain row transforms (the adjoint's input R2C and the

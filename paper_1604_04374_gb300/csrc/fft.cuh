@@ -204,9 +204,27 @@ __device__ __forceinline__ void load_tw(float2 (&t)[kR - 1], int j, const float2
     }
 }
 
+// Barrier among the threads that share one FFT's buffers.  kGroupSync: the T
+// threads of one row-layout FFT (threadIdx.x / T is the same for all of them):
+// a warp barrier up to 32 threads, the CTA barrier above.  kCtaSync: the whole
+// CTA, for the column layout (every warp holds threads of every FFT) and for
+// callers that read another FFT's buffers between two of their own.
+enum FftSync { kCtaSync = 0, kGroupSync = 1 };
+
+template <int SY, int T>
+__device__ __forceinline__ void fft_sync() {
+    if constexpr (SY == kCtaSync) {
+        __syncthreads();
+    } else if constexpr (T <= 32) {
+        __syncwarp();
+    } else {
+        __syncthreads();
+    }
+}
+
 // Stage S of the FFT and, by recursion, every later stage.  t holds this
 // stage's twiddles (unused for S = 0).
-template <int N, int S, bool INV, int L>
+template <int N, int S, bool INV, int L, int SY>
 __device__ __forceinline__ void fft_stage(float2 (&v)[kR], int j, float2* b0, float2* b1,
                                           const float2 (&t)[kR - 1], const float2* __restrict__ tw) {
     using P = FftPlan<N>;
@@ -251,7 +269,7 @@ __device__ __forceinline__ void fft_stage(float2 (&v)[kR], int j, float2* b0, fl
     if constexpr (!LAST) {
         float2 tn[kR - 1];
         load_tw<N, S + 1>(tn, j, tw);
-        __syncthreads();
+        fft_sync<SY, T>();
         if constexpr (L == kColLayout && T % 8 == 0) {
             const int pj = xaddr<L, S>(j);
 #pragma unroll
@@ -268,20 +286,21 @@ __device__ __forceinline__ void fft_stage(float2 (&v)[kR], int j, float2* b0, fl
 #pragma unroll
             for (int r = 0; r < kR; ++r) v[r] = buf[xaddr<L, S>(j + r * T)];
         }
-        fft_stage<N, S + 1, INV, L>(v, j, b0, b1, tn, tw);
+        fft_stage<N, S + 1, INV, L, SY>(v, j, b0, b1, tn, tw);
     }
 }
 
 // Complex FFT of N points held as v[r] = x[j + r*T] by threads j = 0..T-1.
 // b0, b1: two shared buffers of pad_len(N) float2 private to this FFT.
-// Begins with a CTA barrier so that the buffers may be reused freely by the
-// caller between FFTs.  All threads of the CTA must call it.
-template <int N, bool INV, int L = kRowLayout>
+// Begins with a barrier so that the buffers may be reused freely by the
+// caller between FFTs.  All threads that the barrier SY names must call it.
+template <int N, bool INV, int L = kRowLayout, int SY = kCtaSync>
 __device__ __forceinline__ void fft(float2 (&v)[kR], int j, float2* b0, float2* b1,
                                     const float2* __restrict__ tw) {
+    static_assert(SY == kCtaSync || L == kRowLayout, "a group's threads are consecutive in the row layout only");
     float2 t0[kR - 1];
-    __syncthreads();
-    fft_stage<N, 0, INV, L>(v, j, b0, b1, t0, tw);
+    fft_sync<SY, FftPlan<N>::T>();
+    fft_stage<N, 0, INV, L, SY>(v, j, b0, b1, t0, tw);
 }
 
 }  // namespace pce

@@ -78,6 +78,22 @@ __device__ __forceinline__ int wrap(int i, int n) { return i & (n - 1); }
 // next item are loaded before the FFT of the current one.
 constexpr int kRowIters = 1;
 
+// Threads of a row-pass CTA and FFTs in it.  From 512 points on (64 threads and
+// more an FFT) a CTA is one FFT: its barriers then hold up nobody else, and an SM
+// keeps as many of them as registers allow.  Up to 256 points an FFT lies inside one
+// warp and needs warp barriers only; four warps a CTA keep the CTA count low.
+// Measured, all passes of an apply, against 256-thread CTAs with CTA barriers:
+// 128 x 512, m = 6, 24 right-hand sides, adjoint structure 81.9 -> 68.9 us (128-thread
+// CTAs 70.5); 1024^2 separable, m = 16, 8 right-hand sides, both directions 504.8 ->
+// 490.6 us; sectioned 2048^2 (rows of 256 points) 984 -> 935 us (64-thread CTAs 954).
+// Named barriers inside 256-thread CTAs were slower than either (93.3 us).
+template <int NX>
+struct RowCfg {
+    static constexpr int T = NX / kR;
+    static constexpr int NT = T >= 64 ? T : 128;
+    static constexpr int FPC = NT / T;
+};
+
 template <typename WT>
 struct RowItem {
     int k, la, lb;
@@ -146,14 +162,14 @@ __device__ __forceinline__ void row_load(float2 (&v)[kR], const RowItem<WT>& it,
 }
 
 template <int NX, bool WINDOW, typename WT = float>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(RowCfg<NX>::NT)
 k_rows_r2c(const float* __restrict__ src, long long src_bstride, int nrows,
            const WT* __restrict__ wbox, const Box* __restrict__ box,
            const int2* __restrict__ items, int nitems,
            float2* __restrict__ dst, long long dst_bstride, long long dst_kstride,
            const float2* __restrict__ tw) {
     constexpr int T = NX / kR;
-    constexpr int FPC = 256 / T;
+    constexpr int FPC = RowCfg<NX>::FPC;
     constexpr int NXh = NX / 2;
     __shared__ float2 sbuf[FPC * fft_region(NX)];
     const int slot = threadIdx.x / T;
@@ -175,14 +191,14 @@ k_rows_r2c(const float* __restrict__ src, long long src_bstride, int nrows,
             nxt = row_item<NX, WINDOW, WT>(first + (it + 1) * FPC, nitems, srcb, nrows, wbox, box, items);
             row_load<NX, WINDOW, WT>(vn, nxt, j);
         }
-        fft<NX, false>(v, j, b0, b1, tw);
+        fft<NX, false, kRowLayout, kGroupSync>(v, j, b0, b1, tw);
 
         // split the spectra of the two real rows
         float2* xs = b0;
-        __syncthreads();
+        fft_sync<kGroupSync, T>();
 #pragma unroll
         for (int r = 0; r < kR; ++r) xs[padi(j + r * T)] = v[r];
-        __syncthreads();
+        fft_sync<kGroupSync, T>();
         float2* da = dst + b * dst_bstride + cur.k * dst_kstride + (long long)cur.la * NXh;
         float2* db = dst + b * dst_bstride + cur.k * dst_kstride + (long long)cur.lb * NXh;
 #pragma unroll
@@ -214,16 +230,16 @@ k_rows_r2c(const float* __restrict__ src, long long src_bstride, int nrows,
 // kptr/klist of the adjoint row pass -- writing Z[b][k] rows (row - r0 of the
 // box), as k_rows_r2c<NX, true> does item by item.  The separable plans'
 // slots share every row, so the loads of u are amortised over the slots
-// instead of repeated per slot.  Grid (ceil(npairs / FPC), batch), 256
-// threads, 64 registers (4 CTAs per SM).
+// instead of repeated per slot.  Grid (ceil(npairs / FPC), batch), RowCfg::NT
+// threads, 64 registers (1024 threads per SM).
 template <int NX, typename WT = float>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(RowCfg<NX>::NT, 1024 / RowCfg<NX>::NT)
 k_rows_r2c_pairs(const float* __restrict__ src, long long src_bstride, int nrows, const WT* __restrict__ wbox,
                  const Box* __restrict__ box, const int* __restrict__ kptr, const int* __restrict__ klist,
                  float2* __restrict__ dst, long long dst_bstride, long long dst_kstride,
                  const float2* __restrict__ tw) {
     constexpr int T = NX / kR;
-    constexpr int FPC = 256 / T;
+    constexpr int FPC = RowCfg<NX>::FPC;
     constexpr int NXh = NX / 2;
     __shared__ float2 sbuf[FPC * fft_region(NX)];
     const int slot = threadIdx.x / T;
@@ -271,13 +287,13 @@ k_rows_r2c_pairs(const float* __restrict__ src, long long src_bstride, int nrows
             const bool in = cc < bx.nc;
             v[r] = make_float2(va && in ? ldw(wa + cc) * ua[r] : 0.f, vb && in ? ldw(wb + cc) * ub[r] : 0.f);
         }
-        fft<NX, false>(v, j, b0, b1, tw);
+        fft<NX, false, kRowLayout, kGroupSync>(v, j, b0, b1, tw);
         // split the spectra of the two real rows
         float2* xs = b0;
-        __syncthreads();
+        fft_sync<kGroupSync, T>();
 #pragma unroll
         for (int r = 0; r < kR; ++r) xs[padi(j + r * T)] = v[r];
-        __syncthreads();
+        fft_sync<kGroupSync, T>();
         float2* da = dst + b * dst_bstride + k * dst_kstride + (long long)la * NXh;
         float2* db = dst + b * dst_bstride + k * dst_kstride + (long long)lb * NXh;
 #pragma unroll
@@ -322,12 +338,12 @@ __device__ __forceinline__ float2 load_half_h(const HT* p, int f, float s) {
 }
 
 template <int NX>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(RowCfg<NX>::NT)
 k_rows_c2r(const float2* __restrict__ src, long long src_bstride, int nrows,
            float* __restrict__ dst, long long dst_bstride, float scale,
            const float2* __restrict__ tw) {
     constexpr int T = NX / kR;
-    constexpr int FPC = 256 / T;
+    constexpr int FPC = RowCfg<NX>::FPC;
     constexpr int NXh = NX / 2;
     __shared__ float2 sbuf[FPC * fft_region(NX)];
     const int slot = threadIdx.x / T;
@@ -348,7 +364,7 @@ k_rows_c2r(const float2* __restrict__ src, long long src_bstride, int nrows,
         const float2 xb = vb ? load_half<NX>(pb, f) : make_float2(0.f, 0.f);
         v[r] = make_float2(xa.x - xb.y, xa.y + xb.x);
     }
-    fft<NX, true>(v, j, b0, b1, tw);
+    fft<NX, true, kRowLayout, kGroupSync>(v, j, b0, b1, tw);
     float* ya = dst + b * dst_bstride + (long long)la * NX;
     float* yb = dst + b * dst_bstride + (long long)lb * NX;
 #pragma unroll
@@ -392,18 +408,18 @@ __device__ __forceinline__ void adj_load(float2 (&v)[kR], float (&wa)[kR], float
 }
 
 // RV = 0: the next term's Q rows and window values are prefetched into
-// registers during the current term's FFT (128 registers, 2 CTAs per SM);
-// RV = 1: no prefetch, 80 registers, 3 CTAs per SM (more warps hide the
+// registers during the current term's FFT (128 registers, 512 threads per SM);
+// RV = 1: no prefetch, 80 registers, 768 threads per SM (more warps hide the
 // loads instead).  The autotuner picks one per plan.
 template <int NX, typename WT = float, int RV = 0>
-__global__ void __launch_bounds__(256, RV == 1 ? 3 : 1)
+__global__ void __launch_bounds__(RowCfg<NX>::NT, RV == 1 ? 768 / RowCfg<NX>::NT : 1)
 k_rows_adj(const float2* __restrict__ Q, long long q_bstride, long long q_kstride, int nrows,
            const WT* __restrict__ wbox, const Box* __restrict__ box,
            const int* __restrict__ kptr, const int* __restrict__ klist,
            float* __restrict__ dst, long long dst_bstride, float scale,
            const float2* __restrict__ tw, int kmin, int kmax, int accumulate) {
     constexpr int T = NX / kR;
-    constexpr int FPC = 256 / T;
+    constexpr int FPC = RowCfg<NX>::FPC;
     constexpr int NXh = NX / 2;
     __shared__ float2 sbuf[FPC * fft_region(NX)];
     const int slot = threadIdx.x / T;
@@ -465,7 +481,7 @@ k_rows_adj(const float2* __restrict__ Q, long long q_bstride, long long q_kstrid
     if constexpr (RV == 1) {
         for (int t = 0; t < nk; ++t) {
             adj_load<NX, WT>(v, wa, wb, term(t), j);
-            fft<NX, true>(v, j, b0, b1, tw);
+            fft<NX, true, kRowLayout, kGroupSync>(v, j, b0, b1, tw);
 #pragma unroll
             for (int r = 0; r < kR; ++r) {
                 acc[r].x = fmaf(wa[r], v[r].x, acc[r].x);
@@ -479,7 +495,7 @@ k_rows_adj(const float2* __restrict__ Q, long long q_bstride, long long q_kstrid
             float wan[kR], wbn[kR];
             const bool more = t + 1 < nk;
             if (more) adj_load<NX, WT>(vn, wan, wbn, term(t + 1), j);
-            fft<NX, true>(v, j, b0, b1, tw);
+            fft<NX, true, kRowLayout, kGroupSync>(v, j, b0, b1, tw);
 #pragma unroll
             for (int r = 0; r < kR; ++r) {
                 acc[r].x = fmaf(wa[r], v[r].x, acc[r].x);
@@ -932,12 +948,12 @@ k_cols_grad_h(const float2* __restrict__ Z, long long z_bstride, long long z_kst
 // dw: grid (ceil(npairs / FPC), m).  Qf: [nb][m][nrows][NXh] packed row spectra
 // of conj(hhat_k) . R_b (every row).  dw: [m][nrows][NX]; accumulate adds.
 template <int NX>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(RowCfg<NX>::NT)
 k_rows_grad_w(const float2* __restrict__ Qf, long long q_bstride, long long q_kstride, int nrows,
               int nb, const float* __restrict__ u, long long u_bstride, float* __restrict__ dw,
               float scale, int accumulate, const float2* __restrict__ tw) {
     constexpr int T = NX / kR;
-    constexpr int FPC = 256 / T;
+    constexpr int FPC = RowCfg<NX>::FPC;
     constexpr int NXh = NX / 2;
     __shared__ float2 sbuf[FPC * fft_region(NX)];
     const int slot = threadIdx.x / T;
@@ -975,7 +991,7 @@ k_rows_grad_w(const float2* __restrict__ Qf, long long q_bstride, long long q_ks
         float2 vn[kR];
         float uan[kR], ubn[kR];
         if (more) load(b + 1, vn, uan, ubn);
-        fft<NX, true>(v, j, b0, b1, tw);
+        fft<NX, true, kRowLayout, kGroupSync>(v, j, b0, b1, tw);
 #pragma unroll
         for (int r = 0; r < kR; ++r) {
             acc[r].x = fmaf(ua[r], v[r].x, acc[r].x);

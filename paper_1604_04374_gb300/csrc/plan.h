@@ -65,7 +65,7 @@ struct pce_plan {
                                 // 2 (separable plans) one-warp with the warp state in tensor memory,
                                 // 3 the same with pruned column transforms (sep_prune),
                                 // 4 variant 2 run slot by slot (row and column pass per slot)
-    int row_variant = 0;        // adjoint row pass: 0 register prefetch, 1 none (3 CTAs per SM)
+    int row_variant = 0;        // adjoint row pass: 0 register prefetch, 1 none (768 threads per SM)
     double tuned_ms = 0.0;      // measured ms per right-hand side (forward + adjoint) / 2
     std::vector<double> tune_log;   // (chunk, col variant, row variant, ms per apply) per timed candidate
     long long zalloc = 0;   // Z scratch per right-hand side (float2)

@@ -5,11 +5,18 @@
 
 namespace pce {
 
-int rows_pairs_per_cta(int nx) { return 256 / (nx / kR); }
-int rows_grad_pairs_per_cta(int nx) { return 256 / (nx / kR); }
-int rows_r2c_items_per_cta(int nx) { return kRowIters * (256 / (nx / kR)); }
-
 #define PCE_ROW_SIZES(X) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048)
+
+int rows_pairs_per_cta(int nx) {
+    switch (nx) {
+#define X(N) case N: return RowCfg<N>::FPC;
+        PCE_ROW_SIZES(X)
+#undef X
+    }
+    return 1;
+}
+int rows_grad_pairs_per_cta(int nx) { return rows_pairs_per_cta(nx); }
+int rows_r2c_items_per_cta(int nx) { return kRowIters * rows_pairs_per_cta(nx); }
 
 cudaError_t launch_rows_r2c(int nx, bool window, dim3 grid, cudaStream_t s,
                             const float* src, long long src_bstride, int nrows,
@@ -21,17 +28,17 @@ cudaError_t launch_rows_r2c(int nx, bool window, dim3 grid, cudaStream_t s,
 #define X(N)                                                                                   \
     case N:                                                                                    \
         if (window && lowp)                                                                    \
-            k_rows_r2c<N, true, bf16><<<grid, 256, 0, s>>>(src, src_bstride, nrows,            \
+            k_rows_r2c<N, true, bf16><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, nrows,            \
                                                           static_cast<const bf16*>(wbox), box,  \
                                                           items, nitems, dst, dst_bstride,     \
                                                           dst_kstride, tw);                    \
         else if (window)                                                                       \
-            k_rows_r2c<N, true, float><<<grid, 256, 0, s>>>(src, src_bstride, nrows,           \
+            k_rows_r2c<N, true, float><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, nrows,           \
                                                            static_cast<const float*>(wbox), box, \
                                                            items, nitems, dst, dst_bstride,    \
                                                            dst_kstride, tw);                   \
         else                                                                                   \
-            k_rows_r2c<N, false, float><<<grid, 256, 0, s>>>(src, src_bstride, nrows, nullptr,  \
+            k_rows_r2c<N, false, float><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, nrows, nullptr,  \
                                                             box, items, nitems, dst,           \
                                                             dst_bstride, dst_kstride, tw);     \
         break;
@@ -55,11 +62,11 @@ cudaError_t launch_rows_r2c_pairs(int nx, int nb, cudaStream_t s, const float* s
         const int fpc = rows_pairs_per_cta(N);                                                    \
         const dim3 grid((npairs + fpc - 1) / fpc, nb);                                            \
         if (lowp)                                                                                 \
-            k_rows_r2c_pairs<N, bf16><<<grid, 256, 0, s>>>(src, src_bstride, nrows,                \
+            k_rows_r2c_pairs<N, bf16><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, nrows,                \
                                                          static_cast<const bf16*>(wbox), box, kptr, \
                                                          klist, dst, dst_bstride, dst_kstride, tw); \
         else                                                                                      \
-            k_rows_r2c_pairs<N, float><<<grid, 256, 0, s>>>(src, src_bstride, nrows,               \
+            k_rows_r2c_pairs<N, float><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, nrows,               \
                                                           static_cast<const float*>(wbox), box, kptr, \
                                                           klist, dst, dst_bstride, dst_kstride, tw); \
         break;                                                                                    \
@@ -78,7 +85,7 @@ cudaError_t launch_rows_c2r(int nx, dim3 grid, cudaStream_t s, const float2* src
     switch (nx) {
 #define X(N)                                                                                  \
     case N:                                                                                   \
-        k_rows_c2r<N><<<grid, 256, 0, s>>>(src, src_bstride, nrows, dst, dst_bstride, scale, tw); \
+        k_rows_c2r<N><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, nrows, dst, dst_bstride, scale, tw); \
         break;
         PCE_ROW_SIZES(X)
 #undef X
@@ -98,19 +105,19 @@ cudaError_t launch_rows_adj(int nx, dim3 grid, cudaStream_t s, const float2* Q, 
 #define X(N)                                                                                   \
     case N:                                                                                    \
         if (lowp && rv)                                                                        \
-            k_rows_adj<N, bf16, 1><<<grid, 256, 0, s>>>(Q, q_bstride, q_kstride, nrows,         \
+            k_rows_adj<N, bf16, 1><<<grid, RowCfg<N>::NT, 0, s>>>(Q, q_bstride, q_kstride, nrows,         \
                                                        static_cast<const bf16*>(wbox), box,    \
                                                        kptr, klist, dst, dst_bstride, scale, tw, kmin, kmax, accumulate); \
         else if (lowp)                                                                         \
-            k_rows_adj<N, bf16, 0><<<grid, 256, 0, s>>>(Q, q_bstride, q_kstride, nrows,         \
+            k_rows_adj<N, bf16, 0><<<grid, RowCfg<N>::NT, 0, s>>>(Q, q_bstride, q_kstride, nrows,         \
                                                        static_cast<const bf16*>(wbox), box,    \
                                                        kptr, klist, dst, dst_bstride, scale, tw, kmin, kmax, accumulate); \
         else if (rv)                                                                           \
-            k_rows_adj<N, float, 1><<<grid, 256, 0, s>>>(Q, q_bstride, q_kstride, nrows,        \
+            k_rows_adj<N, float, 1><<<grid, RowCfg<N>::NT, 0, s>>>(Q, q_bstride, q_kstride, nrows,        \
                                                         static_cast<const float*>(wbox), box,  \
                                                         kptr, klist, dst, dst_bstride, scale, tw, kmin, kmax, accumulate); \
         else                                                                                   \
-            k_rows_adj<N, float, 0><<<grid, 256, 0, s>>>(Q, q_bstride, q_kstride, nrows,        \
+            k_rows_adj<N, float, 0><<<grid, RowCfg<N>::NT, 0, s>>>(Q, q_bstride, q_kstride, nrows,        \
                                                         static_cast<const float*>(wbox), box,  \
                                                         kptr, klist, dst, dst_bstride, scale, tw, kmin, kmax, accumulate); \
         break;
@@ -158,7 +165,7 @@ cudaError_t launch_rows_grad_w(int nx, dim3 grid, cudaStream_t s, const float2* 
     switch (nx) {
 #define X(N)                                                                                   \
     case N:                                                                                    \
-        k_rows_grad_w<N><<<grid, 256, 0, s>>>(Qf, q_bstride, q_kstride, nrows, nb, u, u_bstride, \
+        k_rows_grad_w<N><<<grid, RowCfg<N>::NT, 0, s>>>(Qf, q_bstride, q_kstride, nrows, nb, u, u_bstride, \
                                               dw, scale, accumulate, tw);                      \
         break;
         PCE_ROW_SIZES(X)

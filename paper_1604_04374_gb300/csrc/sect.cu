@@ -11,7 +11,7 @@ static_assert(ColCfg<1024>::C == kWColWarps, "columns per CTA of the 1024-point 
 
 int sec_rows_per_cta(int lc) {
     switch (lc) {
-#define X(N) case N: return 256 / (N / kR) > 0 ? 256 / (N / kR) : 1;
+#define X(N) case N: return RowCfg<N>::FPC;
         PCE_SEC_SIZES(X)
 #undef X
     }
@@ -35,10 +35,10 @@ void sec_r2c(bool win, dim3 grid, cudaStream_t s, const float* src, long long sr
              const WT* wbox, const SecGeom* geo, const int2* items, int nitems, float2* dst, long long dst_bstride,
              long long dst_kstride, const float2* tw) {
     if (win)
-        k_sec_r2c<N, true, WT><<<grid, 256, 0, s>>>(src, src_bstride, nyg, nxg, wbox, geo, items, nitems, dst,
+        k_sec_r2c<N, true, WT><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, nyg, nxg, wbox, geo, items, nitems, dst,
                                                     dst_bstride, dst_kstride, tw);
     else
-        k_sec_r2c<N, false, WT><<<grid, 256, 0, s>>>(src, src_bstride, nyg, nxg, wbox, geo, items, nitems, dst,
+        k_sec_r2c<N, false, WT><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, nyg, nxg, wbox, geo, items, nitems, dst,
                                                      dst_bstride, dst_kstride, tw);
 }
 
@@ -47,10 +47,10 @@ void sec_c2r(bool win, dim3 grid, cudaStream_t s, const float2* src, long long s
              const SecGeom* geo, const int2* items, int nitems, const WT* wbox, float* dst, long long dst_bstride,
              int nyg, int nxg, float scale, const float2* tw) {
     if (win)
-        k_sec_c2r<N, true, WT><<<grid, 256, 0, s>>>(src, src_bstride, src_kstride, geo, items, nitems, wbox, dst,
+        k_sec_c2r<N, true, WT><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, src_kstride, geo, items, nitems, wbox, dst,
                                                     dst_bstride, nyg, nxg, scale, tw);
     else
-        k_sec_c2r<N, false, WT><<<grid, 256, 0, s>>>(src, src_bstride, src_kstride, geo, items, nitems, wbox, dst,
+        k_sec_c2r<N, false, WT><<<grid, RowCfg<N>::NT, 0, s>>>(src, src_bstride, src_kstride, geo, items, nitems, wbox, dst,
                                                      dst_bstride, nyg, nxg, scale, tw);
 }
 

@@ -52,13 +52,13 @@ __device__ __forceinline__ int sec_col(int c0, int rc, int n, bool narrow) {
 
 // Input rows: items (k, q) take window rows 2q, 2q+1 of term k.
 template <int NX, bool WIN, typename WT = float>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(RowCfg<NX>::NT)
 k_sec_r2c(const float* __restrict__ src, long long src_bstride, int NYg, int NXg,
           const WT* __restrict__ wbox, const SecGeom* __restrict__ geo, const int2* __restrict__ items,
           int nitems, float2* __restrict__ dst, long long dst_bstride, long long dst_kstride,
           const float2* __restrict__ tw) {
     constexpr int T = NX / kR;
-    constexpr int FPC = 256 / T;
+    constexpr int FPC = RowCfg<NX>::FPC;
     constexpr int NXh = NX / 2;
     __shared__ float2 sbuf[FPC * fft_region(NX)];
     const int slot = threadIdx.x / T;
@@ -94,11 +94,11 @@ k_sec_r2c(const float* __restrict__ src, long long src_bstride, int NYg, int NXg
         }
         v[r] = make_float2(xa, xb);
     }
-    fft<NX, false>(v, j, b0, b1, tw);
-    __syncthreads();
+    fft<NX, false, kRowLayout, kGroupSync>(v, j, b0, b1, tw);
+    fft_sync<kGroupSync, T>();
 #pragma unroll
     for (int r = 0; r < kR; ++r) b0[padi(j + r * T)] = v[r];
-    __syncthreads();
+    fft_sync<kGroupSync, T>();
     float2* da = dst + b * dst_bstride + kq.x * dst_kstride + (long long)ia * NXh;
     float2* db = dst + b * dst_bstride + kq.x * dst_kstride + (long long)ib * NXh;
 #pragma unroll
@@ -238,13 +238,13 @@ kw_sec_cols(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
 // Output rows: items (k, q) take output-window rows 2q, 2q+1 of term k; C2R,
 // times scale (and the window in the adjoint), added into the grid.
 template <int NX, bool WIN, typename WT = float>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(RowCfg<NX>::NT)
 k_sec_c2r(const float2* __restrict__ src, long long src_bstride, long long src_kstride,
           const SecGeom* __restrict__ geo, const int2* __restrict__ items, int nitems,
           const WT* __restrict__ wbox, float* __restrict__ dst, long long dst_bstride, int NYg, int NXg,
           float scale, const float2* __restrict__ tw) {
     constexpr int T = NX / kR;
-    constexpr int FPC = 256 / T;
+    constexpr int FPC = RowCfg<NX>::FPC;
     constexpr int NXh = NX / 2;
     __shared__ float2 sbuf[FPC * fft_region(NX)];
     const int slot = threadIdx.x / T;
@@ -285,7 +285,7 @@ k_sec_c2r(const float2* __restrict__ src, long long src_bstride, long long src_k
             wb[r] = (in && vb) ? ldw(wbox + g.woff + (long long)rb * g.ldw + rc) : 0.f;
         }
     }
-    fft<NX, true>(v, j, b0, b1, tw);
+    fft<NX, true, kRowLayout, kGroupSync>(v, j, b0, b1, tw);
     float* db = dst + b * dst_bstride;
     float* ya = db + (long long)(((g.r0 + ra) % NYg + NYg) % NYg) * NXg;
     float* yb = db + (long long)(((g.r0 + rb) % NYg + NYg) % NYg) * NXg;
