@@ -458,6 +458,8 @@ pce_status pce_schedule_lpt(const double* cost, int n, int lanes, int* lane_of, 
  *     forward's output C2R) by one warp per row pair;
  *   - right-hand sides per launch: powers of two up to the plan's scratch
  *     chunk (2D plans and 1D plans above 8192 points).
+ * A plan that was never tuned runs column variant 2 where it has it, else 0,
+ * row variant 1 (2D), and as many right-hand sides per launch as its scratch holds.
  * 1D plans up to 8192 points have nothing to choose and are only timed.  The
  * choice changes no value an apply computes beyond rounding order (the
  * column variants' FFTs round differently).  cache_path (may be NULL): a

@@ -891,6 +891,11 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
     if ((flags & PCE_FLAG_SECTIONED) && (st = setup_sectioned(p, h, s))) return bail(st);
     cudaError_t e = cudaStreamSynchronize(s);
     if (e) return bail(fail(PCE_ERR_CUDA, "plan set-up: %s", cudaGetErrorString(e)));
+    // untuned row variant: the adjoint rows without register prefetch.  128 x 512, m = 6,
+    // 24 right-hand sides 68.8 -> 65.4 us; 256-task uneven batch 3.20 -> 2.91 ms with the
+    // separable default below.  Variant 2 (forward rows by row pairs) loses on small grids
+    // (256^2, one right-hand side: 20.5 -> 28.7 us) and stays the autotuner's to pick.
+    if (ndims == 2) p->row_variant = 1;
     *out = p;
     return PCE_OK;
 }
@@ -1035,6 +1040,9 @@ pce_status setup_separable(pce_plan* p, const float* wy, const float* wx, cudaSt
     p->zk_s = zk;
     p->sep = true;
     p->sep_prune = prune;
+    // untuned column variant: the warp state in tensor memory (1024^2, m = 16, one
+    // right-hand side, both directions: 222 us with it in registers, 132 us so)
+    p->col_variant = 2;
     return PCE_OK;
 }
 

@@ -59,7 +59,8 @@ struct pce_plan {
     float2* scrA = nullptr;
     int nrmax = 0;
     int bchunk = 1;             // right-hand sides the plan's scratch holds
-    // autotuned choices (pce_plan_autotune): 0 = default
+    // autotuned choices (pce_plan_autotune); untuned plans: run_chunk 0 (all the scratch holds),
+    // column variant 2 where separable kernels exist, row variant 1
     int run_chunk = 0;          // right-hand sides per launch, <= bchunk
     int col_variant = 0;        // columns of 1024: 0 one-warp four-step, 1 radix-8 Stockham,
                                 // 2 (separable plans) one-warp with the warp state in tensor memory,
