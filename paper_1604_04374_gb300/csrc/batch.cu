@@ -274,6 +274,7 @@ extern "C" pce_status pce_batch_create(pce_batch_t* out, const pce_task* tasks, 
         s.chunk = ch[i];
         s.Z = base;
         s.A = base ? base + round_up(zs[i] * ch[i], 32) : nullptr;
+        s.beside = lanes > 1 && n > 1;
     }
     if ((st = make_lanes(lanes, b->streams, b->fork, b->join))) {
         delete b;
@@ -384,6 +385,7 @@ extern "C" pce_status pce_apply_batch(const pce_task* tasks, int n, void* stream
     for (int i = 0; i < n; ++i) {
         order[lane_of_group[group[i]]].push_back(i);
         scr[i] = pce_rt::plan_scratch(tasks[i].plan);
+        scr[i].beside = lanes > 1;
     }
     std::lock_guard<std::mutex> lock(g_pool_mutex);
     Pool& pool = g_pools[device];

@@ -208,8 +208,11 @@ __device__ __forceinline__ void load_tw(float2 (&t)[kR - 1], int j, const float2
 // threads of one row-layout FFT (threadIdx.x / T is the same for all of them):
 // a warp barrier up to 32 threads, the CTA barrier above.  kCtaSync: the whole
 // CTA, for the column layout (every warp holds threads of every FFT) and for
-// callers that read another FFT's buffers between two of their own.
-enum FftSync { kCtaSync = 0, kGroupSync = 1 };
+// callers that read another FFT's buffers between two of their own.  kNamedSync:
+// a warp barrier up to 32 threads, else barrier 1 + threadIdx.x / T of the T threads:
+// the FFTs of a large CTA run independently (it reserves every named barrier of
+// the CTA, so it is for kernels with one or two CTAs per SM).
+enum FftSync { kCtaSync = 0, kGroupSync = 1, kNamedSync = 2 };
 
 template <int SY, int T>
 __device__ __forceinline__ void fft_sync() {
@@ -217,6 +220,8 @@ __device__ __forceinline__ void fft_sync() {
         __syncthreads();
     } else if constexpr (T <= 32) {
         __syncwarp();
+    } else if constexpr (SY == kNamedSync) {
+        asm volatile("bar.sync %0, %1;\n" ::"r"(1 + (int)threadIdx.x / T), "n"(T) : "memory");
     } else {
         __syncthreads();
     }

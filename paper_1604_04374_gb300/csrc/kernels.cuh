@@ -23,6 +23,7 @@
 // A[f] = (Z[f] + conj Z[-f]) / 2, B[f] = (Z[f] - conj Z[-f]) / (2i).
 #pragma once
 
+#include "cluster.cuh"
 #include "fft.cuh"
 
 namespace pce {
@@ -55,6 +56,8 @@ struct SepTerms {
     const int* korder = nullptr;   // [nterms] the terms to run, grouped by slot
     int nterms = 0;
     const int* kq0 = nullptr;      // [m] pruned column kernels: wy_k's rows lie in [32 kq0, 32 kq0 + 512)
+    const int* slot_toff = nullptr;   // [nslots + 1] slot j's terms are korder[slot_toff[j] .. slot_toff[j + 1])
+    int nslots = 0;
     // slot-by-slot schedule of the tensor-memory column kernels: the terms
     // korder[t0 .. t1) of this pass (t1 < 0: all) and the pass's mode bits
     int t0 = 0, t1 = -1, mode = 0;
@@ -558,6 +561,9 @@ __device__ __forceinline__ void load_col(float2 (&v)[kR], const float2* __restri
     }
 }
 
+// Share z of n of the terms [0, count) for CTA z of n.
+__device__ __forceinline__ int share_beg(int count, int z, int n) { return (int)((long long)count * z / n); }
+
 // F2: forward column pass.  Grid (batch, NXh / C): the right-hand sides of a
 // column tile are neighbours in launch order and share hhat_k through L2.
 // hh: [m][NY][NXh] (column 0 = DC column spectrum), hN: [m][NY] (Nyquist).
@@ -666,8 +672,9 @@ k_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstrid
 // G1b + G2: adjoint column pass.  Column FFT of V once; per k the product
 // with conj(hhat_k), an inverse column FFT, and a store of the box rows only
 // (FULL: of every row, Q[b][k][NY][NXh], for the window gradient).
-// Grid (batch, NXh / C).  The next term's spectrum is loaded before the
-// current inverse FFT.
+// Grid (batch, NXh / C, split): CTA z of a column tile takes its share of the
+// terms (each forms the FFT of V itself; the outputs are separate).  The next
+// term's spectrum is loaded before the current inverse FFT.
 template <int NY, bool FULL, typename HT = float2>
 __global__ void __launch_bounds__(ColCfg<NY>::NT)
 k_cols_adj(const float2* __restrict__ V, long long v_bstride,
@@ -696,10 +703,11 @@ k_cols_adj(const float2* __restrict__ V, long long v_bstride,
 #pragma unroll
     for (int r = 0; r < kR; ++r)
         vv[r] = cv ? __ldg(&Vb[(long long)(j + r * T) * NXh + col]) : make_float2(0.f, 0.f);
-    int k = 0;
-    while (k < m && !FULL && box[k].nr == 0) ++k;
+    const int kend = share_beg(m, blockIdx.z + 1, gridDim.z);
+    int k = share_beg(m, blockIdx.z, gridDim.z);
+    while (k < kend && !FULL && box[k].nr == 0) ++k;
     float2 hv[kR];
-    if (k < m) {
+    if (k < kend) {
         const HT* hk = hh + (long long)k * NY * NXh;
         const float sk = hscale_of<HT>(hscale, k);
 #pragma unroll
@@ -714,9 +722,9 @@ k_cols_adj(const float2* __restrict__ V, long long v_bstride,
         }
         __syncthreads();
     }
-    while (k < m) {
+    while (k < kend) {
         int kn = k + 1;
-        while (kn < m && !FULL && box[kn].nr == 0) ++kn;
+        while (kn < kend && !FULL && box[kn].nr == 0) ++kn;
         const Box bx = box[k];
         float2 p[kR];
 #pragma unroll
@@ -734,7 +742,7 @@ k_cols_adj(const float2* __restrict__ V, long long v_bstride,
                 p[r] = cmulc(vv[r], hv[r]);
             }
         }
-        if (kn < m) {
+        if (kn < kend) {
             const HT* hk = hh + (long long)kn * NY * NXh;
             const float sk = hscale_of<HT>(hscale, kn);
 #pragma unroll
@@ -1027,6 +1035,12 @@ struct Cfg1d {
                                   : ((256 / T) > 0 ? (256 / T) : 1);
     static constexpr int NT = T * G;
     static constexpr int SMEM = G * fft_region(N) * (int)sizeof(float2);
+    // slots whose FFTs run independently of one another: whole warps, with barriers
+    // of their own (named ones in the wide CTAs, one or two of which fill an SM), so
+    // that slots without a pair stop and one FFT of V serves the CTA.  N = 2048,
+    // m = 11, 300 right-hand sides, adjoint: 26.6 -> 22.5 us
+    static constexpr bool OWN = G == 1 || T == 32 || (T > 32 && WIDE);
+    static constexpr int SY = OWN && G > 1 ? kNamedSync : kGroupSync;
 };
 
 // Ask L2 for the `bytes` at p (one 128-byte line per thread of the CTA), so that
@@ -1037,28 +1051,44 @@ __device__ __forceinline__ void prefetch_l2_block(const void* p, long long bytes
         asm volatile("prefetch.global.L2 [%0];\n" ::"l"(c + o));
 }
 
-// y_b = (1/N) C2R( sum_k hhat_k . R2C(w_k . u_b) ).  One CTA per b; each
-// slot takes pairs of terms (w_k u + i w_{k+1} u in one complex FFT) and
-// accumulates the half spectrum in registers; the slots' sums are reduced in
-// shared memory and one inverse FFT follows.  hp: [m][N/2] packed spectra.
+// Rounds of term pairs one FFT slot runs: slot `first` of `stride` takes pairs
+// first, first + stride, ...  Independent slots stop at their last pair; the
+// others run as many rounds as their CTA's slot 0.
+template <bool OWN>
+__device__ __forceinline__ int rounds_1d(int npairs, int first, int stride, int slot0) {
+    const int f = OWN ? first : slot0;
+    return f < npairs ? (npairs - f + stride - 1) / stride : 0;
+}
+
+// y_b = (1/N) C2R( sum_k hhat_k . R2C(w_k . u_b) ).  One cluster of cl CTAs per
+// b (cl = 1: one CTA); each FFT slot takes pairs of terms (w_k u + i w_{k+1} u in
+// one complex FFT) and accumulates the half spectrum in registers; the slots'
+// sums are reduced in shared memory, the CTAs' sums by rank 0 through the
+// cluster's shared memory, and one inverse FFT follows.  hp: [m][N/2] packed
+// spectra.  The slots' FFTs use barriers of their own.
+//
+// Bound by the chain of FFTs of one slot when there are few right-hand sides:
+// the cluster shortens it to ceil(pairs / (cl G)) rounds.
 template <int N, typename WT = float, typename HT = float2, int WIDE = 0>
 __global__ void __launch_bounds__(Cfg1d<N, WIDE>::NT)
 k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
          const HT* __restrict__ hp, const float* __restrict__ hscale, int m, float* __restrict__ y, float scale,
-         const float2* __restrict__ tw) {
+         const float2* __restrict__ tw, int cl) {
     using CF = Cfg1d<N, WIDE>;
     constexpr int T = CF::T;
     constexpr int G = CF::G;
     constexpr int Nh = N / 2;
+    constexpr int SY = CF::SY;
     extern __shared__ float2 smem[];
     const int slot = threadIdx.x / T;
     const int j = threadIdx.x - slot * T;
     float2* b0 = smem + slot * fft_region(N);
     float2* b1 = b0 + pad_len(N);
-    const int b = blockIdx.x;
+    const int b = blockIdx.x / cl;
+    const int rank = cl > 1 ? cluster_rank() : 0;
     // the twiddles and spectra are read stage by stage and after the first FFT:
     // with few right-hand sides (a latency-bound launch) start them towards L2 now
-    if (gridDim.x <= 8) {
+    if (gridDim.x <= 8 * cl && rank == 0) {
         prefetch_l2_block(tw, (long long)FftPlan<N>::TWLEN * sizeof(float2));
         prefetch_l2_block(hp, (long long)m * Nh * sizeof(HT));
     }
@@ -1071,9 +1101,9 @@ k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
     for (int r = 0; r < kR / 2; ++r) acc[r] = make_float2(0.f, 0.f);
 
     const int npairs = (m + 1) / 2;
-    const int iters = (npairs + G - 1) / G;
+    const int iters = rounds_1d<CF::OWN>(npairs, rank * G + slot, cl * G, rank * G);
     for (int it = 0; it < iters; ++it) {
-        const int pr = it * G + slot;
+        const int pr = (it * cl + rank) * G + slot;
         const bool a0 = pr < npairs;
         const int k0 = 2 * pr, k1 = k0 + 1;
         const bool a1 = a0 && k1 < m;
@@ -1084,11 +1114,11 @@ k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
             v[r] = make_float2(a0 ? ldw(w + (long long)k0 * N + n) * ureg[r] : 0.f,
                                a1 ? ldw(w + (long long)k1 * N + n) * ureg[r] : 0.f);
         }
-        fft<N, false>(v, j, b0, b1, tw);
-        __syncthreads();
+        fft<N, false, kRowLayout, SY>(v, j, b0, b1, tw);
+        fft_sync<SY, T>();
 #pragma unroll
         for (int r = 0; r < kR; ++r) b0[padi(j + r * T)] = v[r];
-        __syncthreads();
+        fft_sync<SY, T>();
         if (a0) {
             const HT* h0 = hp + (long long)k0 * Nh;
             const HT* h1 = hp + (long long)(a1 ? k1 : k0) * Nh;
@@ -1116,26 +1146,38 @@ k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
             }
         }
     }
-    // reduce over slots into slot 0's second buffer (packed half spectrum)
+    // the slots' sums into slot 0's second buffer (packed half spectrum), by
+    // the whole CTA; then the other CTAs' sums by rank 0
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < kR / 2; ++r) b0[j + r * T] = acc[r];
     __syncthreads();
     float2* red = smem + pad_len(N);
-    if (slot == 0) {
-#pragma unroll
-        for (int r = 0; r < kR / 2; ++r) {
-            float2 s = smem[j + r * T];
-            for (int g = 1; g < G; ++g) s = cadd(s, smem[g * fft_region(N) + j + r * T]);
-            red[j + r * T] = s;
+    for (int f = threadIdx.x; f < Nh; f += CF::NT) {
+        float2 s = smem[f];
+        for (int g = 1; g < G; ++g) s = cadd(s, smem[g * fft_region(N) + f]);
+        red[f] = s;
+    }
+    if (cl > 1) {
+        cluster_sync();
+        if (rank == 0) {
+            for (int f = threadIdx.x; f < Nh; f += CF::NT) {
+                float2 s = red[f];
+                for (int g = 1; g < cl; ++g) s = cadd(s, cluster_ld2(cluster_map(&red[f], g)));
+                red[f] = s;
+            }
         }
+        cluster_sync();   // rank 0 has read the others' shared memory
+        if (rank != 0) return;
     }
     __syncthreads();
+    // slots that share barriers stay together in the FFT
+    if (CF::OWN && slot != 0) return;
     float2 v[kR];
 #pragma unroll
     for (int r = 0; r < kR; ++r)
         v[r] = (slot == 0) ? load_half<N>(red, j + r * T) : make_float2(0.f, 0.f);
-    fft<N, true>(v, j, b0, b1, tw);
+    fft<N, true, kRowLayout, SY>(v, j, b0, b1, tw);
     if (slot == 0) {
         float* yb = y + (long long)b * N;
 #pragma unroll
@@ -1143,45 +1185,65 @@ k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
     }
 }
 
-// x_b = (1/N) sum_k w_k . IFFT( conj(hhat_k) . FFT(v_b) ).  One CTA per b;
-// every slot forms FFT(v_b) and takes pairs of terms: the two inverse FFTs
-// of a pair are real, so they share one complex inverse FFT.
+// x_b = (1/N) sum_k w_k . IFFT( conj(hhat_k) . FFT(v_b) ).  One cluster of cl
+// CTAs per b; every CTA forms FFT(v_b) (independent slots get it from slot 0 through
+// shared memory), and its slots take pairs of terms: the two inverse FFTs of
+// a pair are real, so they share one complex inverse FFT.  The windowed sums of
+// the slots are added in shared memory, those of the CTAs through the cluster's
+// shared memory, each rank storing its part of x.
 template <int N, typename WT = float, typename HT = float2, int WIDE = 0>
 __global__ void __launch_bounds__(Cfg1d<N, WIDE>::NT)
 k_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w,
          const HT* __restrict__ hp, const float* __restrict__ hscale, int m, float* __restrict__ x, float scale,
-         const float2* __restrict__ tw) {
+         const float2* __restrict__ tw, int cl) {
     using CF = Cfg1d<N, WIDE>;
     constexpr int T = CF::T;
     constexpr int G = CF::G;
     constexpr int Nh = N / 2;
+    constexpr int SY = CF::SY;
     extern __shared__ float2 smem[];
     const int slot = threadIdx.x / T;
     const int j = threadIdx.x - slot * T;
     float2* b0 = smem + slot * fft_region(N);
     float2* b1 = b0 + pad_len(N);
-    const int b = blockIdx.x;
+    const int b = blockIdx.x / cl;
+    const int rank = cl > 1 ? cluster_rank() : 0;
     // the twiddles, spectra and windows are read stage by stage and after the
     // FFT of v: with few right-hand sides (a latency-bound launch) start them
     // towards L2 now
-    if (gridDim.x <= 8) {
+    if (gridDim.x <= 8 * cl && rank == 0) {
         prefetch_l2_block(tw, (long long)FftPlan<N>::TWLEN * sizeof(float2));
         prefetch_l2_block(hp, (long long)m * Nh * sizeof(HT));
         prefetch_l2_block(w, (long long)m * N * sizeof(WT));
     }
     const float* vb = vin + (long long)b * N;
     float2 V[kR];
+    if (!CF::OWN || slot == 0) {
 #pragma unroll
-    for (int r = 0; r < kR; ++r) V[r] = make_float2(__ldg(vb + j + r * T), 0.f);
-    fft<N, false>(V, j, b0, b1, tw);
+        for (int r = 0; r < kR; ++r) V[r] = make_float2(__ldg(vb + j + r * T), 0.f);
+        fft<N, false, kRowLayout, SY>(V, j, b0, b1, tw);
+    }
+    if (CF::OWN && G > 1) {
+        __syncthreads();
+        if (slot == 0) {
+#pragma unroll
+            for (int r = 0; r < kR; ++r) smem[j + r * T] = V[r];
+        }
+        __syncthreads();
+        if (slot != 0) {
+#pragma unroll
+            for (int r = 0; r < kR; ++r) V[r] = smem[j + r * T];
+        }
+        __syncthreads();   // read before slot 0's next FFT reuses its buffers
+    }
     float ax[kR];
 #pragma unroll
     for (int r = 0; r < kR; ++r) ax[r] = 0.f;
 
     const int npairs = (m + 1) / 2;
-    const int iters = (npairs + G - 1) / G;
+    const int iters = rounds_1d<CF::OWN>(npairs, rank * G + slot, cl * G, rank * G);
     for (int it = 0; it < iters; ++it) {
-        const int pr = it * G + slot;
+        const int pr = (it * cl + rank) * G + slot;
         const bool a0 = pr < npairs;
         const int k0 = 2 * pr, k1 = k0 + 1;
         const bool a1 = a0 && k1 < m;
@@ -1202,7 +1264,7 @@ k_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w,
             }
             p[r] = t;
         }
-        fft<N, true>(p, j, b0, b1, tw);
+        fft<N, true, kRowLayout, SY>(p, j, b0, b1, tw);
 #pragma unroll
         for (int r = 0; r < kR; ++r) {
             const int n = j + r * T;
@@ -1215,15 +1277,23 @@ k_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w,
 #pragma unroll
     for (int r = 0; r < kR; ++r) fb[j + r * T] = ax[r];
     __syncthreads();
-    if (slot == 0) {
-        float* xb = x + (long long)b * N;
-#pragma unroll
-        for (int r = 0; r < kR; ++r) {
-            float s = fb[j + r * T];
-            for (int g = 1; g < G; ++g)
-                s += reinterpret_cast<const float*>(smem + g * fft_region(N))[j + r * T];
-            xb[j + r * T] = s * scale;
+    float* xb = x + (long long)b * N;
+    float* red = reinterpret_cast<float*>(smem + pad_len(N));
+    for (int n = threadIdx.x; n < N; n += CF::NT) {
+        float s = reinterpret_cast<const float*>(smem)[n];
+        for (int g = 1; g < G; ++g) s += reinterpret_cast<const float*>(smem + g * fft_region(N))[n];
+        if (cl > 1) red[n] = s;
+        else xb[n] = s * scale;
+    }
+    if (cl > 1) {
+        cluster_sync();
+        const int part = N / cl;   // both powers of two, cl <= 8 < N
+        for (int n = rank * part + threadIdx.x; n < (rank + 1) * part; n += CF::NT) {
+            float s = 0.f;
+            for (int g = 0; g < cl; ++g) s += cluster_ld(cluster_map(&red[n], g));
+            xb[n] = s * scale;
         }
+        cluster_sync();   // every rank has read the others' shared memory
     }
 }
 

@@ -1025,7 +1025,6 @@ pce_status setup_separable(pce_plan* p, const float* wy, const float* wx, cudaSt
                                                                             (int)nxh, p->hhTr, p->hNr);
         PCE_CK(cudaGetLastError());
     }
-    PCE_CK(cudaStreamSynchronize(s));   // the host vectors die at return
     p->slot_item_off.assign(ns + 1, 0);
     p->slot_term_off.assign(ns + 1, 0);
     for (int j = 0; j < ns; ++j) {
@@ -1034,6 +1033,9 @@ pce_status setup_separable(pce_plan* p, const float* wy, const float* wx, cudaSt
         for (int k : korder) n += kslot[k] == j;
         p->slot_term_off[j + 1] = p->slot_term_off[j] + n;
     }
+    if ((st = dev_alloc(&p->d_slot_toff, (size_t)ns + 1))) return st;
+    PCE_CK(cudaMemcpyAsync(p->d_slot_toff, p->slot_term_off.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice, s));
+    PCE_CK(cudaStreamSynchronize(s));   // the host vectors die at return
     p->nslots = ns;
     p->nterms = (int)korder.size();
     p->nsitems = (int)items.size();
@@ -1470,6 +1472,17 @@ pce_status apply_plain(pce_plan_t p, const float* in, float* out, int64_t batch,
     return PCE_OK;
 }
 
+// CTAs that share a column tile's terms in the adjoint: doubled while the grid of ctas
+// column CTAs fills no more than the GPU's `per_sm` resident CTAs an SM and every CTA
+// keeps a unit of work (a term or a slot).  Beyond one wave a split only adds work, an
+// FFT of V a CTA.  Every unit's result is formed by one CTA: the same bits for any split.
+// 1024^2 separable, m = 16, one right-hand side, forward and adjoint: 223 -> 180 us.
+int col_split(long long ctas, int per_sm, int units) {
+    int n = 1;
+    while (n < pce::kMaxCluster && 2 * n <= units && ctas * 2 * n <= (long long)pce::kSms * per_sm) n *= 2;
+    return n;
+}
+
 pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, bool adjoint,
                       cudaStream_t s, const pce_rt::Scratch& scr, bool allow_timing = true) {
     TimingScope ts(allow_timing && !stream_capturing(s));
@@ -1530,11 +1543,8 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
     }
     if (p->ndims == 1) {
         e = timed(p, adjoint ? PCE_KERNEL_ADJ_1D : PCE_KERNEL_FWD_1D, s, [&] {
-            return adjoint
-                ? pce::launch_adj_1d(nx, (int)batch, s, in, wstore(p), hstore(p), p->hscale, p->lowp, m, out, scale, p->twx,
-                                     p->tw1024)
-                : pce::launch_fwd_1d(nx, (int)batch, s, in, wstore(p), hstore(p), p->hscale, p->lowp, m, out, scale, p->twx,
-                                     p->tw1024);
+            return pce::launch_1d(adjoint, nx, (int)batch, s, in, wstore(p), hstore(p), p->hscale, p->lowp, m, out,
+                                  scale, p->twx, p->tw1024);
         });
         if (e) return fail(PCE_ERR_CUDA, "1D apply launch: %s", cudaGetErrorString(e));
         return PCE_OK;
@@ -1602,6 +1612,8 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
     sept.kslot = p->d_kslot;
     sept.korder = p->d_korder;
     sept.nterms = p->nterms;
+    sept.slot_toff = p->d_slot_toff;
+    sept.nslots = p->nslots;
     // the tensor-memory kernels; variant 3 runs the pruned ones (rotated spectra),
     // which the plan has when every term allows them
     const bool prune = colv == 3 && p->sep_prune;
@@ -1620,10 +1632,18 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
     const int fpc = pce::rows_pairs_per_cta(nx);
     const int cpc = pce::cols_columns_per_cta(ny);  // same for both variants
     const int npairs = (ny + 1) / 2;
+    // column CTAs per SM, and the units the adjoint's column tile divides into.  Columns
+    // of 2048 keep a tile in one CTA; so does a batch's lane, where every further CTA
+    // repeats the FFT of V while other tasks could use the SM
+    const int col_ctas = septm ? (ny == 1024 ? 4 : 6) : warp && ny == 1024 ? 3 : warp && ny == 512 ? 5 : 4;
+    const bool whole = !adjoint || (warp && ny == 2048) || scr.beside;
+    const int col_units = whole ? 1 : sepx ? p->nslots : m;
     for (long long b0 = 0; b0 < batch && e == cudaSuccess; b0 += bal) {
         const int nb = (int)std::min<long long>(bal, batch - b0);
         const float* src = in + b0 * P;
         float* dst = out + b0 * P;
+        dim3 cgrid(nb, (nxh + cpc - 1) / cpc);
+        if (!slotwise) cgrid.z = col_split((long long)cgrid.x * cgrid.y, col_ctas, col_units);
         if (slotwise && !adjoint) {
             for (size_t a = 0; a < active.size() && e == cudaSuccess; ++a) {
                 const int j = active[a];
@@ -1640,7 +1660,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
                     });
                 if (e == cudaSuccess)
                     e = timed(p, PCE_KERNEL_COLS_FWD, s, [&] {
-                        return pce::launch_cols_fwd_sep_tm(ny, dim3(nb, (nxh + cpc - 1) / cpc), s, scr.Z, zb, p->zk_s,
+                        return pce::launch_cols_fwd_sep_tm(ny, cgrid, s, scr.Z, zb, p->zk_s,
                                                            tm_hT, tm_hN, p->d_vbox, nxh, scr.A, ab, p->tw1024,
                                                            p->d_status, p->wait_limit, p->skip_copy, sj);
                     });
@@ -1666,7 +1686,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
                 // the first pass stores V's column spectrum in place for the later ones
                 sj.mode = a == 0 ? pce::kSepSpecOut : pce::kSepSpecIn;
                 e = timed(p, PCE_KERNEL_COLS_ADJ, s, [&] {
-                    return pce::launch_cols_adj_sep_tm(ny, dim3(nb, (nxh + cpc - 1) / cpc), s, scr.A, ab, tm_hT, tm_hN,
+                    return pce::launch_cols_adj_sep_tm(ny, cgrid, s, scr.A, ab, tm_hT, tm_hN,
                                                        p->d_vbox, nxh, scr.Z, zb, p->zk_s, p->tw1024, p->d_status,
                                                        p->wait_limit, p->skip_copy, sj);
                 });
@@ -1690,10 +1710,10 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_COLS_FWD, s, [&] {
                     if (septm)
-                        return pce::launch_cols_fwd_sep_tm(ny, dim3(nb, (nxh + cpc - 1) / cpc), s, scr.Z, zb, p->zk_s,
+                        return pce::launch_cols_fwd_sep_tm(ny, cgrid, s, scr.Z, zb, p->zk_s,
                                                            tm_hT, tm_hN, p->d_vbox, nxh, scr.A, ab, p->tw1024,
                                                            p->d_status, p->wait_limit, p->skip_copy, septp);
-                    return pce::launch_cols_fwd_sep(ny, dim3(nb, (nxh + cpc - 1) / cpc), s, scr.Z, zb, p->zk_s,
+                    return pce::launch_cols_fwd_sep(ny, cgrid, s, scr.Z, zb, p->zk_s,
                                                     p->hhT, p->hN, m, p->d_vbox, nxh, scr.A, ab, p->tw1024,
                                                     p->d_status, p->wait_limit, p->skip_copy, sept);
                 });
@@ -1713,10 +1733,10 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_COLS_ADJ, s, [&] {
                     if (septm)
-                        return pce::launch_cols_adj_sep_tm(ny, dim3(nb, (nxh + cpc - 1) / cpc), s, scr.A, ab, tm_hT,
+                        return pce::launch_cols_adj_sep_tm(ny, cgrid, s, scr.A, ab, tm_hT,
                                                            tm_hN, p->d_vbox, nxh, scr.Z, zb, p->zk_s, p->tw1024,
                                                            p->d_status, p->wait_limit, p->skip_copy, septp);
-                    return pce::launch_cols_adj_sep(ny, dim3(nb, (nxh + cpc - 1) / cpc), s, scr.A, ab, p->hhT, p->hN,
+                    return pce::launch_cols_adj_sep(ny, cgrid, s, scr.A, ab, p->hhT, p->hN,
                                                     m, p->d_vbox, nxh, scr.Z, zb, p->zk_s, p->tw1024,
                                                     p->d_status, p->wait_limit, p->skip_copy, sept);
                 });
@@ -1738,7 +1758,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
                 });
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_COLS_FWD, s, [&] {
-                    return pce::launch_cols_fwd(ny, dim3(nb, (nxh + cpc - 1) / cpc), s, scr.Z, zb, zk,
+                    return pce::launch_cols_fwd(ny, cgrid, s, scr.Z, zb, zk,
                                                 hstore(p), hNstore(p), p->hscale, p->lowp, m, p->d_box, nxh, scr.A, ab, p->twy, hTstore(p), p->tw1024, p->d_status, p->wait_limit, p->skip_copy, warp,
                                                 hN2store(p), p->tw2048l);
                 });
@@ -1757,7 +1777,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
             });
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_COLS_ADJ, s, [&] {
-                    return pce::launch_cols_adj(ny, dim3(nb, (nxh + cpc - 1) / cpc), s, scr.A, ab,
+                    return pce::launch_cols_adj(ny, cgrid, s, scr.A, ab,
                                                 hstore(p), hNstore(p), p->hscale, p->lowp, m, p->d_box, nxh, scr.Z, zb, zk, p->twy, hTstore(p), p->tw1024, p->d_status, p->wait_limit, p->skip_copy, warp,
                                                 hN2store(p), p->tw2048l);
                 });

@@ -90,6 +90,7 @@ struct pce_plan {
     // sitems[slot_item_off[j] .. slot_item_off[j + 1]), its terms
     // korder[slot_term_off[j] .. slot_term_off[j + 1])
     std::vector<int> slot_item_off, slot_term_off;
+    int* d_slot_toff = nullptr; // slot_term_off on the device
     // pruned tensor-memory column kernels: every active term's row factor lies in
     // rows [32 kq0[k], 32 kq0[k] + 512) mod 1024; spectra rotated by W1024^{32 f kq0[k]}
     bool sep_prune = false;
@@ -135,7 +136,7 @@ struct pce_plan {
                         items,  kptr,  klist,  scrZ, scrA,  wbox16, hh16,     hN16, hhT16, hscale,
                         twN,    hh4,   wrow, wxbox, d_vbox, d_kslot, d_korder, sitems, skptr, sklist,
                         hN2,    hN2_16, tw2048l, d_geo_f, d_geo_a, sec_items_box, sec_items_win, hsT, hsN,
-                        sec_twc, scrZs, scrAs, hsT16, hsN16, sec_hscale, d_kq0, hhTr, hNr};
+                        sec_twc, scrZs, scrAs, hsT16, hsN16, sec_hscale, d_kq0, hhTr, hNr, d_slot_toff};
         for (void* q : ptrs)
             if (q) cudaFree(q);
     }
@@ -153,6 +154,7 @@ struct Scratch {
     int chunk = 1;
     int col_variant = -1;   // >= 0: overrides the plan's column variant for this apply
     int row_variant = -1;   // >= 0: overrides the plan's row variant for this apply
+    bool beside = false;    // other applies run beside this one (lanes of a batch)
 };
 
 pce_status fail(pce_status s, const char* fmt, ...);

@@ -322,8 +322,8 @@ kt_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     tm_end(&tm_slot, kt_tm_cols<NY>());
 }
 
-// G1b + G2 for separable plans, Ny = 1024.  Grid (batch, NXh / 4), 128
-// threads, kTColSmem bytes.  Arguments as kw_cols_adj<false, float2, true>:
+// G1b + G2 for separable plans, Ny = 1024.  Grid (batch, NXh / 4, split), 128
+// threads, kTColSmem bytes; CTA z of a column tile takes its share of the slots.  Arguments as kw_cols_adj<false, float2, true>:
 // Q receives, per slot, S_j on the slot box rows.
 template <bool PRUNE, int NY = kWarpN>
 __global__ void __launch_bounds__(kWColWarps * 32, NY == kWarpN ? 4 : 6)
@@ -352,8 +352,8 @@ kt_cols_adj(float2* __restrict__ V, long long v_bstride, const float2* __restric
     const unsigned t_hold = tbase, t_acc = tbase + 2 * QN;
     unsigned parity = 0;
     bool failed = false;
-    const int tbeg = sep.t1 < 0 ? 0 : sep.t0;
-    const int tend = sep.t1 < 0 ? sep.nterms : sep.t1;
+    int tbeg = sep.t0, tend = sep.t1;
+    if (sep.t1 < 0) sep_share(sep, tbeg, tend);
     const int mode = sep.t1 < 0 ? 0 : sep.mode;
     const int swl = tix_sw(lane, warp);
 

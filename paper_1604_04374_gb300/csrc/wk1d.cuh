@@ -2,10 +2,10 @@
 //
 // The same operators as k_fwd_1d / k_adj_1d (kernels.cuh), with the same
 // packed spectra, for the latency-bound case of a handful of right-hand
-// sides: one CTA per right-hand side, whose warps take the term pairs in
-// turn and run their FFTs with the one-warp 1024-point FFT (warpfft.cuh), so
-// that no CTA barrier sits inside an FFT; the warps' partial sums meet once in
-// shared memory at the end.  Lane l holds samples l + 32 q, and after a
+// sides: one CTA, or one cluster of cl CTAs, per right-hand side, whose warps take
+// the term pairs in turn and run their FFTs with the one-warp 1024-point FFT
+// (warpfft.cuh), so that no CTA barrier sits inside an FFT; the warps' partial
+// sums meet once in shared memory at the end, the CTAs' through the cluster's.  Lane l holds samples l + 32 q, and after a
 // forward FFT frequencies l + 32 q (the four-step layout), so the products
 // with the spectra and the windows are lane-local.
 #pragma once
@@ -16,8 +16,9 @@ namespace pce {
 
 constexpr int kW1dWarps = 4;   // warps per CTA: term pairs in flight
 
-// y_b = (1/N) C2R( sum_k hhat_k . R2C(w_k . u_b) ), N = 1024.  Grid (batch),
-// kW1dWarps * 32 threads.  Warp w takes the term pairs w, w + kW1dWarps, ...:
+// y_b = (1/N) C2R( sum_k hhat_k . R2C(w_k . u_b) ), N = 1024.  Grid
+// (batch cl), kW1dWarps * 32 threads.  Warp w of rank r takes the term pairs
+// r kW1dWarps + w, ... in steps of cl kW1dWarps:
 // w_k u + i w_{k+1} u in one complex FFT, the two half spectra separated with
 // the partner frequencies X[N - f] (shuffles), hhat . X accumulated for
 // f = lane + 32 j (j < 16; lane 0, j = 0 packs the real DC and Nyquist terms
@@ -27,13 +28,14 @@ template <typename WT, typename HT>
 __global__ void __launch_bounds__(kW1dWarps * 32)
 kw_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w, const HT* __restrict__ hp,
           const float* __restrict__ hscale, int m, float* __restrict__ y, float scale,
-          const float2* __restrict__ tw) {
+          const float2* __restrict__ tw, int cl) {
     constexpr int N = kWarpN, Nh = N / 2;
     __shared__ __align__(16) float2 tiles[kW1dWarps][N];
     __shared__ __align__(16) float2 hsum[Nh];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float2* tr = tiles[warp];
-    const int b = blockIdx.x;
+    const int b = blockIdx.x / cl;
+    const int rank = cl > 1 ? cluster_rank() : 0;
     // the twiddles and the spectra are read after the first FFT's start and end
     prefetch_l2_block(tw, (long long)kWarpTwLen * sizeof(float2));
     prefetch_l2_block(hp, (long long)m * Nh * sizeof(HT));
@@ -45,7 +47,7 @@ kw_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w, const HT* __res
 #pragma unroll
     for (int j = 0; j < 16; ++j) acc[j] = make_float2(0.f, 0.f);
     const int npairs = (m + 1) / 2;
-    for (int pr = warp; pr < npairs; pr += kW1dWarps) {
+    for (int pr = rank * kW1dWarps + warp; pr < npairs; pr += cl * kW1dWarps) {
         const int k0 = 2 * pr, k1 = k0 + 1;
         const bool a1 = k1 < m;
         const WT* w0 = w + (long long)k0 * N;
@@ -84,19 +86,35 @@ kw_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w, const HT* __res
             }
         }
     }
-    // the warps' half spectra, summed in warp order by warp 0
+    // the warps' half spectra, summed in warp order by the CTA, then the CTAs' in
+    // rank order by rank 0
     __syncthreads();   // every warp is done with its transpose tile
 #pragma unroll
     for (int j = 0; j < 16; ++j) tr[lane + 32 * j] = acc[j];
     __syncthreads();
-    if (warp != 0) return;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        float2 s = tiles[0][lane + 32 * j];
-        for (int g = 1; g < kW1dWarps; ++g) s = cadd(s, tiles[g][lane + 32 * j]);
-        hsum[lane + 32 * j] = s;
+    for (int i = 0; i < Nh / (kW1dWarps * 32); ++i) {
+        const int f = threadIdx.x + i * kW1dWarps * 32;
+        float2 s = tiles[0][f];
+        for (int g = 1; g < kW1dWarps; ++g) s = cadd(s, tiles[g][f]);
+        hsum[f] = s;
     }
-    __syncwarp();
+    if (cl > 1) {
+        cluster_sync();
+        if (rank == 0) {
+#pragma unroll
+            for (int i = 0; i < Nh / (kW1dWarps * 32); ++i) {
+                const int f = threadIdx.x + i * kW1dWarps * 32;
+                float2 s = hsum[f];
+                for (int g = 1; g < cl; ++g) s = cadd(s, cluster_ld2(cluster_map(&hsum[f], g)));
+                hsum[f] = s;
+            }
+        }
+        cluster_sync();   // rank 0 has read the others' sums
+        if (rank != 0) return;
+    }
+    __syncthreads();
+    if (warp != 0) return;
     float2 v[32];
 #pragma unroll
     for (int q = 0; q < 32; ++q) v[q] = load_half<N>(hsum, lane + 32 * q);
@@ -107,20 +125,22 @@ kw_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w, const HT* __res
 }
 
 // x_b = (1/N) sum_k w_k . IFFT( conj(hhat_k) . FFT(v_b) ), N = 1024.  Grid
-// (batch), kW1dWarps * 32 threads.  Every warp transforms v itself, then takes
-// the term pairs w, w + kW1dWarps, ...: the two inverse FFTs of a pair are
+// (batch cl), kW1dWarps * 32 threads.  Every warp transforms v itself, then takes
+// the term pairs as above: the two inverse FFTs of a pair are
 // real, so they share one complex inverse FFT; the windowed sums of the warps
 // are added in warp order at the end.
 template <typename WT, typename HT>
 __global__ void __launch_bounds__(kW1dWarps * 32)
 kw_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w, const HT* __restrict__ hp,
           const float* __restrict__ hscale, int m, float* __restrict__ x, float scale,
-          const float2* __restrict__ tw) {
+          const float2* __restrict__ tw, int cl) {
     constexpr int N = kWarpN, Nh = N / 2;
     __shared__ __align__(16) float2 tiles[kW1dWarps][N];
+    __shared__ float red[N];   // this CTA's sums (clusters)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float2* tr = tiles[warp];
-    const int b = blockIdx.x;
+    const int b = blockIdx.x / cl;
+    const int rank = cl > 1 ? cluster_rank() : 0;
     prefetch_l2_block(tw, (long long)kWarpTwLen * sizeof(float2));
     prefetch_l2_block(hp, (long long)m * Nh * sizeof(HT));
     prefetch_l2_block(w, (long long)m * N * sizeof(WT));
@@ -133,7 +153,7 @@ kw_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w, const HT* __r
 #pragma unroll
     for (int q = 0; q < 32; ++q) ax[q] = 0.f;
     const int npairs = (m + 1) / 2;
-    for (int pr = warp; pr < npairs; pr += kW1dWarps) {
+    for (int pr = rank * kW1dWarps + warp; pr < npairs; pr += cl * kW1dWarps) {
         const int k0 = 2 * pr, k1 = k0 + 1;
         const bool a1 = k1 < m;
         const HT* h0 = hp + (long long)k0 * Nh;
@@ -167,13 +187,24 @@ kw_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w, const HT* __r
 #pragma unroll
     for (int q = 0; q < 32; ++q) fb[lane + 32 * q] = ax[q];
     __syncthreads();
-    if (warp != 0) return;
     float* xb = x + (long long)b * N;
 #pragma unroll
-    for (int q = 0; q < 32; ++q) {
-        float s = reinterpret_cast<const float*>(tiles[0])[lane + 32 * q];
-        for (int g = 1; g < kW1dWarps; ++g) s += reinterpret_cast<const float*>(tiles[g])[lane + 32 * q];
-        xb[lane + 32 * q] = s * scale;
+    for (int i = 0; i < N / (kW1dWarps * 32); ++i) {
+        const int n = threadIdx.x + i * kW1dWarps * 32;
+        float s = reinterpret_cast<const float*>(tiles[0])[n];
+        for (int g = 1; g < kW1dWarps; ++g) s += reinterpret_cast<const float*>(tiles[g])[n];
+        if (cl > 1) red[n] = s;
+        else xb[n] = s * scale;
+    }
+    if (cl > 1) {
+        cluster_sync();
+        const int part = N / cl;
+        for (int n = rank * part + threadIdx.x; n < (rank + 1) * part; n += kW1dWarps * 32) {
+            float s = 0.f;
+            for (int g = 0; g < cl; ++g) s += cluster_ld(cluster_map(&red[n], g));
+            xb[n] = s * scale;
+        }
+        cluster_sync();   // every rank has read the others' sums
     }
 }
 

@@ -277,9 +277,22 @@ kw_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     }
 }
 
+// Terms [tbeg, tend) of korder for CTA z of a column tile: those of its share of
+// the slots (a slot's sum is formed by one CTA).
+__device__ __forceinline__ void sep_share(const SepTerms& sep, int& tbeg, int& tend) {
+    if (gridDim.z == 1) {
+        tbeg = 0;
+        tend = sep.nterms;
+    } else {
+        tbeg = __ldg(&sep.slot_toff[share_beg(sep.nslots, blockIdx.z, gridDim.z)]);
+        tend = __ldg(&sep.slot_toff[share_beg(sep.nslots, blockIdx.z + 1, gridDim.z)]);
+    }
+}
+
 // G1b + G2 for Ny = NY (1024 or 512; FULL: every row of Q, for the window
 // gradient).
-// Grid (batch, NXh / 4).
+// Grid (batch, NXh / 4, split): CTA z of a column tile takes its share of the terms
+// (SEP: of the slots) and forms the FFT of V itself.
 // SEP: Q receives one slot per column factor: S_j = sum over the slot's terms of
 // wy_k . IFFT_y(conj(hhat_k) V), on the slot box rows (box[] indexed by slot),
 // accumulated in the shared tile and stored once per slot.
@@ -309,10 +322,16 @@ kw_cols_adj(const float2* __restrict__ V, long long v_bstride,
     bool failed = false;
     const bool use_bulk = !dcn && cv;
     // the sequence of terms (see kw_cols_fwd)
-    const int tend = SEP ? sep.nterms : m;
+    int tbeg, tend;
+    if constexpr (SEP) {
+        sep_share(sep, tbeg, tend);
+    } else {
+        tbeg = share_beg(m, blockIdx.z, gridDim.z);
+        tend = share_beg(m, blockIdx.z + 1, gridDim.z);
+    }
     auto next_t = [&](int t) {
         if constexpr (!SEP) {
-            while (t < m && !FULL && box[t].nr == 0) ++t;
+            while (t < tend && !FULL && box[t].nr == 0) ++t;
         }
         return t;
     };
@@ -322,7 +341,7 @@ kw_cols_adj(const float2* __restrict__ V, long long v_bstride,
     // SEP: row factors of the t-th term in buffer (t & 1), prefetched one term ahead
     float* wys = reinterpret_cast<float*>(smem + 2 * NY * kWColWarps);
     if constexpr (SEP) {
-        if (sep.nterms > 0) wy_load<NY>(wys, sep.wrow, __ldg(&sep.korder[0]));
+        if (tbeg < tend) wy_load<NY>(wys + (tbeg & 1) * NY, sep.wrow, __ldg(&sep.korder[tbeg]));
     }
     tile_load(tile, V + b * v_bstride, NY, NXh, col0);
     cp_async_wait_all();
@@ -330,7 +349,7 @@ kw_cols_adj(const float2* __restrict__ V, long long v_bstride,
     float2 vv[QN];
 #pragma unroll
     for (int q = 0; q < QN; ++q) vv[q] = tile[4 * (lane + 32 * q) + tix_sw(lane, warp)];
-    int t = next_t(0);
+    int t = next_t(tbeg);
     int prev_slot = -1;
     // the spectrum of the first term arrives while the FFT of V finishes
     warp_fft<NY, false, SEP>(vv, tr, tw, [&] {

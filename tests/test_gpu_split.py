@@ -1,0 +1,108 @@
+"""GPU: applies whose terms are split over several CTAs (few right-hand sides).
+
+1D, N <= 8192: cluster sizes 1 to 8 by batch and m, with remainders (terms that do not
+divide into rounds, odd m, one term), batches on both sides of each size's last one,
+both directions and both storage precisions, against the FP64 oracle.
+
+Bar: an FFT of n points in FP32 has a relative l2 error of at most about
+eps log2 n (eps = 6e-8); a forward and an inverse one with the products between them,
+n <= 8192, stay below 30 eps = 2e-6.  Reduced storage: the project's bar of 3e-3.
+"""
+import numpy as np
+import pytest
+
+import synth
+from oracle import direct as O
+
+pytestmark = pytest.mark.gpu
+
+TOL = 2e-6
+TOL_LOWP = 3e-3
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    import torch
+    from paper_1604_04374_gb300 import build
+    build.build()
+    O.build()
+    torch.cuda.init()
+    return torch
+
+
+def dev(torch, a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def rel(got, ref):
+    got = got.detach().cpu().numpy().astype(np.float64).reshape(ref.shape[0], -1)
+    ref = ref.reshape(ref.shape[0], -1)
+    return float(np.max(np.linalg.norm(got - ref, axis=1) / np.linalg.norm(ref, axis=1)))
+
+
+def problem_1d(n, m, batch):
+    rng = np.random.default_rng(1000 * n + 10 * m + batch)
+    w = synth.hat_windows_1d(n, m) if m >= 2 else np.ones((1, n), np.float32)
+    h = np.zeros((m, n), np.float32)
+    offs = np.unique(np.arange(-6, 7) % n)
+    h[:, offs] = rng.standard_normal((m, offs.size)).astype(np.float32)
+    return w, h, rng.standard_normal((batch, n)).astype(np.float32)
+
+
+@pytest.mark.parametrize("n", [16, 64, 256, 512, 1024, 2048, 4096, 8192])
+@pytest.mark.parametrize("m,batch", [(1, 1), (2, 3), (5, 1), (9, 38), (17, 19), (33, 1), (32, 20), (6, 77)])
+def test_1d_clusters(torch_cuda, n, m, batch):
+    torch = torch_cuda
+    from paper_1604_04374_gb300 import Plan, pce
+    w, h, u = problem_1d(n, m, batch)
+    yr, xr = O.apply(u, w, h), O.apply_adjoint(u, w, h)
+    for flags, tol in ((0, TOL), (pce.PCE_FLAG_LOWP_STORAGE, TOL_LOWP)):
+        plan = Plan(dev(torch, w), h=dev(torch, h), flags=flags)
+        assert rel(plan.apply(dev(torch, u)), yr) <= tol
+        assert rel(plan.apply_adjoint(dev(torch, u)), xr) <= tol
+        plan.close()
+
+
+def problem_2d(ny, nx, gy, gx, batch, zero=()):
+    rng = np.random.default_rng(ny + 7 * nx + 100 * gy + 1000 * gx + batch)
+    wy, wx = synth.hat_factors_2d(ny, nx, gy, gx)
+    for k in zero:
+        wy[k] = 0.0
+    h = np.zeros((gy * gx, ny, nx), np.float32)
+    offs = np.arange(-2, 3)
+    h[:, (offs % ny)[:, None], (offs % nx)[None, :]] = rng.standard_normal((gy * gx, 5, 5)).astype(np.float32)
+    return wy, wx, h, rng.standard_normal((batch, ny, nx)).astype(np.float32)
+
+
+@pytest.mark.parametrize("ny,nx", [(16, 32), (64, 64), (256, 128), (512, 64), (1024, 32), (2048, 32)])
+@pytest.mark.parametrize("gy,gx,batch,zero", [(1, 1, 1, ()), (3, 3, 1, ()), (4, 4, 3, (0, 1, 2, 15)),
+                                              (5, 1, 2, ()), (3, 5, 1, (14, 13))])
+def test_2d_column_splits(torch_cuda, ny, nx, gy, gx, batch, zero):
+    """The terms (or slots) of a column tile over CTAs: dense and separable plans, the column variants that split, empty windows in a CTA's share, the
+    product form and reduced storage."""
+    torch = torch_cuda
+    from paper_1604_04374_gb300 import Plan, pce
+    wy, wx, h, u = problem_2d(ny, nx, gy, gx, batch, zero)
+    w = (wy[:, :, None] * wx[:, None, :]).astype(np.float32)
+    yr, xr = O.apply(u, w, h), O.apply_adjoint(u, w, h)
+    ud, hd = dev(torch, u), dev(torch, h)
+
+    def check(plan, tol):
+        assert rel(plan.apply(ud), yr) <= tol
+        assert rel(plan.apply_adjoint(ud), xr) <= tol
+
+    plan = Plan(dev(torch, w), h=hd)
+    check(plan, TOL)
+    if ny >= 512:
+        plan.set_tuning(0, 1, 0)   # block Stockham columns
+        check(plan, TOL)
+    check(Plan(dev(torch, w), h=hd, flags=pce.PCE_FLAG_LOWP_STORAGE), TOL_LOWP)
+    p = Plan(dev(torch, w), h=hd, flags=pce.PCE_FLAG_PRODUCT_CONVOLUTION)
+    # P_m = sum_k w_k . (h_k * u): the adjoint operator's structure with h reversed
+    hr = np.ascontiguousarray(np.roll(h[:, ::-1, ::-1], (1, 1), (1, 2)))
+    assert rel(p.apply(ud), O.apply_adjoint(u, w, hr)) <= TOL
+    sep = Plan(wy=dev(torch, wy), wx=dev(torch, wx), h=hd)
+    check(sep, TOL)
+    for cv in {512: (0, 2), 1024: (0, 2)}.get(ny, ()):
+        sep.set_tuning(0, cv, 2)
+        check(sep, TOL)
