@@ -1,0 +1,397 @@
+// ckernels.cuh -- column kernels of dense (not separable) plans for columns of
+// NY = NF PAR points: 512 and 1024 (PAR = 1) and 2048 (NF = 1024, PAR = 2).
+//
+// Every column is transformed by PAR warps with the one-warp FFT of NF points
+// (warpfft.cuh).  PAR = 2 splits the 2048-point DFT by decimation in frequency:
+//   X[2k]     = DFT1024( x[n] + x[n + 1024] )[k]
+//   X[2k + 1] = DFT1024( (x[n] - x[n + 1024]) W2048^n )[k]
+// and warp `par` of a column takes the even (0) or the odd (1) frequencies; the
+// inverse runs the two halves backwards, a = IDFT(even), b = W2048^-n IDFT(odd),
+// x[n] = a + b, x[n + 1024] = a - b, combined when the column is stored.  Spectra:
+// hhT [m][NXh][PAR][NF] (column 0: the DC column), hN [m][PAR][NF] (Nyquist column).
+//
+// A CTA takes four columns (4 PAR warps).  What bounds these kernels is latency
+// (a term's rows and spectrum come from L2 or DRAM) and the instructions around
+// the FFT, so:
+//  - the state a warp carries from term to term (forward: the spectral accumulator,
+//    adjoint: the column spectrum of V) lives in tensor memory (tmem.cuh), which
+//    leaves 128 registers a thread and 16 warps an SM (20 and more at 512 points);
+//  - a term's rows are staged for the CTA by cp.async while the previous term's FFT
+//    runs, on a frame that starts at a multiple of 32 rows (the box's first row
+//    rounded down, zeros around the box): register q then reads tile rows lane + 32 j
+//    with j = q - frame, the same for the whole warp, without per-lane index or
+//    bounds arithmetic, and absent blocks are not read at all;
+//  - the next term's spectrum is started towards L2 a term ahead (one bulk prefetch
+//    a warp); the forward brings it into the warp's transpose tile during the second
+//    half of the FFT, the adjoint loads it straight into registers;
+//  - the power-of-two scale of a term's reduced spectrum is applied where the fewest
+//    values pass (exact): to the staged rows (forward), to the stored rows (adjoint).
+#pragma once
+
+#include "tkernels.cuh"
+
+namespace pce {
+
+constexpr int kCCols = 4;   // columns per CTA
+
+// cos(2 pi j / 64) on [0, 16] (FP32, rounded from FP64; exact at 0 and 16)
+__host__ __device__ constexpr float cos64q(int j) {
+    return j == 0 ? 1.0f : j == 1 ? 0.9951847f : j == 2 ? 0.98078525f : j == 3 ? 0.95694035f
+         : j == 4 ? 0.9238795f : j == 5 ? 0.8819213f : j == 6 ? 0.8314696f : j == 7 ? 0.77301043f
+         : j == 8 ? 0.70710677f : j == 9 ? 0.6343933f : j == 10 ? 0.55557024f : j == 11 ? 0.47139674f
+         : j == 12 ? 0.38268343f : j == 13 ? 0.29028466f : j == 14 ? 0.19509032f : j == 15 ? 0.09801714f
+         : 0.0f;
+}
+__host__ __device__ constexpr float cos64(int j) {
+    return (j & 63) <= 16 ? cos64q(j & 63)
+         : (j & 63) <= 32 ? -cos64q(32 - (j & 63))
+         : (j & 63) <= 48 ? -cos64q((j & 63) - 32)
+         : cos64q(64 - (j & 63));
+}
+// W64^q = exp(-2 pi i q / 64)
+__host__ __device__ constexpr float2 w64(int q) { return float2{cos64(q), -cos64((q + 48) & 63)}; }
+
+// tensor-memory columns of a CTA: 2 NF / 32 a warp, four warps side by side
+template <int NF, int PAR>
+__host__ __device__ constexpr int kc_tm_cols() { return PAR * 2 * (NF / 32); }
+// CTAs per SM the kernels are compiled for (128 registers; 80 at 512 points)
+template <int NF, int PAR>
+__host__ __device__ constexpr int kc_min_ctas() { return NF == 512 ? 6 : PAR == 1 ? 4 : 2; }
+// shared memory: the transpose tiles, and in the forward zblk blocks of 32 rows
+template <int NF, int PAR>
+__host__ __device__ constexpr int kc_smem(int zblk) {
+    return (kCCols * PAR * NF + zblk * 32 * kCCols) * (int)sizeof(float2);
+}
+
+// Frame of a term's rows: tile row i holds row 32 s + i of the column (mod NY),
+// i < 32 nblk.  Boxes that would cover a frame block of the period twice take
+// the whole period (PAR = 1 only).
+struct CFrame {
+    int s, nblk;
+};
+template <int NF, int NY>
+__host__ __device__ __forceinline__ CFrame col_frame(const Box& b) {
+    const int a = b.r0 & 31;
+    if (a + b.nr > NF) return CFrame{0, NF / 32};
+    return CFrame{b.r0 >> 5, (a + b.nr + 31) >> 5};
+}
+
+__device__ __forceinline__ void bulk_prefetch_l2(const void* p, unsigned bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// Cooperative async copy of the frame f of a term's box rows (src [nr][nxh],
+// columns col0 .. col0 + 3) into the swizzled tile, zeros outside the box.
+template <int NY, int NT>
+__device__ __forceinline__ void frame_load(float2* tile, const float2* __restrict__ src, const Box& b, CFrame f,
+                                           int nxh, int col0) {
+    for (int e = threadIdx.x; e < f.nblk * 32 * kCCols; e += NT) {
+        const int i = e >> 2, c = e & 3;
+        const int r = wrap(32 * f.s + i - b.r0, NY);
+        const bool ok = r < b.nr && col0 + c < nxh;
+        cp_async8(tile + tix(i, c), src + (ok ? (long long)r * nxh + col0 + c : 0), ok);
+    }
+    cp_async_commit();
+}
+
+// X[NY - f] of a packed DC/Nyquist column from the transpose tile holding this
+// warp's half: index NF - f' (even half) or NF - 1 - f' (odd half).
+template <int NF>
+__device__ __forceinline__ float2 half_partner(const float2* tr, int f, int par) {
+    return tr[par ? NF - 1 - f : (NF - f) & (NF - 1)];
+}
+
+// The four columns' inverse transforms (transpose tiles of the CTA, element n of
+// column c, half p at (c PAR + p) NF + ((n + 4 c) mod NF)) combined and stored:
+// rows i < nr of dst ([rows][nxh], columns col0 ..) from rows r0 + i (mod NY),
+// times sc.  Two columns a 16-byte store where dst allows it.
+template <int NF, int PAR, int NT>
+__device__ __forceinline__ void store_halves(float2* __restrict__ dst, const float2* tiles, int r0, int nr, int nxh,
+                                             int col0, float sc) {
+    constexpr int NY = NF * PAR;
+    auto get = [&](int g, int c) {
+        const int n = (g + 4 * c) & (NF - 1);
+        const float2* t = tiles + c * PAR * NF;
+        float2 x = t[n];
+        if constexpr (PAR == 2) {
+            const float2 y = t[NF + n];
+            x = g < NF ? cadd(x, y) : csub(x, y);
+        }
+        return cscale(x, sc);
+    };
+    if ((reinterpret_cast<unsigned long long>(dst) & 15) == 0 && (nxh & 3) == 0) {
+        for (int e = threadIdx.x; e < nr * 2; e += NT) {
+            const int i = e >> 1, c = (e & 1) * 2;
+            const int g = wrap(r0 + i, NY);
+            const float2 x0 = get(g, c), x1 = get(g, c + 1);
+            *reinterpret_cast<float4*>(dst + (long long)i * nxh + col0 + c) = make_float4(x0.x, x0.y, x1.x, x1.y);
+        }
+    } else {
+        for (int e = threadIdx.x; e < nr * kCCols; e += NT) {
+            const int i = e >> 2, c = e & 3;
+            if (col0 + c < nxh) dst[(long long)i * nxh + col0 + c] = get(wrap(r0 + i, NY), c);
+        }
+    }
+}
+
+// F2.  Grid (batch, ceil(NXh / 4)), 128 PAR threads, kc_smem<NF, PAR>(zblk)
+// bytes; zblk >= every term's frame blocks.
+template <int NF, int PAR, typename HT>
+__global__ void __launch_bounds__(kCCols * PAR * 32, (kc_min_ctas<NF, PAR>()))
+kc_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstride, const HT* __restrict__ hhT,
+            const HT* __restrict__ hN, const float* __restrict__ hscale, int m, const Box* __restrict__ box, int NXh,
+            float2* __restrict__ A, long long a_bstride, const float2* __restrict__ tw,
+            const float2* __restrict__ tw2048l, int* __restrict__ status, long long wait_limit, int skip_copy) {
+    constexpr int NY = NF * PAR, QN = NF / 32, NQ = QN / 8, NT = kCCols * PAR * 32;
+    extern __shared__ __align__(16) float2 smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cl = warp / PAR, par = warp % PAR;
+    float2* tr = smem + warp * NF;                  // this warp's transpose tile
+    float2* tile = smem + kCCols * PAR * NF;        // the term's rows
+    __shared__ unsigned long long bars[kCCols * PAR];
+    __shared__ unsigned tm_slot;
+    const int b = blockIdx.x;
+    const int col0 = blockIdx.y * kCCols, col = col0 + cl;
+    const bool cv = col < NXh;
+    const bool dcn = col == 0;
+    const float2* Zb = Z + b * z_bstride;
+    unsigned long long* bar = &bars[warp];
+    if (lane == 0) mbar_init(bar);
+    if (warp == 0) tm_alloc(&tm_slot, kc_tm_cols<NF, PAR>());
+    tm_fence_before();
+    __syncthreads();
+    tm_fence_after();
+    const unsigned t_acc = tm_slot + ((unsigned)(32 * (warp & 3)) << 16) + (warp >> 2) * 2 * QN;
+    {
+        float2 z[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) z[j] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int qq = 0; qq < NQ; ++qq) tm_store8c(t_acc + 16 * qq, z);
+        tm_wait_st();
+    }
+    unsigned parity = 0;
+    bool failed = false;
+    const float2 wl = PAR == 2 ? __ldg(&tw2048l[lane]) : make_float2(1.f, 0.f);
+    const HT* hcol = hhT + ((long long)(cv ? col : 0) * PAR + par) * NF;   // + k NXh PAR NF
+    const long long hstride = (long long)NXh * PAR * NF;
+    const int sw = tix_sw(lane, cl);
+
+    const int kend = m;
+    auto next_k = [&](int k) {
+        while (k < kend && box[k].nr == 0) ++k;
+        return k;
+    };
+    int k = next_k(0);
+    if (k < kend) {
+        const Box bx = box[k];
+        frame_load<NY, NT>(tile, Zb + k * z_kstride, bx, col_frame<NF, NY>(bx), NXh, col0);
+        if (lane == 0 && cv) bulk_prefetch_l2(hcol + k * hstride, NF * sizeof(HT));
+    }
+    while (k < kend) {
+        const CFrame f = col_frame<NF, NY>(box[k]);
+        const int kn = next_k(k + 1);
+        cp_async_wait_all();
+        __syncthreads();   // the term's rows have landed
+        float2 v[QN];
+        const float sk = hscale_of<HT>(hscale, k);
+        const float2* tb = tile + 4 * lane + sw;
+#pragma unroll
+        for (int q = 0; q < QN; ++q) {
+            const int j = (q - f.s) & (QN - 1);   // the same for the whole warp
+            v[q] = make_float2(0.f, 0.f);
+            if (j < f.nblk) {
+                float2 x = tb[128 * j];
+                // PAR = 2: rows n and n + 1024 never both hold a frame block, so the even
+                // half's input is either one and the odd half's x[n] or -x[n + 1024]
+                if (PAR == 2 && par)
+                    x = cmul(cmul(x, cscale(wl, (f.s + j) & QN ? -sk : sk)), w64(q));
+                else if (sizeof(HT) != sizeof(float2))
+                    x = cscale(x, sk);
+                v[q] = x;
+            }
+        }
+        __syncthreads();   // every warp has read its rows: the next term's may come
+        if (kn < kend) {
+            const Box bn = box[kn];
+            frame_load<NY, NT>(tile, Zb + kn * z_kstride, bn, col_frame<NF, NY>(bn), NXh, col0);
+            if (lane == 0 && cv) bulk_prefetch_l2(hcol + kn * hstride, NF * sizeof(HT));
+        }
+        const bool bulk = !dcn && cv && !failed;
+        auto hook = [&] {
+            if (bulk && lane == 0) bulk_load(tr, hcol + k * hstride, NF * sizeof(HT), bar, skip_copy);
+        };
+        warp_fft<NF, false, kTmSplit, decltype(hook)>(v, tr, tw, hook);
+        if (bulk) {
+            if (!mbar_wait(bar, parity, wait_limit)) {
+                failed = true;
+                if (lane == 0) atomicOr(status, kStatusTimeout);
+                // a copy may still be in flight into the tile: wait for it once more
+                // (bounded); no further copies are issued, the products are skipped
+                mbar_wait(bar, parity, wait_limit);
+            }
+            parity ^= 1;
+        }
+        if (dcn) {
+            const HT* h0 = hcol + k * hstride;
+            const HT* hn = hN + ((long long)k * PAR + par) * NF;
+            __syncwarp();
+#pragma unroll
+            for (int mm = 0; mm < QN; ++mm) tr[lane + 32 * mm] = v[mm];
+            __syncwarp();
+#pragma unroll
+            for (int qq = 0; qq < NQ; ++qq)
+                tm_update8(t_acc, qq, [&](int mm, float2 a) {
+                    const int fr = lane + 32 * mm;
+                    float2 x, y;
+                    split_dc_nyq(v[mm], half_partner<NF>(tr, fr, par), x, y);
+                    a = cfma(ldh(&h0[fr], 1.f), x, a);
+                    const float2 s = cmul(ldh(&hn[fr], 1.f), y);
+                    a.x -= s.y;
+                    a.y += s.x;
+                    return a;
+                });
+            tm_wait_st();
+            __syncwarp();
+        } else if (cv && !failed) {
+            const HT* th = reinterpret_cast<const HT*>(tr);
+#pragma unroll
+            for (int qq = 0; qq < NQ; ++qq)
+                tm_update8(t_acc, qq, [&](int mm, float2 a) { return cfma(lds_h(&th[lane + 32 * mm], 1.f), v[mm], a); });
+            tm_wait_st();
+        }
+        k = kn;
+    }
+    float2 acc[QN];
+    tm_loadq<QN>(t_acc, acc);
+    warp_fft<NF, true, kTmSplit>(acc, tr, tw);
+    if constexpr (PAR == 2) {
+        if (par) {
+#pragma unroll
+            for (int q = 0; q < QN; ++q) acc[q] = cmulc(cmulc(acc[q], wl), w64(q));
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < QN; ++q) tr[(lane + 32 * q + 4 * cl) & (NF - 1)] = acc[q];
+    __syncthreads();
+    store_halves<NF, PAR, NT>(A + b * a_bstride, smem, 0, NY, NXh, col0, 1.f);
+    tm_end(&tm_slot, kc_tm_cols<NF, PAR>());
+}
+
+// G1b + G2.  Grid (batch, ceil(NXh / 4), split), 128 PAR threads,
+// kc_smem<NF, PAR>(0) bytes.  FULL: every row of Q (the window gradient).  split:
+// CTA z of a column tile takes its share of the terms and forms the FFT of V itself.
+template <int NF, int PAR, bool FULL, typename HT>
+__global__ void __launch_bounds__(kCCols * PAR * 32, (kc_min_ctas<NF, PAR>()))
+kc_cols_adj(const float2* __restrict__ V, long long v_bstride, const HT* __restrict__ hhT, const HT* __restrict__ hN,
+            const float* __restrict__ hscale, int m, const Box* __restrict__ box, int NXh, float2* __restrict__ Q,
+            long long q_bstride, long long q_kstride, const float2* __restrict__ tw,
+            const float2* __restrict__ tw2048l) {
+    constexpr int NY = NF * PAR, QN = NF / 32, NQ = QN / 8, NT = kCCols * PAR * 32;
+    extern __shared__ __align__(16) float2 smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cl = warp / PAR, par = warp % PAR;
+    float2* tr = smem + warp * NF;
+    __shared__ unsigned tm_slot;
+    const int b = blockIdx.x;
+    const int col0 = blockIdx.y * kCCols, col = col0 + cl;
+    const bool cv = col < NXh;
+    const bool dcn = col == 0;
+    if (warp == 0) tm_alloc(&tm_slot, kc_tm_cols<NF, PAR>());
+    tm_fence_before();
+    __syncthreads();
+    tm_fence_after();
+    const unsigned t_hold = tm_slot + ((unsigned)(32 * (warp & 3)) << 16) + (warp >> 2) * 2 * QN;
+    const float2 wl = PAR == 2 ? __ldg(&tw2048l[lane]) : make_float2(1.f, 0.f);
+    const HT* hcol = hhT + ((long long)(cv ? col : 0) * PAR + par) * NF;
+    const long long hstride = (long long)NXh * PAR * NF;
+    const int kend = share_beg(m, blockIdx.z + 1, gridDim.z);
+    auto next_k = [&](int k) {
+        while (!FULL && k < kend && box[k].nr == 0) ++k;
+        return k;
+    };
+    int k = next_k(share_beg(m, blockIdx.z, gridDim.z));
+    if (lane == 0 && k < kend && cv) bulk_prefetch_l2(hcol + k * hstride, NF * sizeof(HT));
+    {
+        // the four columns of V through the transpose tiles, [NY][4] swizzled
+        for (int e = threadIdx.x; e < NY * kCCols; e += NT) {
+            const int i = e >> 2, c = e & 3;
+            const bool ok = col0 + c < NXh;
+            cp_async8(smem + tix(i, c), V + b * v_bstride + (long long)i * NXh + (ok ? col0 + c : 0), ok);
+        }
+        cp_async_commit();
+        cp_async_wait_all();
+        __syncthreads();
+        float2 v[QN];
+        const float2* tb = smem + 4 * lane + tix_sw(lane, cl);
+#pragma unroll
+        for (int q = 0; q < QN; ++q) {
+            v[q] = tb[128 * q];
+            if constexpr (PAR == 2) {
+                const float2 hi = tb[128 * q + 4 * NF];
+                v[q] = par ? cmul(cmul(csub(v[q], hi), wl), w64(q)) : cadd(v[q], hi);
+            }
+        }
+        __syncthreads();   // every warp has read its column: the transpose tiles are free
+        warp_fft<NF, false, kTmSplit>(v, tr, tw);
+        tm_storeq<QN>(t_hold, v);
+        tm_wait_st();
+    }
+    while (k < kend) {
+        const int kn = next_k(k + 1);
+        if (lane == 0 && kn < kend && cv) bulk_prefetch_l2(hcol + kn * hstride, NF * sizeof(HT));
+        const float sk = hscale_of<HT>(hscale, k);
+        const HT* hk = hcol + k * hstride;
+        float2 p[QN];
+        if (dcn) {
+            tm_loadq<QN>(t_hold, p);
+            const HT* hn = hN + ((long long)k * PAR + par) * NF;
+            __syncwarp();
+#pragma unroll
+            for (int mm = 0; mm < QN; ++mm) tr[lane + 32 * mm] = p[mm];
+            __syncwarp();
+#pragma unroll
+            for (int mm = 0; mm < QN; ++mm) {
+                const int fr = lane + 32 * mm;
+                float2 x, y;
+                split_dc_nyq(p[mm], half_partner<NF>(tr, fr, par), x, y);
+                float2 r = cmulc(x, ldh(&hk[fr], 1.f));
+                const float2 s = cmulc(y, ldh(&hn[fr], 1.f));
+                r.x -= s.y;
+                r.y += s.x;
+                p[mm] = r;
+            }
+            __syncwarp();
+        } else {
+#pragma unroll
+            for (int mm = 0; mm < QN; ++mm) p[mm] = ldh(&hk[lane + 32 * mm], 1.f);
+#pragma unroll
+            for (int qq = 0; qq < NQ; ++qq) {
+                float2 x[8];
+                tm_load8c(t_hold + 16 * qq, x);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) p[8 * qq + j] = cmulc(x[j], p[8 * qq + j]);
+            }
+        }
+        warp_fft<NF, true, kTmSplit>(p, tr, tw);
+        if constexpr (PAR == 2) {
+            if (par) {
+#pragma unroll
+                for (int q = 0; q < QN; ++q) p[q] = cmulc(cmulc(p[q], wl), w64(q));
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < QN; ++q) tr[(lane + 32 * q + 4 * cl) & (NF - 1)] = p[q];
+        __syncthreads();
+        const Box bx = box[k];
+        store_halves<NF, PAR, NT>(Q + b * q_bstride + k * q_kstride, smem, FULL ? 0 : bx.r0, FULL ? NY : bx.nr, NXh,
+                                  col0, sk);
+        __syncthreads();   // the transpose tiles are free again
+        k = kn;
+    }
+    tm_end(&tm_slot, kc_tm_cols<NF, PAR>());
+}
+
+}  // namespace pce

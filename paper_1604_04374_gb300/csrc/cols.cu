@@ -3,6 +3,7 @@
 #include "kernels.cuh"
 #include "wkernels.cuh"
 #include "wkernels2.cuh"
+#include "ckernels.cuh"
 #include "tkernels.cuh"
 #include "launch.h"
 
@@ -35,8 +36,30 @@ int cols_smem(int ny) {
     return 0;
 }
 
+template <int NF, int PAR, typename HT>
+cudaError_t prepare_ccols_of() {
+    const void* fns[] = {(const void*)kc_cols_fwd<NF, PAR, HT>, (const void*)kc_cols_adj<NF, PAR, false, HT>,
+                         (const void*)kc_cols_adj<NF, PAR, true, float2>};
+    for (const void* f : fns) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kc_smem<NF, PAR>(NF / 32));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t prepare_ccols() {
+    cudaError_t e = prepare_ccols_of<512, 1, float2>();
+    if (e == cudaSuccess) e = prepare_ccols_of<512, 1, __half2>();
+    if (e == cudaSuccess) e = prepare_ccols_of<1024, 1, float2>();
+    if (e == cudaSuccess) e = prepare_ccols_of<1024, 1, __half2>();
+    if (e == cudaSuccess) e = prepare_ccols_of<1024, 2, float2>();
+    if (e == cudaSuccess) e = prepare_ccols_of<1024, 2, __half2>();
+    return e;
+}
+
 cudaError_t prepare_cols() {
-    cudaError_t e = cudaFuncSetAttribute(kw_cols_fwd<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWColSmem);
+    cudaError_t e = prepare_ccols();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kt_cols_fwd<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTColSmem);
     if (e == cudaSuccess)
@@ -50,26 +73,11 @@ cudaError_t prepare_cols() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kw2_cols_fwd<__half2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kW2Smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kw2_cols_adj<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kW2Smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kw2_cols_adj<__half2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kW2Smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kw_cols_fwd<__half2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWColSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kw_cols_adj<false, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kWColSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kw_cols_adj<false, __half2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kWColSmem);
-    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kw_cols_fwd<float2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kWColSmem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kw_cols_adj<false, float2, true>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, kWColSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kw_cols_adj<true, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kWColSmem);
 #define X(N)                                                                                   \
     if (e == cudaSuccess)                                                                      \
         e = cudaFuncSetAttribute(k_cols_fwd<N, float2>,                                        \
@@ -100,131 +108,116 @@ cudaError_t prepare_cols() {
     return e;
 }
 
-cudaError_t launch_cols_fwd(int ny, dim3 grid, cudaStream_t s, const float2* Z, long long z_bstride,
-                            long long z_kstride, const void* hh, const void* hN, const float* hscale,
-                            bool lowp, int m,
-                            const Box* box, int nxh, float2* A, long long a_bstride,
-                            const float2* tw, const void* hhT, const float2* tw1024, int* status,
-                            long long wait_limit, int skip_copy, bool warp,
-                            const void* hN2, const float2* tw2048l) {
-    // the warp-FFT column kernels index these tables: refuse to launch without them
-    if ((ny == 512 || ny == kWarpN || ny == kW2N) && warp && (!tw1024 || !hhT)) return cudaErrorInvalidValue;
-    if (ny == kW2N && warp && (!tw2048l || !hN2)) return cudaErrorInvalidValue;
-    if (ny == kW2N && warp) {
-        dim3 g2 = grid;
-        if (lowp)
-            kw2_cols_fwd<__half2><<<g2, 128, kW2Smem, s>>>(
-                Z, z_bstride, z_kstride, static_cast<const __half2*>(hhT), static_cast<const __half2*>(hN2),
-                hscale, m, box, nxh, A, a_bstride, tw1024, tw2048l, status, wait_limit, skip_copy);
-        else
-            kw2_cols_fwd<float2><<<g2, 128, kW2Smem, s>>>(
-                Z, z_bstride, z_kstride, static_cast<const float2*>(hhT), static_cast<const float2*>(hN2),
-                hscale, m, box, nxh, A, a_bstride, tw1024, tw2048l, status, wait_limit, skip_copy);
-        return cudaGetLastError();
+bool col_frames(int ny, const Box* box, int m, int& zblk) {
+    zblk = 1;
+    const int nf = ny == 512 ? 512 : 1024;
+    if (ny != 512 && ny != 1024 && ny != 2048) return false;
+    for (int k = 0; k < m; ++k) {
+        if (box[k].nr == 0) continue;
+        if (ny == 2048 && (box[k].r0 & 31) + box[k].nr > nf) return false;
+        const CFrame f = ny == 512    ? col_frame<512, 512>(box[k])
+                         : ny == 1024 ? col_frame<1024, 1024>(box[k])
+                                      : col_frame<1024, 2048>(box[k]);
+        zblk = f.nblk > zblk ? f.nblk : zblk;
     }
-    if (ny == kWarpN && warp) {
-        if (lowp)
-            kw_cols_fwd<__half2><<<grid, kWColWarps * 32, kWColSmem, s>>>(
-                Z, z_bstride, z_kstride, static_cast<const __half2*>(hhT), static_cast<const __half2*>(hN),
-                hscale, m, box, nxh, A, a_bstride, tw1024, status, wait_limit, skip_copy);
-        else
-            kw_cols_fwd<float2><<<grid, kWColWarps * 32, kWColSmem, s>>>(
-                Z, z_bstride, z_kstride, static_cast<const float2*>(hhT), static_cast<const float2*>(hN),
-                hscale, m, box, nxh, A, a_bstride, tw1024, status, wait_limit, skip_copy);
-        return cudaGetLastError();
-    }
-    if (ny == 512 && warp) {
-        constexpr int sm = kw_col_smem<512>();
-        if (lowp)
-            kw_cols_fwd<__half2, false, 512><<<grid, kWColWarps * 32, sm, s>>>(
-                Z, z_bstride, z_kstride, static_cast<const __half2*>(hhT), static_cast<const __half2*>(hN),
-                hscale, m, box, nxh, A, a_bstride, tw1024, status, wait_limit, skip_copy);
-        else
-            kw_cols_fwd<float2, false, 512><<<grid, kWColWarps * 32, sm, s>>>(
-                Z, z_bstride, z_kstride, static_cast<const float2*>(hhT), static_cast<const float2*>(hN),
-                hscale, m, box, nxh, A, a_bstride, tw1024, status, wait_limit, skip_copy);
-        return cudaGetLastError();
-    }
-    switch (ny) {
-#define X(N)                                                                                   \
-    case N:                                                                                    \
-        if (lowp)                                                                              \
-            k_cols_fwd<N, __half2><<<grid, ColCfg<N>::NT, ColCfg<N>::SMEM, s>>>(                 \
-                Z, z_bstride, z_kstride, static_cast<const __half2*>(hh),                      \
-                static_cast<const __half2*>(hN), hscale, m, box, nxh, A, a_bstride, tw);        \
-        else                                                                                   \
-            k_cols_fwd<N, float2><<<grid, ColCfg<N>::NT, ColCfg<N>::SMEM, s>>>(                  \
-                Z, z_bstride, z_kstride, static_cast<const float2*>(hh),                       \
-                static_cast<const float2*>(hN), hscale, m, box, nxh, A, a_bstride, tw);         \
-        break;
-        PCE_COL_SIZES(X)
-#undef X
-        default:
-            return cudaErrorInvalidValue;
-    }
+    return true;
+}
+
+namespace {
+
+dim3 ccols_grid(int nb, int nxh, unsigned split) { return dim3(nb, (nxh + kCCols - 1) / kCCols, split); }
+
+template <int NF, int PAR, typename HT>
+cudaError_t ccols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride, long long z_kstride,
+                      float2* A, long long a_bstride) {
+    kc_cols_fwd<NF, PAR, HT><<<ccols_grid(c.nb, c.nxh, 1), kCCols * PAR * 32, kc_smem<NF, PAR>(c.zblk), s>>>(
+        Z, z_bstride, z_kstride, static_cast<const HT*>(c.hhT), static_cast<const HT*>(PAR == 2 ? c.hN2 : c.hN),
+        c.hscale, c.m, c.box, c.nxh, A, a_bstride, c.tw1024, c.tw2048l, c.status, c.wait_limit, c.skip_copy);
     return cudaGetLastError();
 }
 
-cudaError_t launch_cols_adj(int ny, dim3 grid, cudaStream_t s, const float2* V, long long v_bstride,
-                            const void* hh, const void* hN, const float* hscale, bool lowp, int m,
-                            const Box* box, int nxh, float2* Q, long long q_bstride, long long q_kstride,
-                            const float2* tw, const void* hhT, const float2* tw1024, int* status,
-                            long long wait_limit, int skip_copy, bool warp,
-                            const void* hN2, const float2* tw2048l) {
-    if ((ny == 512 || ny == kWarpN || ny == kW2N) && warp && (!tw1024 || !hhT)) return cudaErrorInvalidValue;
-    if (ny == kW2N && warp && (!tw2048l || !hN2)) return cudaErrorInvalidValue;
-    if (ny == kW2N && warp) {
-        if (lowp)
-            kw2_cols_adj<__half2><<<grid, 128, kW2Smem, s>>>(
-                V, v_bstride, static_cast<const __half2*>(hhT), static_cast<const __half2*>(hN2), hscale, m,
-                box, nxh, Q, q_bstride, q_kstride, tw1024, tw2048l, status, wait_limit, skip_copy);
-        else
-            kw2_cols_adj<float2><<<grid, 128, kW2Smem, s>>>(
-                V, v_bstride, static_cast<const float2*>(hhT), static_cast<const float2*>(hN2), hscale, m,
-                box, nxh, Q, q_bstride, q_kstride, tw1024, tw2048l, status, wait_limit, skip_copy);
+template <int NF, int PAR, bool FULL, typename HT>
+cudaError_t ccols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
+                      long long q_bstride, long long q_kstride) {
+    kc_cols_adj<NF, PAR, FULL, HT><<<ccols_grid(c.nb, c.nxh, c.split), kCCols * PAR * 32, kc_smem<NF, PAR>(0), s>>>(
+        V, v_bstride, static_cast<const HT*>(c.hhT), static_cast<const HT*>(PAR == 2 ? c.hN2 : c.hN), c.hscale, c.m,
+        c.box, c.nxh, Q, q_bstride, q_kstride, c.tw1024, c.tw2048l);
+    return cudaGetLastError();
+}
+
+template <typename HT>
+cudaError_t cols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride, long long z_kstride,
+                     float2* A, long long a_bstride) {
+    if (c.warp && c.ny == 512) return ccols_fwd<512, 1, HT>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
+    if (c.warp && c.ny == 1024) return ccols_fwd<1024, 1, HT>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
+    if (c.warp && c.ny == 2048 && c.zblk > 0)
+        return ccols_fwd<1024, 2, HT>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
+    if (c.warp && c.ny == 2048) {
+        kw2_cols_fwd<HT><<<dim3(c.nb, (c.nxh + kW2Cols - 1) / kW2Cols), 128, kW2Smem, s>>>(
+            Z, z_bstride, z_kstride, static_cast<const HT*>(c.hhT), static_cast<const HT*>(c.hN2), c.hscale, c.m,
+            c.box, c.nxh, A, a_bstride, c.tw1024, c.tw2048l, c.status, c.wait_limit, c.skip_copy);
         return cudaGetLastError();
     }
-    if (ny == kWarpN && warp) {
-        if (lowp)
-            kw_cols_adj<false, __half2><<<grid, kWColWarps * 32, kWColSmem, s>>>(
-                V, v_bstride, static_cast<const __half2*>(hhT), static_cast<const __half2*>(hN), hscale, m,
-                box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit, skip_copy);
-        else
-            kw_cols_adj<false, float2><<<grid, kWColWarps * 32, kWColSmem, s>>>(
-                V, v_bstride, static_cast<const float2*>(hhT), static_cast<const float2*>(hN), hscale, m,
-                box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit, skip_copy);
+    switch (c.ny) {
+#define X(N)                                                                                                     \
+    case N:                                                                                                      \
+        k_cols_fwd<N, HT><<<dim3(c.nb, (c.nxh + ColCfg<N>::C - 1) / ColCfg<N>::C), ColCfg<N>::NT,                \
+                            ColCfg<N>::SMEM, s>>>(Z, z_bstride, z_kstride, static_cast<const HT*>(c.hh),         \
+                                                  static_cast<const HT*>(c.hN), c.hscale, c.m, c.box, c.nxh, A,  \
+                                                  a_bstride, c.tw);                                              \
         return cudaGetLastError();
-    }
-    if (ny == 512 && warp) {
-        constexpr int sm = kw_col_smem<512>();
-        if (lowp)
-            kw_cols_adj<false, __half2, false, 512><<<grid, kWColWarps * 32, sm, s>>>(
-                V, v_bstride, static_cast<const __half2*>(hhT), static_cast<const __half2*>(hN), hscale, m,
-                box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit, skip_copy);
-        else
-            kw_cols_adj<false, float2, false, 512><<<grid, kWColWarps * 32, sm, s>>>(
-                V, v_bstride, static_cast<const float2*>(hhT), static_cast<const float2*>(hN), hscale, m,
-                box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit, skip_copy);
-        return cudaGetLastError();
-    }
-    switch (ny) {
-#define X(N)                                                                                   \
-    case N:                                                                                    \
-        if (lowp)                                                                              \
-            k_cols_adj<N, false, __half2><<<grid, ColCfg<N>::NT, ColCfg<N>::SMEM, s>>>(          \
-                V, v_bstride, static_cast<const __half2*>(hh), static_cast<const __half2*>(hN),  \
-                hscale, m, box, nxh, Q, q_bstride, q_kstride, tw);                             \
-        else                                                                                   \
-            k_cols_adj<N, false, float2><<<grid, ColCfg<N>::NT, ColCfg<N>::SMEM, s>>>(           \
-                V, v_bstride, static_cast<const float2*>(hh), static_cast<const float2*>(hN),    \
-                hscale, m, box, nxh, Q, q_bstride, q_kstride, tw);                             \
-        break;
         PCE_COL_SIZES(X)
 #undef X
-        default:
-            return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
+}
+
+template <bool FULL, typename HT>
+cudaError_t cols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
+                     long long q_bstride, long long q_kstride) {
+    if (c.warp && c.ny == 512) return ccols_adj<512, 1, FULL, HT>(c, s, V, v_bstride, Q, q_bstride, q_kstride);
+    if (c.warp && c.ny == 1024) return ccols_adj<1024, 1, FULL, HT>(c, s, V, v_bstride, Q, q_bstride, q_kstride);
+    if (c.warp && c.ny == 2048) return ccols_adj<1024, 2, FULL, HT>(c, s, V, v_bstride, Q, q_bstride, q_kstride);
+    switch (c.ny) {
+#define X(N)                                                                                                     \
+    case N:                                                                                                      \
+        k_cols_adj<N, FULL, HT><<<dim3(c.nb, (c.nxh + ColCfg<N>::C - 1) / ColCfg<N>::C, c.split), ColCfg<N>::NT, \
+                                  ColCfg<N>::SMEM, s>>>(V, v_bstride, static_cast<const HT*>(c.hh),              \
+                                                        static_cast<const HT*>(c.hN), c.hscale, c.m, c.box,      \
+                                                        c.nxh, Q, q_bstride, q_kstride, c.tw);                   \
+        return cudaGetLastError();
+        PCE_COL_SIZES(X)
+#undef X
+    }
+    return cudaErrorInvalidValue;
+}
+
+// the one-warp column kernels index these tables: refuse to launch without them
+bool tables_missing(const ColArgs& c) {
+    const bool warp_size = c.ny == 512 || c.ny == 1024 || c.ny == 2048;
+    return warp_size && c.warp && (!c.tw1024 || !c.hhT || (c.ny == 2048 && (!c.tw2048l || !c.hN2)));
+}
+
+}  // namespace
+
+cudaError_t launch_cols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride,
+                            long long z_kstride, float2* A, long long a_bstride) {
+    if (tables_missing(c)) return cudaErrorInvalidValue;
+    return c.lowp ? cols_fwd<__half2>(c, s, Z, z_bstride, z_kstride, A, a_bstride)
+                  : cols_fwd<float2>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
+}
+
+cudaError_t launch_cols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
+                            long long q_bstride, long long q_kstride) {
+    if (tables_missing(c)) return cudaErrorInvalidValue;
+    return c.lowp ? cols_adj<false, __half2>(c, s, V, v_bstride, Q, q_bstride, q_kstride)
+                  : cols_adj<false, float2>(c, s, V, v_bstride, Q, q_bstride, q_kstride);
+}
+
+cudaError_t launch_cols_adj_full(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
+                                 long long q_bstride, long long q_kstride) {
+    if (tables_missing(c) || c.lowp) return cudaErrorInvalidValue;
+    return cols_adj<true, float2>(c, s, V, v_bstride, Q, q_bstride, q_kstride);
 }
 
 cudaError_t launch_cols_spec(int ny, dim3 grid, cudaStream_t s, const float2* S, int nxh,
@@ -336,37 +329,6 @@ cudaError_t launch_cols_adj_sep_tm(int ny, dim3 grid, cudaStream_t s, float2* V,
         kt_cols_adj<false><<<grid, kWColWarps * 32, kTColSmem, s>>>(V, v_bstride, hhT, hN, box, nxh, Q, q_bstride,
                                                                     q_kstride, tw1024, status, wait_limit,
                                                                     skip_copy, sep);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cols_adj_full(int ny, dim3 grid, cudaStream_t s, const float2* V, long long v_bstride,
-                                 const float2* hh, const float2* hN, int m, const Box* box, int nxh,
-                                 float2* Q, long long q_bstride, long long q_kstride,
-                                 const float2* tw, const float2* hhT, const float2* tw1024, int* status,
-                                 long long wait_limit, int skip_copy) {
-    if (ny == kWarpN) {
-        kw_cols_adj<true, float2><<<grid, kWColWarps * 32, kWColSmem, s>>>(
-            V, v_bstride, hhT, hN, nullptr, m, box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit,
-            skip_copy);
-        return cudaGetLastError();
-    }
-    if (ny == 512 && hhT && tw1024) {
-        kw_cols_adj<true, float2, false, 512><<<grid, kWColWarps * 32, kw_col_smem<512>(), s>>>(
-            V, v_bstride, hhT, hN, nullptr, m, box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit,
-            skip_copy);
-        return cudaGetLastError();
-    }
-    switch (ny) {
-#define X(N)                                                                                   \
-    case N:                                                                                    \
-        k_cols_adj<N, true, float2><<<grid, ColCfg<N>::NT, ColCfg<N>::SMEM, s>>>(                \
-            V, v_bstride, hh, hN, nullptr, m, box, nxh, Q, q_bstride, q_kstride, tw);         \
-        break;
-        PCE_COL_SIZES(X)
-#undef X
-        default:
-            return cudaErrorInvalidValue;
-    }
     return cudaGetLastError();
 }
 

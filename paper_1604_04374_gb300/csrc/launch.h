@@ -61,20 +61,38 @@ cudaError_t launch_wrows_r2c(int nx, int nb, cudaStream_t s, const float* src, l
 cudaError_t launch_wrows_c2r(int nx, int nb, cudaStream_t s, const float2* src, long long src_bstride, int nrows, float* dst,
                              long long dst_bstride, float scale, const float2* tw1024);
 
-cudaError_t launch_cols_fwd(int ny, dim3 grid, cudaStream_t s, const float2* Z, long long z_bstride,
-                            long long z_kstride, const void* hh, const void* hN, const float* hscale,
-                            bool lowp, int m,
-                            const Box* box, int nxh, float2* A, long long a_bstride,
-                            const float2* tw, const void* hhT, const float2* tw1024, int* status,
-                            long long wait_limit, int skip_copy, bool warp = true,
-                            const void* hN2 = nullptr, const float2* tw2048l = nullptr);
+// What the column passes of a plan (not its separable fast path) read: nb right-hand
+// sides of a launch, the spectra in both layouts (hh [m][ny][nxh], hhT per column; the
+// Nyquist column hN, hN2 split by parity for ny = 2048; half2 with hscale when lowp),
+// twiddles, the plan's status word.  warp: the one-warp column kernels where they
+// exist (ny = 512, 1024, 2048), else block Stockham.  zblk: col_frames' frame blocks,
+// 0 when the frame kernels do not hold the windows (ny = 2048).  split: CTAs that share
+// a column tile's terms in the adjoint.
+struct ColArgs {
+    int ny = 0, nxh = 0, nb = 1, m = 0;
+    unsigned split = 1;
+    bool lowp = false, warp = true;
+    const void *hh = nullptr, *hN = nullptr, *hhT = nullptr, *hN2 = nullptr;
+    const float* hscale = nullptr;
+    const Box* box = nullptr;   // device
+    int zblk = 0;
+    const float2 *tw = nullptr, *tw1024 = nullptr, *tw2048l = nullptr;
+    int* status = nullptr;
+    long long wait_limit = 0;
+    int skip_copy = 0;
+};
+// Most frame blocks (32 rows) of a window's rows in the column kernels of ny = 512, 1024
+// or 2048 rows (ckernels.cuh); false where those kernels do not serve the windows.
+// box: host.
+bool col_frames(int ny, const Box* box, int m, int& zblk);
 
-cudaError_t launch_cols_adj(int ny, dim3 grid, cudaStream_t s, const float2* V, long long v_bstride,
-                            const void* hh, const void* hN, const float* hscale, bool lowp, int m,
-                            const Box* box, int nxh, float2* Q, long long q_bstride, long long q_kstride,
-                            const float2* tw, const void* hhT, const float2* tw1024, int* status,
-                            long long wait_limit, int skip_copy, bool warp = true,
-                            const void* hN2 = nullptr, const float2* tw2048l = nullptr);
+cudaError_t launch_cols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride,
+                            long long z_kstride, float2* A, long long a_bstride);
+cudaError_t launch_cols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
+                            long long q_bstride, long long q_kstride);
+// every row of Q (the window gradient); FP32 storage
+cudaError_t launch_cols_adj_full(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
+                                 long long q_bstride, long long q_kstride);
 
 cudaError_t launch_cols_spec(int ny, dim3 grid, cudaStream_t s, const float2* S, int nxh,
                              float2* hh, float2* hN, const float2* tw);
@@ -124,12 +142,6 @@ cudaError_t launch_cols_adj_sep_tm(int ny, dim3 grid, cudaStream_t s, float2* V,
                                    const float2* hhT, const float2* hN, const Box* box, int nxh, float2* Q,
                                    long long q_bstride, long long q_kstride, const float2* tw1024, int* status,
                                    long long wait_limit, int skip_copy, const SepTerms& sep);
-
-cudaError_t launch_cols_adj_full(int ny, dim3 grid, cudaStream_t s, const float2* V, long long v_bstride,
-                                 const float2* hh, const float2* hN, int m, const Box* box, int nxh,
-                                 float2* Q, long long q_bstride, long long q_kstride,
-                                 const float2* tw, const float2* hhT, const float2* tw1024, int* status,
-                                 long long wait_limit, int skip_copy);
 
 cudaError_t launch_cols_grad_h(int ny, dim3 grid, cudaStream_t s, const float2* Z, long long z_bstride,
                                long long z_kstride, int nb, const float2* Rh, const float2* RhN,

@@ -467,9 +467,6 @@ namespace {
 // Window and spectrum storage the fused kernels read.
 const void* wstore(pce_plan_t p) { return p->lowp ? p->wbox16 : (const void*)p->wbox; }
 const void* hstore(pce_plan_t p) { return p->lowp ? p->hh16 : (const void*)p->hh; }
-const void* hNstore(pce_plan_t p) { return p->lowp ? p->hN16 : (const void*)p->hN; }
-const void* hTstore(pce_plan_t p) { return p->lowp ? p->hhT16 : (const void*)p->hhT; }
-const void* hN2store(pce_plan_t p) { return p->lowp ? p->hN2_16 : (const void*)p->hN2; }
 
 pce_status validate_shape(int ndims, const int64_t* shape, int& ny, int& nx) {
     if (ndims != 1 && ndims != 2) return fail(PCE_ERR_INVALID, "ndims must be 1 or 2 (got %d)", ndims);
@@ -577,6 +574,7 @@ pce_status setup_windows(pce_plan* p, const float* w, cudaStream_t s) {
         p->box[k] = b;
         p->nrmax = std::max(p->nrmax, b.nr);
     }
+    if (!pce::col_frames(ny, p->box.data(), m, p->zblk)) p->zblk = 0;
     pce_status st = dev_alloc(&p->wbox, (size_t)std::max<long long>(woff, 4));
     if (st) return st;
     for (int k = 0; k < m; ++k) {
@@ -1472,6 +1470,32 @@ pce_status apply_plain(pce_plan_t p, const float* in, float* out, int64_t batch,
     return PCE_OK;
 }
 
+// The column passes' arguments for nb right-hand sides (launch.h).
+pce::ColArgs col_args(const pce_plan* p, int nb, bool warp, bool lowp, unsigned split = 1) {
+    pce::ColArgs c;
+    c.ny = p->ny;
+    c.nxh = p->nx / 2;
+    c.nb = nb;
+    c.m = p->m;
+    c.split = split;
+    c.lowp = lowp;
+    c.warp = warp;
+    c.hh = lowp ? p->hh16 : p->hh;
+    c.hN = lowp ? p->hN16 : p->hN;
+    c.hhT = lowp ? p->hhT16 : p->hhT;
+    c.hN2 = lowp ? p->hN2_16 : p->hN2;
+    c.hscale = p->hscale;
+    c.box = p->d_box;
+    c.zblk = p->zblk;
+    c.tw = p->twy;
+    c.tw1024 = p->tw1024;
+    c.tw2048l = p->tw2048l;
+    c.status = p->d_status;
+    c.wait_limit = p->wait_limit;
+    c.skip_copy = p->skip_copy;
+    return c;
+}
+
 // CTAs that share a column tile's terms in the adjoint: doubled while the grid of ctas
 // column CTAs fills no more than the GPU's `per_sm` resident CTAs an SM and every CTA
 // keeps a unit of work (a term or a slot).  Beyond one wave a split only adds work, an
@@ -1630,13 +1654,13 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
     const bool wrows = rowv == 2 && (nx == 1024 || nx == 512) && p->tw1024 != nullptr;
     const int brv = rowv == 0 ? 0 : 1;
     const int fpc = pce::rows_pairs_per_cta(nx);
-    const int cpc = pce::cols_columns_per_cta(ny);  // same for both variants
+    const int cpc = warp && ny == 2048 ? 4 : pce::cols_columns_per_cta(ny);   // columns a CTA
     const int npairs = (ny + 1) / 2;
-    // column CTAs per SM, and the units the adjoint's column tile divides into.  Columns
-    // of 2048 keep a tile in one CTA; so does a batch's lane, where every further CTA
-    // repeats the FFT of V while other tasks could use the SM
-    const int col_ctas = septm ? (ny == 1024 ? 4 : 6) : warp && ny == 1024 ? 3 : warp && ny == 512 ? 5 : 4;
-    const bool whole = !adjoint || (warp && ny == 2048) || scr.beside;
+    // column CTAs per SM, and the units the adjoint's column tile divides into: one in a
+    // batch's lane, where every further CTA repeats the FFT of V while other tasks could
+    // use the SM
+    const int col_ctas = !warp ? 4 : ny == 512 ? 6 : ny == 2048 ? 2 : 4;
+    const bool whole = !adjoint || scr.beside;
     const int col_units = whole ? 1 : sepx ? p->nslots : m;
     for (long long b0 = 0; b0 < batch && e == cudaSuccess; b0 += bal) {
         const int nb = (int)std::min<long long>(bal, batch - b0);
@@ -1758,9 +1782,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
                 });
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_COLS_FWD, s, [&] {
-                    return pce::launch_cols_fwd(ny, cgrid, s, scr.Z, zb, zk,
-                                                hstore(p), hNstore(p), p->hscale, p->lowp, m, p->d_box, nxh, scr.A, ab, p->twy, hTstore(p), p->tw1024, p->d_status, p->wait_limit, p->skip_copy, warp,
-                                                hN2store(p), p->tw2048l);
+                    return pce::launch_cols_fwd(col_args(p, nb, warp, p->lowp), s, scr.Z, zb, zk, scr.A, ab);
                 });
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_ROWS_C2R, s, [&] {
@@ -1777,9 +1799,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
             });
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_COLS_ADJ, s, [&] {
-                    return pce::launch_cols_adj(ny, cgrid, s, scr.A, ab,
-                                                hstore(p), hNstore(p), p->hscale, p->lowp, m, p->d_box, nxh, scr.Z, zb, zk, p->twy, hTstore(p), p->tw1024, p->d_status, p->wait_limit, p->skip_copy, warp,
-                                                hN2store(p), p->tw2048l);
+                    return pce::launch_cols_adj(col_args(p, nb, warp, p->lowp, cgrid.z), s, scr.A, ab, scr.Z, zb, zk);
                 });
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_ROWS_ADJ, s, [&] {
@@ -2099,8 +2119,7 @@ extern "C" pce_status pce_backward(pce_plan_t p, const float* u, const float* r,
                                             reinterpret_cast<float2*>(dhhat), scale, acc, p->twy);
         }
         if (dw && e == cudaSuccess) {
-            e = pce::launch_cols_adj_full(ny, dim3(nb, tiles), s, S, H, p->hh, p->hN, m, p->d_box, nxh, Qf,
-                                          (long long)m * H, H, p->twy, p->hhT, p->tw1024, p->d_status, p->wait_limit, p->skip_copy);
+            e = pce::launch_cols_adj_full(col_args(p, nb, true, false), s, S, H, Qf, (long long)m * H, H);
             if (e == cudaSuccess)
                 e = pce::launch_rows_grad_w(nx, dim3((npairs + gpc - 1) / gpc, m), s, Qf, (long long)m * H, H,
                                             ny, nb, ub, P, dw, scale, acc, p->twx);
@@ -2187,10 +2206,7 @@ extern "C" pce_status pce_apply_noalloc(pce_plan_t plan, const float* u, float* 
                                      ny, wstore(plan), plan->lowp, plan->d_box, plan->items, plan->nitems, scrZ, zb, zk,
                                      plan->twx, plan->tw1024);
         if (e == cudaSuccess)
-            e = pce::launch_cols_fwd(ny, dim3(nb, (nxh + cpc - 1) / cpc), s, scrZ, zb, zk, hstore(plan),
-                                     hNstore(plan), plan->hscale, plan->lowp, m, plan->d_box, nxh, scrA, ab,
-                                     plan->twy, hTstore(plan), plan->tw1024, plan->d_status, plan->wait_limit,
-                                     plan->skip_copy, plan->col_variant != 1, hN2store(plan), plan->tw2048l);
+            e = pce::launch_cols_fwd(col_args(plan, nb, plan->col_variant != 1, plan->lowp), s, scrZ, zb, zk, scrA, ab);
         if (e == cudaSuccess)
             e = pce::launch_rows_c2r(nx, dim3((npairs + fpc - 1) / fpc, nb), s, scrA, ab, ny, y + b0 * P, P,
                                      scale, plan->twx, plan->tw1024);

@@ -58,6 +58,7 @@ struct pce_plan {
     float2* scrZ = nullptr;
     float2* scrA = nullptr;
     int nrmax = 0;
+    int zblk = 0;               // frame blocks of the dense column kernels (launch.h col_frames), 0: not served
     int bchunk = 1;             // right-hand sides the plan's scratch holds
     // autotuned choices (pce_plan_autotune); untuned plans: run_chunk 0 (all the scratch holds),
     // column variant 2 where separable kernels exist, row variant 1
