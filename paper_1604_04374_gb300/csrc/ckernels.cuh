@@ -17,15 +17,28 @@
 //    adjoint: the column spectrum of V) lives in tensor memory (tmem.cuh), which
 //    leaves 128 registers a thread and 16 warps an SM (20 and more at 512 points);
 //  - a term's rows are staged for the CTA by cp.async while the previous term's FFT
-//    runs, on a frame that starts at a multiple of 32 rows (the box's first row
-//    rounded down, zeros around the box): register q then reads tile rows lane + 32 j
-//    with j = q - frame, the same for the whole warp, without per-lane index or
-//    bounds arithmetic, and absent blocks are not read at all;
+//    runs, on a frame that starts at a multiple of 32 rows, 32 s (the box's first row
+//    rounded down), zeros around the box.  The warps transform the frame's rows in
+//    place, x'[i] = x[32 s + i], i < NF: no index or bounds arithmetic a value, for
+//    PAR = 2 no second half (i < 1024), and where every frame holds at most NF / 2
+//    rows (HALF; Lemma 3.2) an FFT without the butterflies of its zero half, an
+//    inverse without the outputs outside the frame.  The shift costs nothing:
+//    FFT(x)[f] = W^(32 s f) FFT(x')[f], and with f = PAR (p + 32 j) + par the phase is
+//    W^(32 s (PAR p + par)), independent of j, so it is folded into the twiddles of
+//    the four-step FFT, which the first transform leaves at register p (forward) or
+//    lane p (inverse): one table a value of (s, par) and direction (col_tables);
 //  - the next term's spectrum is started towards L2 a term ahead (one bulk prefetch
 //    a warp); the forward brings it into the warp's transpose tile during the second
 //    half of the FFT, the adjoint loads it straight into registers;
+//    The twiddle tables cost 2 MB a plan of 2048 rows (0.5 and 0.1 MB at 1024 and 512);
 //  - the power-of-two scale of a term's reduced spectrum is applied where the fewest
 //    values pass (exact): to the staged rows (forward), to the stored rows (adjoint).
+//
+// 2048^2, m = 64, 4 right-hand sides, reduced storage, forward, whole apply: 3742 us
+// with the register kernels, 2286 with tensor memory and frames read behind uniform
+// branches, 1907 with the shifted transforms.  At 2048^2, m = 16, 2 right-hand sides
+// the forward / adjoint kernels execute 123 / 115 M warp instructions (164 / 132 M
+// before the shift) at 57 % of the issue slots: 192 / 185 us.
 #pragma once
 
 #include "tkernels.cuh"
@@ -57,37 +70,46 @@ __host__ __device__ constexpr int kc_tm_cols() { return PAR * 2 * (NF / 32); }
 // CTAs per SM the kernels are compiled for (128 registers; 80 at 512 points)
 template <int NF, int PAR>
 __host__ __device__ constexpr int kc_min_ctas() { return NF == 512 ? 6 : PAR == 1 ? 4 : 2; }
-// shared memory: the transpose tiles, and in the forward zblk blocks of 32 rows
+// shared memory: the transpose tiles, and in the forward a term's frame rows
 template <int NF, int PAR>
-__host__ __device__ constexpr int kc_smem(int zblk) {
-    return (kCCols * PAR * NF + zblk * 32 * kCCols) * (int)sizeof(float2);
+__host__ __device__ constexpr int kc_smem(int rows) {
+    return (kCCols * PAR * warp_tile(NF) + rows * kCCols) * (int)sizeof(float2);
 }
 
-// Frame of a term's rows: tile row i holds row 32 s + i of the column (mod NY),
-// i < 32 nblk.  Boxes that would cover a frame block of the period twice take
-// the whole period (PAR = 1 only).
+// Frame of a term's rows: frame row i is row 32 s + i of the column (mod NY), the
+// box's row r is frame row (a + r) mod NY.  Boxes that do not fit a frame of NF rows
+// take the whole period (PAR = 1; columns of 2048 with such boxes use wkernels2.cuh).
 struct CFrame {
-    int s, nblk;
+    int s, a;
 };
-template <int NF, int NY>
+template <int NF>
 __host__ __device__ __forceinline__ CFrame col_frame(const Box& b) {
     const int a = b.r0 & 31;
-    if (a + b.nr > NF) return CFrame{0, NF / 32};
-    return CFrame{b.r0 >> 5, (a + b.nr + 31) >> 5};
+    return a + b.nr > NF ? CFrame{0, b.r0} : CFrame{b.r0 >> 5, a};
+}
+
+// Phased twiddles: tab[dir][s][par][p * 32 + l] = W_NF^(l p) W_NY^(32 s (PAR k + par)),
+// k = p for dir 0 (forward), k = l for dir 1 (inverse, used conjugated).
+template <int NF, int PAR>
+__host__ __device__ constexpr int col_table_len() { return NF * PAR * (NF * PAR / 32); }
+template <int NF, int PAR>
+__device__ __forceinline__ const float2* col_table(const float2* tab, int dir, int s, int par) {
+    return tab + (long long)dir * col_table_len<NF, PAR>() + (s * PAR + par) * NF;
 }
 
 __device__ __forceinline__ void bulk_prefetch_l2(const void* p, unsigned bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// Cooperative async copy of the frame f of a term's box rows (src [nr][nxh],
-// columns col0 .. col0 + 3) into the swizzled tile, zeros outside the box.
-template <int NY, int NT>
+// Cooperative async copy of a term's box rows (src [nr][nxh], columns col0 ..
+// col0 + 3) to ROWS rows of its frame in the swizzled tile, zeros outside the box.
+template <int NY, int ROWS, int NT>
 __device__ __forceinline__ void frame_load(float2* tile, const float2* __restrict__ src, const Box& b, CFrame f,
                                            int nxh, int col0) {
-    for (int e = threadIdx.x; e < f.nblk * 32 * kCCols; e += NT) {
+#pragma unroll 4
+    for (int e = threadIdx.x; e < ROWS * kCCols; e += NT) {
         const int i = e >> 2, c = e & 3;
-        const int r = wrap(32 * f.s + i - b.r0, NY);
+        const int r = wrap(i - f.a, NY);
         const bool ok = r < b.nr && col0 + c < nxh;
         cp_async8(tile + tix(i, c), src + (ok ? (long long)r * nxh + col0 + c : 0), ok);
     }
@@ -102,7 +124,7 @@ __device__ __forceinline__ float2 half_partner(const float2* tr, int f, int par)
 }
 
 // The four columns' inverse transforms (transpose tiles of the CTA, element n of
-// column c, half p at (c PAR + p) NF + ((n + 4 c) mod NF)) combined and stored:
+// column c, half p at (c PAR + p) warp_tile(NF) + ((n + 4 c) mod NF)) combined and stored:
 // rows i < nr of dst ([rows][nxh], columns col0 ..) from rows r0 + i (mod NY),
 // times sc.  Two columns a 16-byte store where dst allows it.
 template <int NF, int PAR, int NT>
@@ -111,10 +133,10 @@ __device__ __forceinline__ void store_halves(float2* __restrict__ dst, const flo
     constexpr int NY = NF * PAR;
     auto get = [&](int g, int c) {
         const int n = (g + 4 * c) & (NF - 1);
-        const float2* t = tiles + c * PAR * NF;
+        const float2* t = tiles + c * PAR * warp_tile(NF);
         float2 x = t[n];
         if constexpr (PAR == 2) {
-            const float2 y = t[NF + n];
+            const float2 y = t[warp_tile(NF) + n];
             x = g < NF ? cadd(x, y) : csub(x, y);
         }
         return cscale(x, sc);
@@ -134,20 +156,22 @@ __device__ __forceinline__ void store_halves(float2* __restrict__ dst, const flo
     }
 }
 
-// F2.  Grid (batch, ceil(NXh / 4)), 128 PAR threads, kc_smem<NF, PAR>(zblk)
-// bytes; zblk >= every term's frame blocks.
-template <int NF, int PAR, typename HT>
+// F2.  Grid (batch, ceil(NXh / 4)), 128 PAR threads, kc_smem<NF, PAR>(frame rows)
+// bytes.  tab: the phased twiddles (forward part), tw: the plain ones.
+template <int NF, int PAR, bool HALF, typename HT>
 __global__ void __launch_bounds__(kCCols * PAR * 32, (kc_min_ctas<NF, PAR>()))
 kc_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstride, const HT* __restrict__ hhT,
             const HT* __restrict__ hN, const float* __restrict__ hscale, int m, const Box* __restrict__ box, int NXh,
             float2* __restrict__ A, long long a_bstride, const float2* __restrict__ tw,
-            const float2* __restrict__ tw2048l, int* __restrict__ status, long long wait_limit, int skip_copy) {
+            const float2* __restrict__ tab, const float2* __restrict__ tw2048l, int* __restrict__ status,
+            long long wait_limit, int skip_copy) {
+    constexpr int ROWS = HALF ? NF / 2 : NF;
     constexpr int NY = NF * PAR, QN = NF / 32, NQ = QN / 8, NT = kCCols * PAR * 32;
     extern __shared__ __align__(16) float2 smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cl = warp / PAR, par = warp % PAR;
-    float2* tr = smem + warp * NF;                  // this warp's transpose tile
-    float2* tile = smem + kCCols * PAR * NF;        // the term's rows
+    float2* tr = smem + warp * warp_tile(NF);           // this warp's transpose tile
+    float2* tile = smem + kCCols * PAR * warp_tile(NF);   // the term's rows
     __shared__ unsigned long long bars[kCCols * PAR];
     __shared__ unsigned tm_slot;
     const int b = blockIdx.x;
@@ -185,43 +209,36 @@ kc_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     int k = next_k(0);
     if (k < kend) {
         const Box bx = box[k];
-        frame_load<NY, NT>(tile, Zb + k * z_kstride, bx, col_frame<NF, NY>(bx), NXh, col0);
+        frame_load<NY, ROWS, NT>(tile, Zb + k * z_kstride, bx, col_frame<NF>(bx), NXh, col0);
         if (lane == 0 && cv) bulk_prefetch_l2(hcol + k * hstride, NF * sizeof(HT));
     }
     while (k < kend) {
-        const CFrame f = col_frame<NF, NY>(box[k]);
+        const float2* twk = col_table<NF, PAR>(tab, 0, col_frame<NF>(box[k]).s, par);
         const int kn = next_k(k + 1);
         cp_async_wait_all();
         __syncthreads();   // the term's rows have landed
         float2 v[QN];
         const float sk = hscale_of<HT>(hscale, k);
         const float2* tb = tile + 4 * lane + sw;
+        const float2 wls = cscale(wl, sk);
 #pragma unroll
-        for (int q = 0; q < QN; ++q) {
-            const int j = (q - f.s) & (QN - 1);   // the same for the whole warp
-            v[q] = make_float2(0.f, 0.f);
-            if (j < f.nblk) {
-                float2 x = tb[128 * j];
-                // PAR = 2: rows n and n + 1024 never both hold a frame block, so the even
-                // half's input is either one and the odd half's x[n] or -x[n + 1024]
-                if (PAR == 2 && par)
-                    x = cmul(cmul(x, cscale(wl, (f.s + j) & QN ? -sk : sk)), w64(q));
-                else if (sizeof(HT) != sizeof(float2))
-                    x = cscale(x, sk);
-                v[q] = x;
-            }
+        for (int q = 0; q < ROWS / 32; ++q) {
+            float2 x = tb[128 * q];
+            if (PAR == 2 && par) x = cmul(cmul(x, wls), w64(q));   // W2048^i of the odd half
+            else if (sizeof(HT) != sizeof(float2)) x = cscale(x, sk);
+            v[q] = x;
         }
         __syncthreads();   // every warp has read its rows: the next term's may come
         if (kn < kend) {
             const Box bn = box[kn];
-            frame_load<NY, NT>(tile, Zb + kn * z_kstride, bn, col_frame<NF, NY>(bn), NXh, col0);
+            frame_load<NY, ROWS, NT>(tile, Zb + kn * z_kstride, bn, col_frame<NF>(bn), NXh, col0);
             if (lane == 0 && cv) bulk_prefetch_l2(hcol + kn * hstride, NF * sizeof(HT));
         }
         const bool bulk = !dcn && cv && !failed;
         auto hook = [&] {
             if (bulk && lane == 0) bulk_load(tr, hcol + k * hstride, NF * sizeof(HT), bar, skip_copy);
         };
-        warp_fft<NF, false, kTmSplit, decltype(hook)>(v, tr, tw, hook);
+        warp_fft_phased<NF, false, HALF, false, decltype(hook)>(v, tr, twk, hook);
         if (bulk) {
             if (!mbar_wait(bar, parity, wait_limit)) {
                 failed = true;
@@ -264,7 +281,7 @@ kc_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     }
     float2 acc[QN];
     tm_loadq<QN>(t_acc, acc);
-    warp_fft<NF, true, kTmSplit>(acc, tr, tw);
+    warp_fft<NF, true, kTmSplit, NoHook, true>(acc, tr, tw);
     if constexpr (PAR == 2) {
         if (par) {
 #pragma unroll
@@ -280,19 +297,21 @@ kc_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
 }
 
 // G1b + G2.  Grid (batch, ceil(NXh / 4), split), 128 PAR threads,
-// kc_smem<NF, PAR>(0) bytes.  FULL: every row of Q (the window gradient).  split:
+// kc_smem<NF, PAR>(0) bytes.  WHOLE: the inverse transforms give the whole column (not
+// HALF), for boxes that no frame holds and for full (every row of Q: the window gradient).  split:
 // CTA z of a column tile takes its share of the terms and forms the FFT of V itself.
-template <int NF, int PAR, bool FULL, typename HT>
+template <int NF, int PAR, bool WHOLE, bool HALF, typename HT>
 __global__ void __launch_bounds__(kCCols * PAR * 32, (kc_min_ctas<NF, PAR>()))
 kc_cols_adj(const float2* __restrict__ V, long long v_bstride, const HT* __restrict__ hhT, const HT* __restrict__ hN,
             const float* __restrict__ hscale, int m, const Box* __restrict__ box, int NXh, float2* __restrict__ Q,
             long long q_bstride, long long q_kstride, const float2* __restrict__ tw,
-            const float2* __restrict__ tw2048l) {
+            const float2* __restrict__ tab, const float2* __restrict__ tw2048l, int full) {
+    constexpr int QS = HALF ? NF / 64 : NF / 32;   // output values a lane needs
     constexpr int NY = NF * PAR, QN = NF / 32, NQ = QN / 8, NT = kCCols * PAR * 32;
     extern __shared__ __align__(16) float2 smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cl = warp / PAR, par = warp % PAR;
-    float2* tr = smem + warp * NF;
+    float2* tr = smem + warp * warp_tile(NF);
     __shared__ unsigned tm_slot;
     const int b = blockIdx.x;
     const int col0 = blockIdx.y * kCCols, col = col0 + cl;
@@ -308,7 +327,7 @@ kc_cols_adj(const float2* __restrict__ V, long long v_bstride, const HT* __restr
     const long long hstride = (long long)NXh * PAR * NF;
     const int kend = share_beg(m, blockIdx.z + 1, gridDim.z);
     auto next_k = [&](int k) {
-        while (!FULL && k < kend && box[k].nr == 0) ++k;
+        while (!full && k < kend && box[k].nr == 0) ++k;
         return k;
     };
     int k = next_k(share_beg(m, blockIdx.z, gridDim.z));
@@ -334,7 +353,7 @@ kc_cols_adj(const float2* __restrict__ V, long long v_bstride, const HT* __restr
             }
         }
         __syncthreads();   // every warp has read its column: the transpose tiles are free
-        warp_fft<NF, false, kTmSplit>(v, tr, tw);
+        warp_fft<NF, false, kTmSplit, NoHook, true>(v, tr, tw);
         tm_storeq<QN>(t_hold, v);
         tm_wait_st();
     }
@@ -374,20 +393,23 @@ kc_cols_adj(const float2* __restrict__ V, long long v_bstride, const HT* __restr
                 for (int j = 0; j < 8; ++j) p[8 * qq + j] = cmulc(x[j], p[8 * qq + j]);
             }
         }
-        warp_fft<NF, true, kTmSplit>(p, tr, tw);
+        // frame rows lane + 32 q of the inverse (WHOLE: rows of the column)
+        const Box bx = box[k];
+        const CFrame f = col_frame<NF>(bx);
+        if constexpr (WHOLE) warp_fft<NF, true, kTmSplit, NoHook, true>(p, tr, tw);
+        else warp_fft_phased<NF, true, false, HALF>(p, tr, col_table<NF, PAR>(tab, 1, f.s, par));
         if constexpr (PAR == 2) {
             if (par) {
 #pragma unroll
-                for (int q = 0; q < QN; ++q) p[q] = cmulc(cmulc(p[q], wl), w64(q));
+                for (int q = 0; q < QS; ++q) p[q] = cmulc(cmulc(p[q], wl), w64(q));
             }
         }
         __syncwarp();
 #pragma unroll
-        for (int q = 0; q < QN; ++q) tr[(lane + 32 * q + 4 * cl) & (NF - 1)] = p[q];
+        for (int q = 0; q < QS; ++q) tr[(lane + 32 * q + 4 * cl) & (NF - 1)] = p[q];
         __syncthreads();
-        const Box bx = box[k];
-        store_halves<NF, PAR, NT>(Q + b * q_bstride + k * q_kstride, smem, FULL ? 0 : bx.r0, FULL ? NY : bx.nr, NXh,
-                                  col0, sk);
+        store_halves<NF, PAR, NT>(Q + b * q_bstride + k * q_kstride, smem,
+                                  full ? 0 : WHOLE ? bx.r0 : f.a, full ? NY : bx.nr, NXh, col0, sk);
         __syncthreads();   // the transpose tiles are free again
         k = kn;
     }

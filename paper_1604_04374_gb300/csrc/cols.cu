@@ -38,11 +38,13 @@ int cols_smem(int ny) {
 
 template <int NF, int PAR, typename HT>
 cudaError_t prepare_ccols_of() {
-    const void* fns[] = {(const void*)kc_cols_fwd<NF, PAR, HT>, (const void*)kc_cols_adj<NF, PAR, false, HT>,
-                         (const void*)kc_cols_adj<NF, PAR, true, float2>};
+    const void* fns[] = {(const void*)kc_cols_fwd<NF, PAR, false, HT>, (const void*)kc_cols_fwd<NF, PAR, true, HT>,
+                         (const void*)kc_cols_adj<NF, PAR, false, false, HT>,
+                         (const void*)kc_cols_adj<NF, PAR, false, true, HT>,
+                         (const void*)kc_cols_adj<NF, PAR, true, false, HT>};
     for (const void* f : fns) {
         const cudaError_t e =
-            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kc_smem<NF, PAR>(NF / 32));
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kc_smem<NF, PAR>(NF));
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -108,19 +110,24 @@ cudaError_t prepare_cols() {
     return e;
 }
 
-bool col_frames(int ny, const Box* box, int m, int& zblk) {
-    zblk = 1;
+int col_frame_rows(int ny, const Box* box, int m) {
+    if (ny != 512 && ny != 1024 && ny != 2048) return 0;
     const int nf = ny == 512 ? 512 : 1024;
-    if (ny != 512 && ny != 1024 && ny != 2048) return false;
+    int rows = 1;
     for (int k = 0; k < m; ++k) {
-        if (box[k].nr == 0) continue;
-        if (ny == 2048 && (box[k].r0 & 31) + box[k].nr > nf) return false;
-        const CFrame f = ny == 512    ? col_frame<512, 512>(box[k])
-                         : ny == 1024 ? col_frame<1024, 1024>(box[k])
-                                      : col_frame<1024, 2048>(box[k]);
-        zblk = f.nblk > zblk ? f.nblk : zblk;
+        const int need = (box[k].r0 & 31) + box[k].nr;
+        if (box[k].nr == 0 || need <= rows) continue;
+        if (need > nf && ny == 2048) return 0;
+        rows = need < nf ? need : nf;
     }
-    return true;
+    return rows;
+}
+
+long long col_table_size(int ny) {
+    return 2ll * (ny == 512    ? col_table_len<512, 1>()
+                  : ny == 1024 ? col_table_len<1024, 1>()
+                  : ny == 2048 ? col_table_len<1024, 2>()
+                               : 0);
 }
 
 namespace {
@@ -130,18 +137,23 @@ dim3 ccols_grid(int nb, int nxh, unsigned split) { return dim3(nb, (nxh + kCCols
 template <int NF, int PAR, typename HT>
 cudaError_t ccols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride, long long z_kstride,
                       float2* A, long long a_bstride) {
-    kc_cols_fwd<NF, PAR, HT><<<ccols_grid(c.nb, c.nxh, 1), kCCols * PAR * 32, kc_smem<NF, PAR>(c.zblk), s>>>(
+    const bool half = c.frame_rows <= NF / 2;
+    auto kernel = half ? kc_cols_fwd<NF, PAR, true, HT> : kc_cols_fwd<NF, PAR, false, HT>;
+    kernel<<<ccols_grid(c.nb, c.nxh, 1), kCCols * PAR * 32, kc_smem<NF, PAR>(half ? NF / 2 : NF), s>>>(
         Z, z_bstride, z_kstride, static_cast<const HT*>(c.hhT), static_cast<const HT*>(PAR == 2 ? c.hN2 : c.hN),
-        c.hscale, c.m, c.box, c.nxh, A, a_bstride, c.tw1024, c.tw2048l, c.status, c.wait_limit, c.skip_copy);
+        c.hscale, c.m, c.box, c.nxh, A, a_bstride, c.tw1024, c.tab, c.tw2048l, c.status, c.wait_limit, c.skip_copy);
     return cudaGetLastError();
 }
 
-template <int NF, int PAR, bool FULL, typename HT>
-cudaError_t ccols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
+template <int NF, int PAR, typename HT>
+cudaError_t ccols_adj(const ColArgs& c, bool full, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
                       long long q_bstride, long long q_kstride) {
-    kc_cols_adj<NF, PAR, FULL, HT><<<ccols_grid(c.nb, c.nxh, c.split), kCCols * PAR * 32, kc_smem<NF, PAR>(0), s>>>(
+    auto kernel = full || c.frame_rows == 0     ? kc_cols_adj<NF, PAR, true, false, HT>
+                  : c.frame_rows <= NF / 2 ? kc_cols_adj<NF, PAR, false, true, HT>
+                                           : kc_cols_adj<NF, PAR, false, false, HT>;
+    kernel<<<ccols_grid(c.nb, c.nxh, c.split), kCCols * PAR * 32, kc_smem<NF, PAR>(0), s>>>(
         V, v_bstride, static_cast<const HT*>(c.hhT), static_cast<const HT*>(PAR == 2 ? c.hN2 : c.hN), c.hscale, c.m,
-        c.box, c.nxh, Q, q_bstride, q_kstride, c.tw1024, c.tw2048l);
+        c.box, c.nxh, Q, q_bstride, q_kstride, c.tw1024, c.tab, c.tw2048l, full ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -150,7 +162,7 @@ cudaError_t cols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long lon
                      float2* A, long long a_bstride) {
     if (c.warp && c.ny == 512) return ccols_fwd<512, 1, HT>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
     if (c.warp && c.ny == 1024) return ccols_fwd<1024, 1, HT>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
-    if (c.warp && c.ny == 2048 && c.zblk > 0)
+    if (c.warp && c.ny == 2048 && c.frame_rows > 0)
         return ccols_fwd<1024, 2, HT>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
     if (c.warp && c.ny == 2048) {
         kw2_cols_fwd<HT><<<dim3(c.nb, (c.nxh + kW2Cols - 1) / kW2Cols), 128, kW2Smem, s>>>(
@@ -175,9 +187,9 @@ cudaError_t cols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long lon
 template <bool FULL, typename HT>
 cudaError_t cols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
                      long long q_bstride, long long q_kstride) {
-    if (c.warp && c.ny == 512) return ccols_adj<512, 1, FULL, HT>(c, s, V, v_bstride, Q, q_bstride, q_kstride);
-    if (c.warp && c.ny == 1024) return ccols_adj<1024, 1, FULL, HT>(c, s, V, v_bstride, Q, q_bstride, q_kstride);
-    if (c.warp && c.ny == 2048) return ccols_adj<1024, 2, FULL, HT>(c, s, V, v_bstride, Q, q_bstride, q_kstride);
+    if (c.warp && c.ny == 512) return ccols_adj<512, 1, HT>(c, FULL, s, V, v_bstride, Q, q_bstride, q_kstride);
+    if (c.warp && c.ny == 1024) return ccols_adj<1024, 1, HT>(c, FULL, s, V, v_bstride, Q, q_bstride, q_kstride);
+    if (c.warp && c.ny == 2048) return ccols_adj<1024, 2, HT>(c, FULL, s, V, v_bstride, Q, q_bstride, q_kstride);
     switch (c.ny) {
 #define X(N)                                                                                                     \
     case N:                                                                                                      \
@@ -195,7 +207,7 @@ cudaError_t cols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long lon
 // the one-warp column kernels index these tables: refuse to launch without them
 bool tables_missing(const ColArgs& c) {
     const bool warp_size = c.ny == 512 || c.ny == 1024 || c.ny == 2048;
-    return warp_size && c.warp && (!c.tw1024 || !c.hhT || (c.ny == 2048 && (!c.tw2048l || !c.hN2)));
+    return warp_size && c.warp && (!c.tw1024 || !c.tab || !c.hhT || (c.ny == 2048 && (!c.tw2048l || !c.hN2)));
 }
 
 }  // namespace

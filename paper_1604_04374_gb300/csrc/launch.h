@@ -65,9 +65,8 @@ cudaError_t launch_wrows_c2r(int nx, int nb, cudaStream_t s, const float2* src, 
 // sides of a launch, the spectra in both layouts (hh [m][ny][nxh], hhT per column; the
 // Nyquist column hN, hN2 split by parity for ny = 2048; half2 with hscale when lowp),
 // twiddles, the plan's status word.  warp: the one-warp column kernels where they
-// exist (ny = 512, 1024, 2048), else block Stockham.  zblk: col_frames' frame blocks,
-// 0 when the frame kernels do not hold the windows (ny = 2048).  split: CTAs that share
-// a column tile's terms in the adjoint.
+// exist (ny = 512, 1024, 2048), else block Stockham.  frame_rows: col_frame_rows(), tab
+// the phased twiddles.  split: CTAs that share a column tile's terms in the adjoint.
 struct ColArgs {
     int ny = 0, nxh = 0, nb = 1, m = 0;
     unsigned split = 1;
@@ -75,16 +74,18 @@ struct ColArgs {
     const void *hh = nullptr, *hN = nullptr, *hhT = nullptr, *hN2 = nullptr;
     const float* hscale = nullptr;
     const Box* box = nullptr;   // device
-    int zblk = 0;
-    const float2 *tw = nullptr, *tw1024 = nullptr, *tw2048l = nullptr;
+    int frame_rows = 0;
+    const float2 *tw = nullptr, *tw1024 = nullptr, *tab = nullptr, *tw2048l = nullptr;
     int* status = nullptr;
     long long wait_limit = 0;
     int skip_copy = 0;
 };
-// Most frame blocks (32 rows) of a window's rows in the column kernels of ny = 512, 1024
-// or 2048 rows (ckernels.cuh); false where those kernels do not serve the windows.
+// Frame rows the windows need in the column kernels of ny = 512, 1024 or 2048 rows
+// (ckernels.cuh; at most 512 or 1024), 0 where those kernels do not serve them.
 // box: host.
-bool col_frames(int ny, const Box* box, int m, int& zblk);
+int col_frame_rows(int ny, const Box* box, int m);
+// float2 of the phased twiddle tables of ny rows, both directions (0: none).
+long long col_table_size(int ny);
 
 cudaError_t launch_cols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride,
                             long long z_kstride, float2* A, long long a_bstride);

@@ -105,6 +105,23 @@ __global__ void k_twiddles_1024(float2* tw) {
     tw[idx] = make_float2((float)cs, (float)sn);
 }
 
+// Phased twiddles of the dense column kernels (ckernels.cuh col_table): nf points a
+// warp, par_n warps a column; product of the two phases as one FP64 angle.
+__global__ void k_col_tables(float2* tab, int nf, int par_n) {
+    const int ny = nf * par_n, len = ny * (ny / 32);
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= 2 * len) return;
+    const int dir = idx >= len, e = idx - dir * len;
+    const int sp = e / nf, s = sp / par_n, par = sp % par_n;
+    const int p = (e % nf) >> 5, l = e & 31;
+    // W_nf^(l p) W_ny^(32 s (par_n k + par)) = W_ny^j
+    const int k = dir ? l : p;
+    const int j = (par_n * l * p + 32 * s * (par_n * k + par)) & (ny - 1);
+    double sn, cs;
+    sincospi(-2.0 * (double)j / (double)ny, &sn, &cs);
+    tab[idx] = make_float2((float)cs, (float)sn);
+}
+
 // twN[j] = W_N^j for j < N (FP64 sincospi).
 __global__ void k_twiddles_N(float2* tw, long long n) {
     const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -519,7 +536,16 @@ pce_status make_twiddles(pce_plan* p, cudaStream_t s) {
         k_twiddles_1024<<<4, 256, 0, s>>>(p->tw1024);
         PCE_CK(cudaGetLastError());
     }
-    pce_status st = dev_alloc(&p->twx, (size_t)std::max(1, twiddle_len(p->nx)));
+    pce_status st;
+    if (p->ndims == 2) {
+        const long long n = pce::col_table_size(p->ny);
+        if ((st = dev_alloc(&p->col_tab, (size_t)n))) return st;
+        if (n > 0) {
+            k_col_tables<<<grid_for(n), 256, 0, s>>>(p->col_tab, p->ny == 512 ? 512 : 1024, p->ny == 2048 ? 2 : 1);
+            PCE_CK(cudaGetLastError());
+        }
+    }
+    st = dev_alloc(&p->twx, (size_t)std::max(1, twiddle_len(p->nx)));
     if (st) return st;
     k_twiddles<<<grid_for(twiddle_len(p->nx)), 256, 0, s>>>(p->twx, p->nx);
     PCE_CK(cudaGetLastError());
@@ -574,7 +600,7 @@ pce_status setup_windows(pce_plan* p, const float* w, cudaStream_t s) {
         p->box[k] = b;
         p->nrmax = std::max(p->nrmax, b.nr);
     }
-    if (!pce::col_frames(ny, p->box.data(), m, p->zblk)) p->zblk = 0;
+    p->frame_rows = pce::col_frame_rows(ny, p->box.data(), m);
     pce_status st = dev_alloc(&p->wbox, (size_t)std::max<long long>(woff, 4));
     if (st) return st;
     for (int k = 0; k < m; ++k) {
@@ -1486,7 +1512,8 @@ pce::ColArgs col_args(const pce_plan* p, int nb, bool warp, bool lowp, unsigned 
     c.hN2 = lowp ? p->hN2_16 : p->hN2;
     c.hscale = p->hscale;
     c.box = p->d_box;
-    c.zblk = p->zblk;
+    c.frame_rows = p->frame_rows;
+    c.tab = p->col_tab;
     c.tw = p->twy;
     c.tw1024 = p->tw1024;
     c.tw2048l = p->tw2048l;

@@ -58,7 +58,8 @@ struct pce_plan {
     float2* scrZ = nullptr;
     float2* scrA = nullptr;
     int nrmax = 0;
-    int zblk = 0;               // frame blocks of the dense column kernels (launch.h col_frames), 0: not served
+    int frame_rows = 0;         // of the dense column kernels (launch.h col_frame_rows), 0: not served
+    float2* col_tab = nullptr;  // their phased twiddles (ny = 512, 1024, 2048)
     int bchunk = 1;             // right-hand sides the plan's scratch holds
     // autotuned choices (pce_plan_autotune); untuned plans: run_chunk 0 (all the scratch holds),
     // column variant 2 where separable kernels exist, row variant 1
@@ -137,7 +138,7 @@ struct pce_plan {
                         items,  kptr,  klist,  scrZ, scrA,  wbox16, hh16,     hN16, hhT16, hscale,
                         twN,    hh4,   wrow, wxbox, d_vbox, d_kslot, d_korder, sitems, skptr, sklist,
                         hN2,    hN2_16, tw2048l, d_geo_f, d_geo_a, sec_items_box, sec_items_win, hsT, hsN,
-                        sec_twc, scrZs, scrAs, hsT16, hsN16, sec_hscale, d_kq0, hhTr, hNr, d_slot_toff};
+                        sec_twc, scrZs, scrAs, hsT16, hsN16, sec_hscale, d_kq0, hhTr, hNr, d_slot_toff, col_tab};
         for (void* q : ptrs)
             if (q) cudaFree(q);
     }

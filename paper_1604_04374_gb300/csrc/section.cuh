@@ -125,10 +125,10 @@ k_sec_r2c(const float* __restrict__ src, long long src_bstride, int NYg, int NXg
 // start, and serves every right-hand side (several sections of a term read
 // the same columns, so per-right-hand-side copies multiplied the traffic);
 // the one wait for it is bounded (status bit kStatusTimeout, products skipped
-// after it).  Shared memory: the staging tile, whose four quarters double as
-// the warps' transpose tiles, and the spectrum buffers (64 KB, three CTAs per
-// SM at up to 168 registers).
-constexpr int kSecColSmem = kSecLR * kWColWarps * 8 + kWColWarps * kSecLR * 8;
+// after it).  Shared memory: the warps' transpose tiles, whose space doubles
+// as the staging tile, and the spectrum buffers (65 KB, three CTAs per SM at up
+// to 168 registers).
+constexpr int kSecColSmem = kWColWarps * (fft_tile<kSecLR>() + kSecLR) * 8;
 template <bool CONJ, typename HT = float2>
 __global__ void __launch_bounds__(kWColWarps * 32, 3)
 kw_sec_cols(const float2* __restrict__ Z, long long z_bstride, long long z_kstride, int nb,
@@ -140,7 +140,7 @@ kw_sec_cols(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     extern __shared__ float2 smem[];
     float2* tile = smem;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2* tr = smem + warp * kWarpN;   // a quarter of the staging tile
+    float2* tr = smem + warp * fft_tile<kWarpN>();   // over the staging tile
     const int sec = blockIdx.x;   // section; its term is g.k
     const int col0 = blockIdx.y * kWColWarps;
     const int col = col0 + warp;
@@ -159,7 +159,7 @@ kw_sec_cols(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     const HT* hn = hsN + (long long)k * NY;
     const float sk = hscale_of<HT>(hscale, k);
     const int swl = tix_sw(lane, warp);
-    HT* hb = reinterpret_cast<HT*>(smem + NY * kWColWarps) + warp * NY;
+    HT* hb = reinterpret_cast<HT*>(smem + kWColWarps * fft_tile<NY>()) + warp * NY;
     const bool bulk = !dcn && cv;
     if (bulk && lane == 0) bulk_load(hb, hcol, NY * sizeof(HT), bar, skip_copy);
     for (int b = 0; b < nb; ++b) {

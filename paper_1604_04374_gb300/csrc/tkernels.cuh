@@ -57,7 +57,7 @@ constexpr int kTmCols = kt_tm_cols<1024>();
 constexpr bool kTmSplit = false;
 // four transpose tiles and two row-factor buffers
 template <int NY>
-__host__ __device__ constexpr int kt_smem_used() { return (kWColWarps * NY) * (int)sizeof(float2) + 2 * NY * (int)sizeof(float); }
+__host__ __device__ constexpr int kt_smem_used() { return kWColWarps * fft_tile<NY>() * (int)sizeof(float2) + 2 * NY * (int)sizeof(float); }
 // padded so that no more CTAs fit on an SM than its 512 tensor-memory columns
 // serve (then every resident CTA's allocation is satisfied at once):
 // 1024 points: 5 x (47 KB + the 1 KB per-CTA reserve) exceeds the SM's 228 KB,
@@ -171,8 +171,8 @@ kt_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     extern __shared__ __align__(16) float2 smem[];
     float2* tile = smem;                                     // staging tile [1024][4] (swizzled)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2* tr = smem + warp * NY;                       // this warp's transpose tile
-    float* wys = reinterpret_cast<float*>(smem + NY * kWColWarps);
+    float2* tr = smem + warp * fft_tile<NY>();            // this warp's transpose tile
+    float* wys = reinterpret_cast<float*>(smem + kWColWarps * fft_tile<NY>());
     __shared__ unsigned long long bars[kWColWarps];
     __shared__ unsigned tm_slot;
     const int b = blockIdx.x;
@@ -336,8 +336,8 @@ kt_cols_adj(float2* __restrict__ V, long long v_bstride, const float2* __restric
     extern __shared__ __align__(16) float2 smem[];
     float2* tile = smem;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2* tr = smem + warp * NY;
-    float* wys = reinterpret_cast<float*>(smem + NY * kWColWarps);
+    float2* tr = smem + warp * fft_tile<NY>();
+    float* wys = reinterpret_cast<float*>(smem + kWColWarps * fft_tile<NY>());
     __shared__ unsigned long long bars[kWColWarps];
     __shared__ unsigned tm_slot;
     const int b = blockIdx.x;

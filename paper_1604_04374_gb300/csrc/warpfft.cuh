@@ -6,9 +6,12 @@
 // so the FFT is
 //   1. a 32-point DFT over q in each lane's registers,
 //   2. the twiddles W1024^{l p} (table, FP32 rounded from FP64),
-//   3. a transpose of the 32 x 32 block through a warp-private shared tile
-//      (XOR-swizzled: element (l, p) at l*32 + (p ^ l), conflict-free both
-//      for the column writes and the row reads of a half-warp),
+//   3. a transpose of the 32 x 32 block through a warp-private shared tile,
+//      conflict-free both for the column writes and the row reads of a half-warp:
+//      element (l, p) at 32 l + (p ^ l), or with PAD at 33 l + p, where every address
+//      is a lane's base plus a constant, in a tile of warp_tile(1024) values (2048^2
+//      dense columns 2286 -> 2239 us an apply; but 493 -> 504 us in the separable and
+//      932 -> 1006 us in the sectioned kernels, which keep the smaller tile),
 //   4. a 32-point DFT over l in each lane.
 // On exit lane p holds v[m] = X[p + 32 m]: the same layout as on entry, so a
 // forward FFT, a pointwise product and an inverse FFT chain in registers.
@@ -122,6 +125,12 @@ __device__ __forceinline__ void dft32(float2 (&a)[32]) {
     for (int i = 0; i < (OUT_HALF ? 16 : 32); ++i) a[i] = out[i];
 }
 
+// float2 of a warp's padded transpose tile for an FFT of n points (rows of 33 or 17)
+__host__ __device__ constexpr int warp_tile(int n) { return n + 32; }
+// and of the tile of warp_fft<N> without PAD (512 points are always padded)
+template <int N>
+__host__ __device__ constexpr int fft_tile() { return N == 512 ? warp_tile(N) : N; }
+
 // Twiddle table of the four-step 1024-point FFT: tw[p * 32 + l] = W1024^{l p}.
 constexpr int kWarpTwLen = 1024;
 
@@ -129,8 +138,8 @@ struct NoHook {
     __device__ __forceinline__ void operator()() const {}
 };
 
-// One-warp 1024-point FFT (see the file comment).  tile: 1024 float2 of
-// shared memory private to the calling warp.  All 32 lanes must call it.
+// One-warp 1024-point FFT (see the file comment).  tile:
+// 1024 (PAD: warp_tile(1024)) float2 of shared memory private to the calling warp.  All 32 lanes must call it.
 // hook() runs once the transpose has been read back, i.e. when the tile is
 // free again (it may start an asynchronous copy into the tile).
 // SPLIT: the twiddles W1024^{l p} come from ten table loads and products (fewer
@@ -139,7 +148,10 @@ struct NoHook {
 // IN_HALF: the inputs x[l + 32 q] with q >= 16 are zero (v[16..31] not read).
 // OUT_HALF: only the outputs X[p + 32 m] with m < 16 are computed (v[16..31]
 // undefined on exit).
-template <bool INV, bool SPLIT = true, typename Hook = NoHook, bool IN_HALF = false, bool OUT_HALF = false>
+// PHASED: the table's row p = 0 is not 1 (a phase is folded into the table; not
+// with SPLIT).
+template <bool INV, bool SPLIT = true, typename Hook = NoHook, bool IN_HALF = false, bool OUT_HALF = false,
+          bool PHASED = false, bool PAD = false>
 __device__ __forceinline__ void warp_fft1024(float2 (&v)[32], float2* tile, const float2* __restrict__ tw,
                                              Hook hook = Hook()) {
     const int lane = threadIdx.x & 31;
@@ -163,17 +175,17 @@ __device__ __forceinline__ void warp_fft1024(float2 (&v)[32], float2* tile, cons
         }
     } else {
 #pragma unroll
-        for (int p = 1; p < 32; ++p) {
+        for (int p = PHASED ? 0 : 1; p < 32; ++p) {
             const float2 t = __ldg(&tw[p * 32 + lane]);
             v[p] = INV ? cmulc(v[p], t) : cmul(v[p], t);
         }
     }
     __syncwarp();
 #pragma unroll
-    for (int p = 0; p < 32; ++p) tile[lane * 32 + (p ^ lane)] = v[p];
+    for (int p = 0; p < 32; ++p) tile[PAD ? lane * 33 + p : lane * 32 + (p ^ lane)] = v[p];
     __syncwarp();
 #pragma unroll
-    for (int l = 0; l < 32; ++l) v[l] = tile[l * 32 + (lane ^ l)];
+    for (int l = 0; l < 32; ++l) v[l] = tile[PAD ? l * 33 + lane : l * 32 + (lane ^ l)];
     __syncwarp();
     hook();
     dft32<INV, false, OUT_HALF>(v);
@@ -181,12 +193,24 @@ __device__ __forceinline__ void warp_fft1024(float2 (&v)[32], float2* tile, cons
 
 // In-register 16-point DFT, natural order in and out: n = 4 n1 + n2,
 // k = k1 + 4 k2, X[k1 + 4 k2] = sum_n2 W4^{n2 k2} W16^{n2 k1} sum_n1 x[4 n1 + n2] W4^{n1 k1}.
-template <bool INV>
+// IN_HALF: x[8..15] are zero and are not read.  OUT_HALF: only X[0..7] are
+// computed; a[8..15] are left undefined.
+template <bool INV, bool IN_HALF = false, bool OUT_HALF = false>
 __device__ __forceinline__ void dft16(float2 (&a)[16]) {
 #pragma unroll
     for (int n2 = 0; n2 < 4; ++n2) {
-        float2 x[4] = {a[n2], a[4 + n2], a[8 + n2], a[12 + n2]};
-        Dft<4, INV>::run(x);
+        float2 x[4];
+        if constexpr (IN_HALF) {
+            const float2 r = mul_mi<INV>(a[4 + n2]);
+            x[0] = cadd(a[n2], a[4 + n2]);
+            x[1] = cadd(a[n2], r);
+            x[2] = csub(a[n2], a[4 + n2]);
+            x[3] = csub(a[n2], r);
+        } else {
+#pragma unroll
+            for (int n1 = 0; n1 < 4; ++n1) x[n1] = a[4 * n1 + n2];
+            Dft<4, INV>::run(x);
+        }
 #pragma unroll
         for (int k1 = 0; k1 < 4; ++k1) a[4 * k1 + n2] = tw32<INV>(x[k1], 2 * n2 * k1);   // W16 = W32^2
     }
@@ -194,12 +218,13 @@ __device__ __forceinline__ void dft16(float2 (&a)[16]) {
 #pragma unroll
     for (int k1 = 0; k1 < 4; ++k1) {
         float2 y[4] = {a[4 * k1], a[4 * k1 + 1], a[4 * k1 + 2], a[4 * k1 + 3]};
-        Dft<4, INV>::run(y);
+        if constexpr (OUT_HALF) dft4_first_two<INV>(y);
+        else Dft<4, INV>::run(y);
 #pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) out[k1 + 4 * k2] = y[k2];
+        for (int k2 = 0; k2 < (OUT_HALF ? 2 : 4); ++k2) out[k1 + 4 * k2] = y[k2];
     }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) a[i] = out[i];
+    for (int i = 0; i < (OUT_HALF ? 8 : 16); ++i) a[i] = out[i];
 }
 
 // One-warp 512-point FFT with the layout of warp_fft1024: lane l holds
@@ -208,19 +233,22 @@ __device__ __forceinline__ void dft16(float2 (&a)[16]) {
 //   X[p + 16 j] = sum_l W32^{l j} W512^{l p} sum_q x[l + 32 q] W16^{q p},
 //   1. a 16-point DFT over q in each lane's registers,
 //   2. the twiddles W512^{l p} = W1024^{2 l p} (the 1024-point table, rows 2p),
-//   3. the 32 x 16 block y[l][p] through a warp-private shared tile (the 16
-//      entries of row l XOR-swizzled by l & 15: conflict-free per half-warp),
+//   3. the 32 x 16 block y[l][p] through a warp-private shared tile (element (l, p)
+//      at 17 l + p: conflict-free per half-warp),
 //   4. the 32-point DFTs over l, one per p, split by decimation in frequency
 //      over the lane pair (p, p + 16): lane p + 16 s forms
 //      a_s[l'] = (y[l'][p] + (-1)^s y[l' + 16][p]) W32^{s l'} (l' < 16) from the
 //      tile and takes its 16-point DFT, which gives X[p + 16 (2 j' + s)]
 //      = X[lane + 32 j'] (j' < 16): the natural layout again.
-// tile: 512 float2 private to the warp.  Hook and SPLIT as for warp_fft1024.
-template <bool INV, bool SPLIT = true, typename Hook = NoHook>
+// tile: warp_tile(512) float2 private to the warp.  Hook, SPLIT, IN_HALF (x[l + 32 q],
+// q >= 8, zero) and OUT_HALF (m < 8 only) as for warp_fft1024.  PHASED: the twiddles
+// are the sixteen rows p of a table of their own instead of rows 2 p.
+template <bool INV, bool SPLIT = true, typename Hook = NoHook, bool IN_HALF = false, bool OUT_HALF = false,
+          bool PHASED = false>
 __device__ __forceinline__ void warp_fft512(float2 (&v)[16], float2* tile, const float2* __restrict__ tw,
                                             Hook hook = Hook()) {
     const int lane = threadIdx.x & 31;
-    dft16<INV>(v);
+    dft16<INV, IN_HALF>(v);
     __syncwarp();
     if constexpr (SPLIT) {
         // W512^{l p}, p = 8 a + b: W1024^{16 l a} W1024^{2 l b}
@@ -236,37 +264,45 @@ __device__ __forceinline__ void warp_fft512(float2 (&v)[16], float2* tile, const
         }
     } else {
 #pragma unroll
-        for (int p = 1; p < 16; ++p) {
-            const float2 t = __ldg(&tw[2 * p * 32 + lane]);
+        for (int p = PHASED ? 0 : 1; p < 16; ++p) {
+            const float2 t = __ldg(&tw[(PHASED ? p : 2 * p) * 32 + lane]);
             v[p] = INV ? cmulc(v[p], t) : cmul(v[p], t);
         }
     }
     __syncwarp();
 #pragma unroll
-    for (int p = 0; p < 16; ++p) tile[lane * 16 + (p ^ (lane & 15))] = v[p];
+    for (int p = 0; p < 16; ++p) tile[lane * 17 + p] = v[p];
     __syncwarp();
     const int p = lane & 15;
     const bool odd = lane >= 16;
     const float sg = odd ? -1.f : 1.f;
 #pragma unroll
     for (int l = 0; l < 16; ++l) {
-        const float2 y0 = tile[l * 16 + (p ^ l)];
-        const float2 y1 = tile[(l + 16) * 16 + (p ^ l)];
+        const float2 y0 = tile[l * 17 + p];
+        const float2 y1 = tile[(l + 16) * 17 + p];
         float2 a = make_float2(fmaf(sg, y1.x, y0.x), fmaf(sg, y1.y, y0.y));
         if (l > 0 && odd) a = tw32<INV>(a, l);
         v[l] = a;
     }
     __syncwarp();
     hook();
-    dft16<INV>(v);
+    dft16<INV, false, OUT_HALF>(v);
+}
+
+// The one-warp FFT of NF points on a phased table, NF / 32 values per lane.
+template <int NF, bool INV, bool IN_HALF, bool OUT_HALF, typename Hook = NoHook>
+__device__ __forceinline__ void warp_fft_phased(float2 (&v)[NF / 32], float2* tile, const float2* __restrict__ tw,
+                                                Hook hook = Hook()) {
+    if constexpr (NF == 1024) warp_fft1024<INV, false, Hook, IN_HALF, OUT_HALF, true, true>(v, tile, tw, hook);
+    else warp_fft512<INV, false, Hook, IN_HALF, OUT_HALF, true>(v, tile, tw, hook);
 }
 
 // One-warp FFT of NY = 512 or 1024 points (NY / 32 values per lane).
-template <int NY, bool INV, bool SPLIT = true, typename Hook = NoHook>
+template <int NY, bool INV, bool SPLIT = true, typename Hook = NoHook, bool PAD = false>
 __device__ __forceinline__ void warp_fft(float2 (&v)[NY / 32], float2* tile, const float2* __restrict__ tw,
                                          Hook hook = Hook()) {
     static_assert(NY == 512 || NY == 1024, "one-warp FFT of 512 or 1024 points");
-    if constexpr (NY == 1024) warp_fft1024<INV, SPLIT, Hook>(v, tile, tw, hook);
+    if constexpr (NY == 1024) warp_fft1024<INV, SPLIT, Hook, false, false, false, PAD>(v, tile, tw, hook);
     else warp_fft512<INV, SPLIT, Hook>(v, tile, tw, hook);
 }
 

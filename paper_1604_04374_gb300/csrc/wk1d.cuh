@@ -30,7 +30,7 @@ kw_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w, const HT* __res
           const float* __restrict__ hscale, int m, float* __restrict__ y, float scale,
           const float2* __restrict__ tw, int cl) {
     constexpr int N = kWarpN, Nh = N / 2;
-    __shared__ __align__(16) float2 tiles[kW1dWarps][N];
+    __shared__ __align__(16) float2 tiles[kW1dWarps][fft_tile<N>()];
     __shared__ __align__(16) float2 hsum[Nh];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float2* tr = tiles[warp];
@@ -135,7 +135,7 @@ kw_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w, const HT* __r
           const float* __restrict__ hscale, int m, float* __restrict__ x, float scale,
           const float2* __restrict__ tw, int cl) {
     constexpr int N = kWarpN, Nh = N / 2;
-    __shared__ __align__(16) float2 tiles[kW1dWarps][N];
+    __shared__ __align__(16) float2 tiles[kW1dWarps][fft_tile<N>()];
     __shared__ float red[N];   // this CTA's sums (clusters)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float2* tr = tiles[warp];

@@ -28,7 +28,7 @@ constexpr int kWColWarps = 4;          // columns per CTA of the column kernels
 // windows)
 template <int NY>
 constexpr int kw_col_smem() {
-    return (NY * kWColWarps + kWColWarps * NY) * (int)sizeof(float2) + 2 * NY * (int)sizeof(float);
+    return (NY * kWColWarps + kWColWarps * fft_tile<NY>()) * (int)sizeof(float2) + 2 * NY * (int)sizeof(float);
 }
 constexpr int kWColSmem = kw_col_smem<kWarpN>();
 // resident CTAs per SM the column kernels are compiled for: 3 at 1024 points
@@ -144,7 +144,7 @@ kw_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     extern __shared__ float2 smem[];
     float2* tile = smem;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2* tr = smem + NY * kWColWarps + warp * NY;
+    float2* tr = smem + NY * kWColWarps + warp * fft_tile<NY>();
     const int b = blockIdx.x;
     const int col0 = blockIdx.y * kWColWarps;
     const int col = col0 + warp;
@@ -173,7 +173,7 @@ kw_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     auto kof = [&](int t) { return SEP ? __ldg(&sep.korder[t]) : t; };
     auto slot_of = [&](int kk) { return SEP ? __ldg(&sep.kslot[kk]) : kk; };
     // SEP: row factors of term t in buffer (t & 1), prefetched one term ahead
-    float* wys = reinterpret_cast<float*>(smem + 2 * NY * kWColWarps);
+    float* wys = reinterpret_cast<float*>(smem + (NY + fft_tile<NY>()) * kWColWarps);
     int t = next_t(0);
     int cur_slot = -1;
     if (t < tend) {
@@ -308,7 +308,7 @@ kw_cols_adj(const float2* __restrict__ V, long long v_bstride,
     extern __shared__ float2 smem[];
     float2* tile = smem;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float2* tr = smem + NY * kWColWarps + warp * NY;
+    float2* tr = smem + NY * kWColWarps + warp * fft_tile<NY>();
     const int b = blockIdx.x;
     const int col0 = blockIdx.y * kWColWarps;
     const int col = col0 + warp;
@@ -339,7 +339,7 @@ kw_cols_adj(const float2* __restrict__ V, long long v_bstride,
     auto slot_of = [&](int kk) { return SEP ? __ldg(&sep.kslot[kk]) : kk; };
 
     // SEP: row factors of the t-th term in buffer (t & 1), prefetched one term ahead
-    float* wys = reinterpret_cast<float*>(smem + 2 * NY * kWColWarps);
+    float* wys = reinterpret_cast<float*>(smem + (NY + fft_tile<NY>()) * kWColWarps);
     if constexpr (SEP) {
         if (tbeg < tend) wy_load<NY>(wys + (tbeg & 1) * NY, sep.wrow, __ldg(&sep.korder[tbeg]));
     }

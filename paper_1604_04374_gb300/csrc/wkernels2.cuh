@@ -15,7 +15,7 @@ namespace pce {
 
 constexpr int kW2N = 2048;
 constexpr int kW2Cols = 2;   // columns per CTA
-constexpr int kW2Smem = (kW2N * kW2Cols + 4 * kWarpN) * (int)sizeof(float2);
+constexpr int kW2Smem = (kW2N * kW2Cols + 4 * fft_tile<kWarpN>()) * (int)sizeof(float2);
 
 __device__ __forceinline__ int tix2(int row, int c) { return 2 * row + (c ^ ((row >> 3) & 1)); }
 
@@ -62,7 +62,7 @@ kw2_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstr
     float2* tile = smem;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int par = warp & 1, cl = warp >> 1;
-    float2* tr = smem + NY * kW2Cols + warp * kWarpN;
+    float2* tr = smem + NY * kW2Cols + warp * fft_tile<kWarpN>();
     const int b = blockIdx.x;
     const int col0 = blockIdx.y * kW2Cols;
     const int col = col0 + cl;

@@ -54,7 +54,7 @@ kw_rows_r2c(const float* __restrict__ src, long long src_bstride, int nrows, flo
             long long dst_bstride, const float2* __restrict__ tw) {
     constexpr int NXh = NX / 2;
     constexpr int QN = NX / 32;
-    __shared__ __align__(16) float2 trs[kWRowWarps][NX];
+    __shared__ __align__(16) float2 trs[kWRowWarps][fft_tile<NX>()];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int p = blockIdx.x * kWRowWarps + warp;
     const int npairs = (nrows + 1) / 2;
@@ -106,7 +106,7 @@ kw_rows_c2r(const float2* __restrict__ src, long long src_bstride, int nrows, fl
             long long dst_bstride, float scale, const float2* __restrict__ tw) {
     constexpr int NXh = NX / 2;
     constexpr int QN = NX / 32;
-    __shared__ __align__(16) float2 trs[kWRowWarps][NX];
+    __shared__ __align__(16) float2 trs[kWRowWarps][fft_tile<NX>()];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int p = blockIdx.x * kWRowWarps + warp;
     const int npairs = (nrows + 1) / 2;
