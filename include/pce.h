@@ -223,8 +223,13 @@ pce_status pce_plan_info(pce_plan_t plan, int* m_out, int* box_out, int64_t* scr
  */
 pce_status pce_plan_hhat(pce_plan_t plan, float* hhat, void* stream);
 
-/* pce_plan_destroy -- free the plan and all its device memory (synchronises the device). */
+/*
+ * pce_plan_destroy -- free the plan and all its device memory (synchronises the device).
+ * The library keeps up to 2 GiB of freed plan memory per device for later plans;
+ * pce_release_memory synchronises and returns what no plan uses to the device.
+ */
 pce_status pce_plan_destroy(pce_plan_t plan);
+pce_status pce_release_memory(void);
 
 /* Message of the last failing call on this thread ("" if none). */
 const char* pce_last_error_string(void);

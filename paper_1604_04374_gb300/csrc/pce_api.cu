@@ -39,6 +39,90 @@ pce_status fail(pce_status s, const char* fmt, ...) {
     return s;
 }
 
+// Plan memory comes from one stream-ordered pool a device.  A training step that makes
+// a plan of new windows every time (autograd.py) otherwise spent more time in cudaMalloc
+// and cudaFree of the plan's arrays than in its kernels: 512^2, m = 16, 16 right-hand
+// sides 2313 -> 1189 us a step.  Between plans the pool keeps at most kPoolKeep bytes;
+// pce_release_memory gives those back too.  The pool serves any thread and stream.
+namespace {
+
+constexpr unsigned long long kPoolKeep = 2ull << 30;
+constexpr int kMaxDevices = 64;
+std::mutex g_mem_mutex;
+cudaMemPool_t g_mem_pool[kMaxDevices] = {};
+bool g_mem_asked[kMaxDevices] = {};
+
+// The device's pool, made at the first call; null where pools are not supported.
+cudaMemPool_t mem_pool(int dev) {
+    if (dev < 0 || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lock(g_mem_mutex);
+    if (!g_mem_asked[dev]) {
+        g_mem_asked[dev] = true;
+        int ok = 0;
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        unsigned long long keep = kPoolKeep;
+        cudaMemPool_t pool = nullptr;
+        if (cudaDeviceGetAttribute(&ok, cudaDevAttrMemoryPoolsSupported, dev) == cudaSuccess && ok &&
+            cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
+            if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+                g_mem_pool[dev] = pool;
+            else
+                cudaMemPoolDestroy(pool);
+        }
+        cudaGetLastError();
+    }
+    return g_mem_pool[dev];
+}
+
+cudaMemPool_t current_pool() {
+    int dev = 0;
+    return cudaGetDevice(&dev) == cudaSuccess ? mem_pool(dev) : nullptr;
+}
+
+}  // namespace
+
+cudaError_t mem_alloc(void** p, size_t bytes, cudaStream_t s) {
+    cudaMemPool_t pool = current_pool();
+    if (!pool) return cudaMalloc(p, bytes);
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    }
+    return e;
+}
+
+void mem_free(void* p, cudaStream_t s) {
+    if (!p) return;
+    if (current_pool()) cudaFreeAsync(p, s);
+    else cudaFree(p);
+}
+
+cudaError_t mem_release() {
+    int cur = 0;
+    cudaError_t e = cudaGetDevice(&cur);
+    if (e != cudaSuccess) return e;
+    for (int d = 0; d < kMaxDevices && e == cudaSuccess; ++d) {
+        cudaMemPool_t pool;
+        {
+            std::lock_guard<std::mutex> lock(g_mem_mutex);
+            pool = g_mem_pool[d];
+        }
+        if (!pool) continue;
+        // only memory whose stream-ordered frees have run can go back
+        e = cudaSetDevice(d);
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        if (e == cudaSuccess) e = cudaMemPoolTrimTo(pool, 0);
+    }
+    const cudaError_t back = cudaSetDevice(cur);
+    return e != cudaSuccess ? e : back;
+}
+
 bool is_device_ptr(const void* p) {
     if (!p) return false;
     cudaPointerAttributes a;
@@ -265,8 +349,10 @@ __global__ void k_support(const float* __restrict__ w, int m, int ny, int nx,
     }
 }
 
-// Box copy of w_k: wbox[woff + i*ldw + cc] = w_k[(r0+i) % ny][(c0+cc) % nx] (0 beyond nc).
-__global__ void k_wbox(const float* __restrict__ w, int ny, int nx, Box bx, float* wbox) {
+// Box copies, term blockIdx.y: wbox[woff + i*ldw + cc] = w_k[(r0+i) % ny][(c0+cc) % nx] (0 beyond nc).
+__global__ void k_wbox(const float* __restrict__ w0, int ny, int nx, const Box* __restrict__ box, float* wbox) {
+    const Box bx = box[blockIdx.y];
+    const float* w = w0 + (size_t)blockIdx.y * ny * nx;
     const long long total = (long long)bx.nr * bx.ldw;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
@@ -469,11 +555,12 @@ void cyclic_support(const unsigned char* f, int n, int& start, int& len) {
     len = n - best;
 }
 
+// count elements of device memory for use after s's current work (pce_rt::mem_alloc)
 template <class T>
-pce_status dev_alloc(T** p, size_t count) {
+pce_status dev_alloc(T** p, size_t count, cudaStream_t s) {
     *p = nullptr;
     if (count == 0) return PCE_OK;
-    PCE_CK(cudaMalloc(reinterpret_cast<void**>(p), count * sizeof(T)));
+    PCE_CK(pce_rt::mem_alloc(reinterpret_cast<void**>(p), count * sizeof(T), s));
     return PCE_OK;
 }
 
@@ -508,17 +595,17 @@ pce_status validate_shape(int ndims, const int64_t* shape, int& ny, int& nx) {
 
 pce_status make_twiddles_l1(pce_plan* p, cudaStream_t s) {
     const long long N = p->nx;
-    pce_status st = dev_alloc(&p->twN, (size_t)N);
+    pce_status st = dev_alloc(&p->twN, (size_t)N, s);
     if (st) return st;
     k_twiddles_N<<<grid_for(N), 256, 0, s>>>(p->twN, N);
     PCE_CK(cudaGetLastError());
-    if ((st = dev_alloc(&p->twx, (size_t)twiddle_len(p->l1nx)))) return st;
+    if ((st = dev_alloc(&p->twx, (size_t)twiddle_len(p->l1nx), s))) return st;
     k_twiddles<<<grid_for(twiddle_len(p->l1nx)), 256, 0, s>>>(p->twx, p->l1nx);
     PCE_CK(cudaGetLastError());
     if (p->l1ny == p->l1nx) {
         p->twy = p->twx;
     } else {
-        if ((st = dev_alloc(&p->twy, (size_t)twiddle_len(p->l1ny)))) return st;
+        if ((st = dev_alloc(&p->twy, (size_t)twiddle_len(p->l1ny), s))) return st;
         k_twiddles<<<grid_for(twiddle_len(p->l1ny)), 256, 0, s>>>(p->twy, p->l1ny);
         PCE_CK(cudaGetLastError());
     }
@@ -531,7 +618,7 @@ pce_status make_twiddles(pce_plan* p, cudaStream_t s) {
     // 1024, columns of 2048 (two warps per column), rows and columns of 512
     // (rows 2p of it)
     if (p->nx == 1024 || (p->ndims == 2 && (p->nx == 512 || p->ny == 512 || p->ny == 1024 || p->ny == 2048))) {
-        pce_status st0 = dev_alloc(&p->tw1024, 1024);
+        pce_status st0 = dev_alloc(&p->tw1024, 1024, s);
         if (st0) return st0;
         k_twiddles_1024<<<4, 256, 0, s>>>(p->tw1024);
         PCE_CK(cudaGetLastError());
@@ -539,13 +626,13 @@ pce_status make_twiddles(pce_plan* p, cudaStream_t s) {
     pce_status st;
     if (p->ndims == 2) {
         const long long n = pce::col_table_size(p->ny);
-        if ((st = dev_alloc(&p->col_tab, (size_t)n))) return st;
+        if ((st = dev_alloc(&p->col_tab, (size_t)n, s))) return st;
         if (n > 0) {
             k_col_tables<<<grid_for(n), 256, 0, s>>>(p->col_tab, p->ny == 512 ? 512 : 1024, p->ny == 2048 ? 2 : 1);
             PCE_CK(cudaGetLastError());
         }
     }
-    st = dev_alloc(&p->twx, (size_t)std::max(1, twiddle_len(p->nx)));
+    st = dev_alloc(&p->twx, (size_t)std::max(1, twiddle_len(p->nx)), s);
     if (st) return st;
     k_twiddles<<<grid_for(twiddle_len(p->nx)), 256, 0, s>>>(p->twx, p->nx);
     PCE_CK(cudaGetLastError());
@@ -553,7 +640,7 @@ pce_status make_twiddles(pce_plan* p, cudaStream_t s) {
         if (p->ny == p->nx) {
             p->twy = p->twx;
         } else {
-            st = dev_alloc(&p->twy, (size_t)std::max(1, twiddle_len(p->ny)));
+            st = dev_alloc(&p->twy, (size_t)std::max(1, twiddle_len(p->ny)), s);
             if (st) return st;
             k_twiddles<<<grid_for(twiddle_len(p->ny)), 256, 0, s>>>(p->twy, p->ny);
             PCE_CK(cudaGetLastError());
@@ -566,7 +653,7 @@ pce_status make_twiddles(pce_plan* p, cudaStream_t s) {
 pce_status setup_windows(pce_plan* p, const float* w, cudaStream_t s) {
     const int m = p->m, ny = p->ny, nx = p->nx;
     if (p->ndims == 1) {
-        pce_status st = dev_alloc(&p->wbox, (size_t)m * nx);
+        pce_status st = dev_alloc(&p->wbox, (size_t)m * nx, s);
         if (st) return st;
         PCE_CK(cudaMemcpyAsync(p->wbox, w, sizeof(float) * m * nx, cudaMemcpyDeviceToDevice, s));
         p->box.assign(m, Box{0, 1, 0, nx, 0, nx, 0});
@@ -574,7 +661,7 @@ pce_status setup_windows(pce_plan* p, const float* w, cudaStream_t s) {
     }
     unsigned char* flags = nullptr;
     const size_t nflags = (size_t)m * (ny + nx);
-    PCE_CK(cudaMalloc(&flags, nflags));
+    PCE_CK(pce_rt::mem_alloc(reinterpret_cast<void**>(&flags), nflags, s));
     cudaError_t e = cudaMemsetAsync(flags, 0, nflags, s);
     if (e == cudaSuccess) {
         k_support<<<grid_for((long long)m * ny * nx), 256, 0, s>>>(w, m, ny, nx, flags,
@@ -584,7 +671,7 @@ pce_status setup_windows(pce_plan* p, const float* w, cudaStream_t s) {
     std::vector<unsigned char> hf(nflags);
     if (e == cudaSuccess) e = cudaMemcpyAsync(hf.data(), flags, nflags, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(flags);
+    pce_rt::mem_free(flags, s);
     PCE_CK(e);
 
     p->box.resize(m);
@@ -601,16 +688,8 @@ pce_status setup_windows(pce_plan* p, const float* w, cudaStream_t s) {
         p->nrmax = std::max(p->nrmax, b.nr);
     }
     p->frame_rows = pce::col_frame_rows(ny, p->box.data(), m);
-    pce_status st = dev_alloc(&p->wbox, (size_t)std::max<long long>(woff, 4));
+    pce_status st = dev_alloc(&p->wbox, (size_t)std::max<long long>(woff, 4), s);
     if (st) return st;
-    for (int k = 0; k < m; ++k) {
-        const Box& b = p->box[k];
-        if (b.nr == 0) continue;
-        k_wbox<<<grid_for((long long)b.nr * b.ldw), 256, 0, s>>>(w + (size_t)k * ny * nx, ny, nx, b,
-                                                                 p->wbox);
-        PCE_CK(cudaGetLastError());
-    }
-
     // F1 items: (k, row pair inside the box)
     std::vector<int2> items;
     for (int k = 0; k < m; ++k)
@@ -633,11 +712,20 @@ pce_status setup_windows(pce_plan* p, const float* w, cudaStream_t s) {
         }
         kptr[q + 1] = (int)klist.size();
     }
-    if ((st = dev_alloc(&p->d_box, (size_t)m))) return st;
-    if ((st = dev_alloc(&p->items, std::max<size_t>(items.size(), 1)))) return st;
-    if ((st = dev_alloc(&p->kptr, kptr.size()))) return st;
-    if ((st = dev_alloc(&p->klist, std::max<size_t>(klist.size(), 1)))) return st;
+    if ((st = dev_alloc(&p->d_box, (size_t)m, s))) return st;
+    if ((st = dev_alloc(&p->items, std::max<size_t>(items.size(), 1), s))) return st;
+    if ((st = dev_alloc(&p->kptr, kptr.size(), s))) return st;
+    if ((st = dev_alloc(&p->klist, std::max<size_t>(klist.size(), 1), s))) return st;
     PCE_CK(cudaMemcpyAsync(p->d_box, p->box.data(), sizeof(Box) * m, cudaMemcpyHostToDevice, s));
+    {
+        long long most = 0;
+        for (const Box& b : p->box) most = std::max(most, (long long)b.nr * b.ldw);
+        for (int k0 = 0; k0 < m && most > 0; k0 += 65535) {   // grid.y limit
+            k_wbox<<<dim3(grid_for(most), std::min(m - k0, 65535)), 256, 0, s>>>(w + (size_t)k0 * ny * nx, ny, nx,
+                                                                              p->d_box + k0, p->wbox);
+            PCE_CK(cudaGetLastError());
+        }
+    }
     if (!items.empty())
         PCE_CK(cudaMemcpyAsync(p->items, items.data(), sizeof(int2) * items.size(),
                                cudaMemcpyHostToDevice, s));
@@ -659,8 +747,8 @@ pce_status setup_windows(pce_plan* p, const float* w, cudaStream_t s) {
     p->zalloc = zalloc;
     const long long per_b = (zalloc + ab) * (long long)sizeof(float2);
     p->bchunk = (int)std::max<long long>(1, std::min<long long>(kMaxChunk, kScratchBudget / per_b));
-    if ((st = dev_alloc(&p->scrZ, (size_t)std::max<long long>(1, zalloc * p->bchunk)))) return st;
-    if ((st = dev_alloc(&p->scrA, (size_t)(ab * p->bchunk)))) return st;
+    if ((st = dev_alloc(&p->scrZ, (size_t)std::max<long long>(1, zalloc * p->bchunk), s))) return st;
+    if ((st = dev_alloc(&p->scrA, (size_t)(ab * p->bchunk), s))) return st;
     p->scratch_bytes = per_b * p->bchunk;
     return PCE_OK;
 }
@@ -672,7 +760,7 @@ pce_status term_scales(const float2* a, long long per, const float2* b, long lon
                        float** sc_dev) {
     unsigned* mx = nullptr;
     pce_status st;
-    if ((st = dev_alloc(&mx, (size_t)m))) return st;
+    if ((st = dev_alloc(&mx, (size_t)m, s))) return st;
     cudaError_t e = cudaMemsetAsync(mx, 0, sizeof(unsigned) * m, s);
     if (e == cudaSuccess) {
         k_term_maxabs<<<grid_for(per * m), 256, 0, s>>>(a, per, m, mx);
@@ -682,7 +770,7 @@ pce_status term_scales(const float2* a, long long per, const float2* b, long lon
     std::vector<unsigned> hmx(m);
     if (e == cudaSuccess) e = cudaMemcpyAsync(hmx.data(), mx, sizeof(unsigned) * m, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(mx);
+    pce_rt::mem_free(mx, s);
     PCE_CK(e);
     std::vector<float> sc(m);
     for (int k = 0; k < m; ++k) {
@@ -692,7 +780,7 @@ pce_status term_scales(const float2* a, long long per, const float2* b, long lon
         const float fr = std::frexp(v, &ex);   // v = fr * 2^ex, fr in [0.5, 1)
         sc[k] = (v > 0.f && std::isfinite(v)) ? std::ldexp(1.0f, fr == 0.5f ? ex - 1 : ex) : 1.0f;
     }
-    if ((st = dev_alloc(sc_dev, (size_t)m))) return st;
+    if ((st = dev_alloc(sc_dev, (size_t)m, s))) return st;
     PCE_CK(cudaMemcpyAsync(*sc_dev, sc.data(), sizeof(float) * m, cudaMemcpyHostToDevice, s));
     PCE_CK(cudaStreamSynchronize(s));   // sc must outlive the copy
     return PCE_OK;
@@ -708,26 +796,26 @@ pce_status quantize_plan(pce_plan* p, cudaStream_t s) {
     pce_status st;
     if ((st = term_scales(p->hh, per, two_d ? p->hN : nullptr, ny, m, s, &p->hscale))) return st;
     __half2* h16 = nullptr;
-    if ((st = dev_alloc(&h16, (size_t)(per * m)))) return st;
+    if ((st = dev_alloc(&h16, (size_t)(per * m), s))) return st;
     p->hh16 = h16;
     k_quantize_h<<<grid_for(per * m), 256, 0, s>>>(p->hh, per, m, p->hscale, h16);
     PCE_CK(cudaGetLastError());
     if (two_d) {
         __half2* n16 = nullptr;
-        if ((st = dev_alloc(&n16, (size_t)ny * m))) return st;
+        if ((st = dev_alloc(&n16, (size_t)ny * m, s))) return st;
         p->hN16 = n16;
         k_quantize_h<<<grid_for((long long)ny * m), 256, 0, s>>>(p->hN, ny, m, p->hscale, n16);
         PCE_CK(cudaGetLastError());
         if (p->hN2) {
             __half2* n2 = nullptr;
-            if ((st = dev_alloc(&n2, (size_t)ny * m))) return st;
+            if ((st = dev_alloc(&n2, (size_t)ny * m, s))) return st;
             p->hN2_16 = n2;
             k_quantize_h<<<grid_for((long long)ny * m), 256, 0, s>>>(p->hN2, ny, m, p->hscale, n2);
             PCE_CK(cudaGetLastError());
         }
         if (p->hhT) {
             __half2* t16 = nullptr;
-            if ((st = dev_alloc(&t16, (size_t)(per * m)))) return st;
+            if ((st = dev_alloc(&t16, (size_t)(per * m), s))) return st;
             p->hhT16 = t16;
             k_quantize_h<<<grid_for(per * m), 256, 0, s>>>(p->hhT, per, m, p->hscale, t16);
             PCE_CK(cudaGetLastError());
@@ -740,7 +828,7 @@ pce_status quantize_plan(pce_plan* p, cudaStream_t s) {
         nw = (long long)m * p->nx;
     }
     __nv_bfloat16* w16 = nullptr;
-    if ((st = dev_alloc(&w16, (size_t)std::max<long long>(nw, 1)))) return st;
+    if ((st = dev_alloc(&w16, (size_t)std::max<long long>(nw, 1), s))) return st;
     p->wbox16 = w16;
     if (nw > 0) {
         k_quantize_w<<<grid_for(nw), 256, 0, s>>>(p->wbox, nw, w16);
@@ -809,7 +897,7 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
         p->l1nx = nx / p->l1ny;
     }
     if ((st = make_twiddles(p, s))) return bail(st);
-    if ((st = dev_alloc(&p->d_status, 1))) return bail(st);
+    if ((st = dev_alloc(&p->d_status, 1, s))) return bail(st);
     if (cudaMemsetAsync(p->d_status, 0, sizeof(int), s) != cudaSuccess)
         return bail(fail(PCE_ERR_CUDA, "status word initialisation failed"));
     if ((st = setup_windows(p, w, s))) return bail(st);
@@ -817,7 +905,7 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
     if (p->l1) {
         const int npairs = (m + 1) / 2;
         const long long N = nx;
-        if ((st = dev_alloc(&p->hh4, (size_t)(m * N)))) return bail(st);
+        if ((st = dev_alloc(&p->hh4, (size_t)(m * N), s))) return bail(st);
         if (spectra) {
             k_from_half_l1<<<grid_for(m * N), 256, 0, s>>>(reinterpret_cast<const float2*>(h), m, p->l1ny,
                                                           p->l1nx, p->hh4);
@@ -825,7 +913,7 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
             if (e) return bail(fail(PCE_ERR_CUDA, "spectrum conversion: %s", cudaGetErrorString(e)));
         } else {
             float2* G = nullptr;
-            if ((st = dev_alloc(&G, (size_t)(npairs * N)))) return bail(st);
+            if ((st = dev_alloc(&G, (size_t)(npairs * N), s))) return bail(st);
             const int cpc = pce::l1_cols_per_cta(p->l1ny);
             cudaError_t e = pce::launch_l1_cols(p->l1ny, 1 /*pair*/, dim3(npairs, 1, (p->l1nx + cpc - 1) / cpc), s,
                                                 h, 0, nullptr, m, p->l1nx, p->twN, G, p->twy);
@@ -834,18 +922,18 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
                 e = pce::launch_l1_rows_spec(p->l1nx, dim3((p->l1ny / 2 + 1 + it - 1) / it, npairs), s, G, npairs,
                                              m, p->l1ny, p->hh4, p->twx);
             cudaError_t e2 = cudaStreamSynchronize(s);
-            cudaFree(G);
+            pce_rt::mem_free(G, s);
             if (e == cudaSuccess) e = e2;
             if (e) return bail(fail(PCE_ERR_CUDA, "spectrum of h: %s", cudaGetErrorString(e)));
         }
         // scratch: per right-hand side npairs * N (G or Q) + N (A or V) complex
         const long long per_b = ((long long)npairs * N + N) * (long long)sizeof(float2);
         p->bchunk = (int)std::max<long long>(1, std::min<long long>(kMaxChunk, kScratchBudget / per_b));
-        if ((st = dev_alloc(&p->scrZ, (size_t)(npairs * N * p->bchunk)))) return bail(st);
-        if ((st = dev_alloc(&p->scrA, (size_t)(N * p->bchunk)))) return bail(st);
+        if ((st = dev_alloc(&p->scrZ, (size_t)(npairs * N * p->bchunk), s))) return bail(st);
+        if ((st = dev_alloc(&p->scrA, (size_t)(N * p->bchunk), s))) return bail(st);
         p->scratch_bytes = per_b * p->bchunk;
     } else if (ndims == 1) {
-        if ((st = dev_alloc(&p->hh, (size_t)m * nxh))) return bail(st);
+        if ((st = dev_alloc(&p->hh, (size_t)m * nxh, s))) return bail(st);
         if (spectra) {
             k_from_half1d<<<grid_for((long long)m * nxh), 256, 0, s>>>(
                 reinterpret_cast<const float2*>(h), m, nxh, p->hh);
@@ -856,8 +944,8 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
             if (e) return bail(fail(PCE_ERR_CUDA, "spectrum of h: %s", cudaGetErrorString(e)));
         }
     } else {
-        if ((st = dev_alloc(&p->hh, (size_t)m * ny * nxh))) return bail(st);
-        if ((st = dev_alloc(&p->hN, (size_t)m * ny))) return bail(st);
+        if ((st = dev_alloc(&p->hh, (size_t)m * ny * nxh, s))) return bail(st);
+        if ((st = dev_alloc(&p->hN, (size_t)m * ny, s))) return bail(st);
         if (spectra) {
             k_from_half2d<<<grid_for((long long)m * ny * (nxh + 1)), 256, 0, s>>>(
                 reinterpret_cast<const float2*>(h), m, ny, nxh, p->hh, p->hN);
@@ -866,7 +954,7 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
         } else {
             // hhat = column FFT of the row R2C spectra of h (rows of all m terms at once)
             float2* S = nullptr;
-            if ((st = dev_alloc(&S, (size_t)m * ny * nxh))) return bail(st);
+            if ((st = dev_alloc(&S, (size_t)m * ny * nxh, s))) return bail(st);
             const int fpc = pce::rows_pairs_per_cta(nx);
             const int npairs = (ny + 1) / 2;
             cudaError_t e = pce::launch_rows_r2c(nx, false, dim3(r2c_blocks(npairs, nx), m), s, h,
@@ -877,7 +965,7 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
                 e = pce::launch_cols_spec(ny, dim3(m, (nxh + cpc - 1) / cpc), s, S, nxh, p->hh, p->hN,
                                           p->twy);
             cudaError_t e2 = cudaStreamSynchronize(s);
-            cudaFree(S);
+            pce_rt::mem_free(S, s);
             if (e == cudaSuccess) e = e2;
             if (e) return bail(fail(PCE_ERR_CUDA, "spectrum of h: %s", cudaGetErrorString(e)));
         }
@@ -896,16 +984,16 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
         if (e1) return bail(fail(PCE_ERR_CUDA, "spectrum conjugation: %s", cudaGetErrorString(e1)));
     }
     if (ndims == 2 && (ny == 1024 || ny == 512)) {
-        if ((st = dev_alloc(&p->hhT, (size_t)m * ny * nxh))) return bail(st);
+        if ((st = dev_alloc(&p->hhT, (size_t)m * ny * nxh, s))) return bail(st);
         k_transpose_hh<<<grid_for((long long)m * ny * nxh), 256, 0, s>>>(p->hh, m, ny, nxh, p->hhT);
         cudaError_t e1 = cudaGetLastError();
         if (e1) return bail(fail(PCE_ERR_CUDA, "spectrum transpose: %s", cudaGetErrorString(e1)));
     }
     if (ndims == 2 && ny == 2048) {
         // spectra of each column split by frequency parity for the two-warp column FFT
-        if ((st = dev_alloc(&p->hhT, (size_t)m * ny * nxh))) return bail(st);
-        if ((st = dev_alloc(&p->hN2, (size_t)m * ny))) return bail(st);
-        if ((st = dev_alloc(&p->tw2048l, 32))) return bail(st);
+        if ((st = dev_alloc(&p->hhT, (size_t)m * ny * nxh, s))) return bail(st);
+        if ((st = dev_alloc(&p->hN2, (size_t)m * ny, s))) return bail(st);
+        if ((st = dev_alloc(&p->tw2048l, 32, s))) return bail(st);
         k_split_hh2<<<grid_for((long long)m * ny * nxh), 256, 0, s>>>(p->hh, p->hN, m, nxh, p->hhT, p->hN2);
         k_tw2048l<<<1, 32, 0, s>>>(p->tw2048l);
         cudaError_t e1 = cudaGetLastError();
@@ -1007,14 +1095,14 @@ pce_status setup_separable(pce_plan* p, const float* wy, const float* wx, cudaSt
         kptr[q + 1] = (int)klist.size();
     }
     pce_status st;
-    if ((st = dev_alloc(&p->wrow, hy.size()))) return st;
-    if ((st = dev_alloc(&p->wxbox, std::max<size_t>(wxb.size(), 4)))) return st;
-    if ((st = dev_alloc(&p->d_vbox, (size_t)ns))) return st;
-    if ((st = dev_alloc(&p->d_kslot, (size_t)m))) return st;
-    if ((st = dev_alloc(&p->d_korder, std::max<size_t>(korder.size(), 1)))) return st;
-    if ((st = dev_alloc(&p->sitems, std::max<size_t>(items.size(), 1)))) return st;
-    if ((st = dev_alloc(&p->skptr, kptr.size()))) return st;
-    if ((st = dev_alloc(&p->sklist, std::max<size_t>(klist.size(), 1)))) return st;
+    if ((st = dev_alloc(&p->wrow, hy.size(), s))) return st;
+    if ((st = dev_alloc(&p->wxbox, std::max<size_t>(wxb.size(), 4), s))) return st;
+    if ((st = dev_alloc(&p->d_vbox, (size_t)ns, s))) return st;
+    if ((st = dev_alloc(&p->d_kslot, (size_t)m, s))) return st;
+    if ((st = dev_alloc(&p->d_korder, std::max<size_t>(korder.size(), 1), s))) return st;
+    if ((st = dev_alloc(&p->sitems, std::max<size_t>(items.size(), 1), s))) return st;
+    if ((st = dev_alloc(&p->skptr, kptr.size(), s))) return st;
+    if ((st = dev_alloc(&p->sklist, std::max<size_t>(klist.size(), 1), s))) return st;
     PCE_CK(cudaMemcpyAsync(p->wrow, hy.data(), sizeof(float) * hy.size(), cudaMemcpyHostToDevice, s));
     if (!wxb.empty())
         PCE_CK(cudaMemcpyAsync(p->wxbox, wxb.data(), sizeof(float) * wxb.size(), cudaMemcpyHostToDevice, s));
@@ -1041,9 +1129,9 @@ pce_status setup_separable(pce_plan* p, const float* wy, const float* wx, cudaSt
         kq0[k] = r0 >> 5;
     }
     if (prune) {
-        if ((st = dev_alloc(&p->d_kq0, (size_t)m))) return st;
-        if ((st = dev_alloc(&p->hhTr, (size_t)m * nxh * ny))) return st;
-        if ((st = dev_alloc(&p->hNr, (size_t)m * ny))) return st;
+        if ((st = dev_alloc(&p->d_kq0, (size_t)m, s))) return st;
+        if ((st = dev_alloc(&p->hhTr, (size_t)m * nxh * ny, s))) return st;
+        if ((st = dev_alloc(&p->hNr, (size_t)m * ny, s))) return st;
         PCE_CK(cudaMemcpyAsync(p->d_kq0, kq0.data(), sizeof(int) * m, cudaMemcpyHostToDevice, s));
         k_rotate_cols<<<grid_for((long long)m * (nxh + 1) * ny), 256, 0, s>>>(p->hhT, p->hN, p->d_kq0, m,
                                                                             (int)nxh, p->hhTr, p->hNr);
@@ -1057,7 +1145,7 @@ pce_status setup_separable(pce_plan* p, const float* wy, const float* wx, cudaSt
         for (int k : korder) n += kslot[k] == j;
         p->slot_term_off[j + 1] = p->slot_term_off[j] + n;
     }
-    if ((st = dev_alloc(&p->d_slot_toff, (size_t)ns + 1))) return st;
+    if ((st = dev_alloc(&p->d_slot_toff, (size_t)ns + 1, s))) return st;
     PCE_CK(cudaMemcpyAsync(p->d_slot_toff, p->slot_term_off.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice, s));
     PCE_CK(cudaStreamSynchronize(s));   // the host vectors die at return
     p->nslots = ns;
@@ -1105,7 +1193,7 @@ pce_status setup_sectioned(pce_plan* p, const float* h, cudaStream_t s) {
     // exact support of every h_k (rows, columns)
     unsigned char* flags = nullptr;
     const size_t nflags = (size_t)m * (ny + nx);
-    PCE_CK(cudaMalloc(&flags, nflags));
+    PCE_CK(pce_rt::mem_alloc(reinterpret_cast<void**>(&flags), nflags, s));
     cudaError_t e = cudaMemsetAsync(flags, 0, nflags, s);
     if (e == cudaSuccess) {
         k_support<<<grid_for((long long)m * ny * nx), 256, 0, s>>>(h, m, ny, nx, flags, flags + (size_t)m * ny);
@@ -1114,7 +1202,7 @@ pce_status setup_sectioned(pce_plan* p, const float* h, cudaStream_t s) {
     std::vector<unsigned char> hf(nflags);
     if (e == cudaSuccess) e = cudaMemcpyAsync(hf.data(), flags, nflags, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(flags);
+    pce_rt::mem_free(flags, s);
     PCE_CK(e);
     std::vector<HSupport> sup(m);
     int max_snc = 1;
@@ -1206,14 +1294,14 @@ pce_status setup_sectioned(pce_plan* p, const float* h, cudaStream_t s) {
     pce_status st;
     // twiddles: one-warp 1024-point columns, Stockham rows of lc
     if (!p->tw1024) {
-        if ((st = dev_alloc(&p->tw1024, 1024))) return st;
+        if ((st = dev_alloc(&p->tw1024, 1024, s))) return st;
         k_twiddles_1024<<<4, 256, 0, s>>>(p->tw1024);
         PCE_CK(cudaGetLastError());
     }
-    if ((st = dev_alloc(&p->sec_twc, (size_t)std::max(1, twiddle_len(lc))))) return st;
+    if ((st = dev_alloc(&p->sec_twc, (size_t)std::max(1, twiddle_len(lc)), s))) return st;
     k_twiddles<<<grid_for(twiddle_len(lc)), 256, 0, s>>>(p->sec_twc, lc);
     float2* twr = nullptr;   // Stockham twiddles of 1024 (the column pass of the section spectra)
-    if ((st = dev_alloc(&twr, (size_t)twiddle_len(1024)))) return st;
+    if ((st = dev_alloc(&twr, (size_t)twiddle_len(1024), s))) return st;
     k_twiddles<<<grid_for(twiddle_len(1024)), 256, 0, s>>>(twr, 1024);
     PCE_CK(cudaGetLastError());
     // section spectra of h_k: place, row R2C, column FFT, transpose
@@ -1223,16 +1311,16 @@ pce_status setup_sectioned(pce_plan* p, const float* h, cudaStream_t s) {
     float2* S = nullptr;
     float2* hs = nullptr;
     auto cleanup = [&]() {
-        if (dsup) cudaFree(dsup);
-        if (sec) cudaFree(sec);
-        if (S) cudaFree(S);
-        if (hs) cudaFree(hs);
-        cudaFree(twr);
+        pce_rt::mem_free(dsup, s);
+        pce_rt::mem_free(sec, s);
+        pce_rt::mem_free(S, s);
+        pce_rt::mem_free(hs, s);
+        pce_rt::mem_free(twr, s);
     };
-    e = cudaMalloc(&dsup, sizeof(HSupport) * m);
-    if (e == cudaSuccess) e = cudaMalloc(&sec, sizeof(float) * (size_t)m * 1024 * lc);
-    if (e == cudaSuccess) e = cudaMalloc(&S, sizeof(float2) * (size_t)m * 1024 * lch);
-    if (e == cudaSuccess) e = cudaMalloc(&hs, sizeof(float2) * (size_t)m * 1024 * lch);
+    e = pce_rt::mem_alloc(reinterpret_cast<void**>(&dsup), sizeof(HSupport) * m, s);
+    if (e == cudaSuccess) e = pce_rt::mem_alloc(reinterpret_cast<void**>(&sec), sizeof(float) * (size_t)m * 1024 * lc, s);
+    if (e == cudaSuccess) e = pce_rt::mem_alloc(reinterpret_cast<void**>(&S), sizeof(float2) * (size_t)m * 1024 * lch, s);
+    if (e == cudaSuccess) e = pce_rt::mem_alloc(reinterpret_cast<void**>(&hs), sizeof(float2) * (size_t)m * 1024 * lch, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dsup, sup.data(), sizeof(HSupport) * m, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
         k_place_h<<<grid_for((long long)m * 1024 * lc), 256, 0, s>>>(h, ny, nx, dsup, m, lc, sec);
@@ -1241,14 +1329,14 @@ pce_status setup_sectioned(pce_plan* p, const float* h, cudaStream_t s) {
     if (e == cudaSuccess)
         e = pce::launch_rows_r2c(lc, false, dim3(r2c_blocks(512, lc), m), s, sec, 1024LL * lc, 1024, nullptr, false,
                                  nullptr, nullptr, 512, S, 1024LL * lch, 0, p->sec_twc, p->tw1024);
-    if (e == cudaSuccess && (st = dev_alloc(&p->hsN, (size_t)m * 1024)) != PCE_OK) {
+    if (e == cudaSuccess && (st = dev_alloc(&p->hsN, (size_t)m * 1024, s)) != PCE_OK) {
         cleanup();
         return st;
     }
     const int cpc = pce::cols_columns_per_cta(1024);
     if (e == cudaSuccess)
         e = pce::launch_cols_spec(1024, dim3(m, (lch + cpc - 1) / cpc), s, S, lch, hs, p->hsN, twr);
-    if (e == cudaSuccess && (st = dev_alloc(&p->hsT, (size_t)m * 1024 * lch)) != PCE_OK) {
+    if (e == cudaSuccess && (st = dev_alloc(&p->hsT, (size_t)m * 1024 * lch, s)) != PCE_OK) {
         cleanup();
         return st;
     }
@@ -1260,10 +1348,10 @@ pce_status setup_sectioned(pce_plan* p, const float* h, cudaStream_t s) {
     cleanup();
     if (e != cudaSuccess) return fail(PCE_ERR_CUDA, "section spectra: %s", cudaGetErrorString(e));
     // windows, work lists, scratch
-    if ((st = dev_alloc(&p->d_geo_f, (size_t)std::max(nsec, 1)))) return st;
-    if ((st = dev_alloc(&p->d_geo_a, (size_t)std::max(nsec, 1)))) return st;
-    if ((st = dev_alloc(&p->sec_items_box, std::max<size_t>(ibox.size(), 1)))) return st;
-    if ((st = dev_alloc(&p->sec_items_win, std::max<size_t>(iwin.size(), 1)))) return st;
+    if ((st = dev_alloc(&p->d_geo_f, (size_t)std::max(nsec, 1), s))) return st;
+    if ((st = dev_alloc(&p->d_geo_a, (size_t)std::max(nsec, 1), s))) return st;
+    if ((st = dev_alloc(&p->sec_items_box, std::max<size_t>(ibox.size(), 1), s))) return st;
+    if ((st = dev_alloc(&p->sec_items_win, std::max<size_t>(iwin.size(), 1), s))) return st;
     if (nsec > 0) {
         PCE_CK(cudaMemcpyAsync(p->d_geo_f, gf.data(), sizeof(SecGeom) * nsec, cudaMemcpyHostToDevice, s));
         PCE_CK(cudaMemcpyAsync(p->d_geo_a, ga.data(), sizeof(SecGeom) * nsec, cudaMemcpyHostToDevice, s));
@@ -1281,20 +1369,20 @@ pce_status setup_sectioned(pce_plan* p, const float* h, cudaStream_t s) {
     p->sec_b = (long long)std::max(nsec, 1) * p->sec_k;
     const long long per_b = 2 * p->sec_b * (long long)sizeof(float2);
     p->sec_chunk = (int)std::max<long long>(1, std::min<long long>(kMaxChunk, kScratchBudget / per_b));
-    if ((st = dev_alloc(&p->scrZs, (size_t)(p->sec_b * p->sec_chunk)))) return st;
-    if ((st = dev_alloc(&p->scrAs, (size_t)(p->sec_b * p->sec_chunk)))) return st;
+    if ((st = dev_alloc(&p->scrZs, (size_t)(p->sec_b * p->sec_chunk), s))) return st;
+    if ((st = dev_alloc(&p->scrAs, (size_t)(p->sec_b * p->sec_chunk), s))) return st;
     if (p->lowp) {
         // reduced storage: half2 section spectra with their own per-term scales
         const long long per = 1024LL * lch;
         if ((st = term_scales(p->hsT, per, p->hsN, 1024, m, s, &p->sec_hscale))) return st;
-        if ((st = dev_alloc(&p->hsT16, (size_t)(per * m)))) return st;
-        if ((st = dev_alloc(&p->hsN16, (size_t)m * 1024))) return st;
+        if ((st = dev_alloc(&p->hsT16, (size_t)(per * m), s))) return st;
+        if ((st = dev_alloc(&p->hsN16, (size_t)m * 1024, s))) return st;
         k_quantize_h<<<grid_for(per * m), 256, 0, s>>>(p->hsT, per, m, p->sec_hscale, p->hsT16);
         k_quantize_h<<<grid_for(1024LL * m), 256, 0, s>>>(p->hsN, 1024, m, p->sec_hscale, p->hsN16);
         PCE_CK(cudaGetLastError());
         PCE_CK(cudaStreamSynchronize(s));
-        cudaFree(p->hsT);
-        cudaFree(p->hsN);
+        pce_rt::mem_free(p->hsT, s);
+        pce_rt::mem_free(p->hsN, s);
         p->hsT = nullptr;
         p->hsN = nullptr;
     }
@@ -1871,15 +1959,15 @@ pce_status create_separable(pce_plan_t* out, const int64_t* shape, int m, const 
         return fail(PCE_ERR_INVALID, "wy and wx must be device pointers");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     float* w = nullptr;
-    if ((st = dev_alloc(&w, (size_t)m * ny * nx))) return st;
+    if ((st = dev_alloc(&w, (size_t)m * ny * nx, s))) return st;
     k_outer<<<grid_for((long long)m * ny * nx), 256, 0, s>>>(wy, wx, m, ny, nx, w);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
-        cudaFree(w);
+        pce_rt::mem_free(w, s);
         return fail(PCE_ERR_CUDA, "window outer products: %s", cudaGetErrorString(e));
     }
     st = create_common(out, 2, shape, m, w, h, spectra, flags, stream);
-    cudaFree(w);
+    pce_rt::mem_free(w, s);
     if (st) return st;
     if ((st = setup_separable(*out, wy, wx, s))) {
         delete *out;
@@ -1963,9 +2051,20 @@ pce_status pce_plan_hhat(pce_plan_t plan, float* hhat, void* stream) {
 
 pce_status pce_plan_destroy(pce_plan_t plan) {
     if (!plan) return PCE_OK;
-    cudaError_t e = cudaDeviceSynchronize();
+    // the plan's own device: its work ends before its memory goes back
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    const bool other = e == cudaSuccess && dev != plan->device;
+    if (other) e = cudaSetDevice(plan->device);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
     delete plan;
+    if (other) cudaSetDevice(dev);
     if (e != cudaSuccess) return fail(PCE_ERR_CUDA, "synchronise before free: %s", cudaGetErrorString(e));
+    return PCE_OK;
+}
+
+pce_status pce_release_memory(void) {
+    PCE_CK(pce_rt::mem_release());
     return PCE_OK;
 }
 

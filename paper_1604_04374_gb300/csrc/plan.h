@@ -14,6 +14,16 @@
 using pce::Box;
 using pce::SecGeom;
 
+namespace pce_rt {
+
+// Plan memory (pce_api.cu): device memory for use after s's current work, and its
+// return, stream-ordered on s, on the current device.
+cudaError_t mem_alloc(void** p, size_t bytes, cudaStream_t s);
+void mem_free(void* p, cudaStream_t s);
+cudaError_t mem_release();
+
+}  // namespace pce_rt
+
 struct pce_plan {
     int ndims = 0, ny = 1, nx = 0, m = 0;
     uint32_t flags = 0;
@@ -139,8 +149,8 @@ struct pce_plan {
                         twN,    hh4,   wrow, wxbox, d_vbox, d_kslot, d_korder, sitems, skptr, sklist,
                         hN2,    hN2_16, tw2048l, d_geo_f, d_geo_a, sec_items_box, sec_items_win, hsT, hsN,
                         sec_twc, scrZs, scrAs, hsT16, hsN16, sec_hscale, d_kq0, hhTr, hNr, d_slot_toff, col_tab};
-        for (void* q : ptrs)
-            if (q) cudaFree(q);
+        // the device is idle (or the plan never ran); the current device is the plan's
+        for (void* q : ptrs) pce_rt::mem_free(q, cudaStreamPerThread);
     }
 };
 

@@ -71,6 +71,8 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
                                   ctypes.POINTER(i64)]
     lib.pce_plan_hhat.argtypes = [P, P, P]
     lib.pce_plan_destroy.argtypes = [P]
+    lib.pce_release_memory.argtypes = []
+    lib.pce_release_memory.restype = ctypes.c_int
     lib.pce_last_error_string.restype = ctypes.c_char_p
     lib.pce_last_error_string.argtypes = []
     lib.pce_launch_count.argtypes = [P, ctypes.c_int, i64]
@@ -222,6 +224,11 @@ def pce_plan_hhat(plan: int, hhat_ptr: int, stream: int = 0) -> None:
 
 def pce_plan_destroy(plan: int) -> None:
     _check(load_library().pce_plan_destroy(plan))
+
+
+def pce_release_memory() -> None:
+    """Return the device memory the library keeps for later plans (at most 2 GiB a device)."""
+    _check(load_library().pce_release_memory())
 
 
 def pce_launch_count(plan: int, adjoint: bool, batch: int) -> int:
