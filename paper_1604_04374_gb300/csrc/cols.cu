@@ -215,6 +215,7 @@ bool tables_missing(const ColArgs& c) {
 cudaError_t launch_cols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride,
                             long long z_kstride, float2* A, long long a_bstride) {
     if (tables_missing(c)) return cudaErrorInvalidValue;
+    if (c.split > 1) return launch_cols_fwd_split(c, s, Z, z_bstride, z_kstride, A, a_bstride);
     return c.lowp ? cols_fwd<__half2>(c, s, Z, z_bstride, z_kstride, A, a_bstride)
                   : cols_fwd<float2>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
 }
@@ -304,7 +305,10 @@ cudaError_t launch_cols_fwd_sep_tm(int ny, dim3 grid, cudaStream_t s, const floa
                                    long long z_kstride, const float2* hhT, const float2* hN, const Box* box,
                                    int nxh, float2* A, long long a_bstride, const float2* tw1024, int* status,
                                    long long wait_limit, int skip_copy, const SepTerms& sep) {
-    if (!tw1024 || !hhT) return cudaErrorInvalidValue;
+    if (!tw1024 || !hhT || (grid.z > 1 && (sep.kq0 || sep.t1 >= 0))) return cudaErrorInvalidValue;
+    if (grid.z > 1)
+        return launch_cols_fwd_sep_split(ny, grid, s, Z, z_bstride, z_kstride, hhT, hN, box, nxh, A, a_bstride, tw1024,
+                                         sep);
     if (ny == 512 && !sep.kq0) {   // 512-point columns: no pruned form
         kt_cols_fwd<false, 512><<<grid, kWColWarps * 32, kt_smem<512>(), s>>>(
             Z, z_bstride, z_kstride, hhT, hN, box, nxh, A, a_bstride, tw1024, status, wait_limit, skip_copy, sep);

@@ -1611,15 +1611,17 @@ pce::ColArgs col_args(const pce_plan* p, int nb, bool warp, bool lowp, unsigned 
     return c;
 }
 
-// CTAs that share a column tile's terms in the adjoint: doubled while the grid of ctas
+// CTAs that share a column tile's terms, 1 or `least` to `most`: doubled while the grid of ctas
 // column CTAs fills no more than the GPU's `per_sm` resident CTAs an SM and every CTA
-// keeps a unit of work (a term or a slot).  Beyond one wave a split only adds work, an
-// FFT of V a CTA.  Every unit's result is formed by one CTA: the same bits for any split.
+// keeps a unit of work (a term or a slot).  Beyond one wave a split only adds work: an
+// FFT of V a CTA (adjoint), the exchange within the cluster (forward).  The same bits for
+// any split: every unit's result is formed by one CTA (adjoint), the terms are added in
+// order (forward, colsplit.cu).
 // 1024^2 separable, m = 16, one right-hand side, forward and adjoint: 223 -> 180 us.
-int col_split(long long ctas, int per_sm, int units) {
+int col_split(long long ctas, int per_sm, int units, int least, int most) {
     int n = 1;
-    while (n < pce::kMaxCluster && 2 * n <= units && ctas * 2 * n <= (long long)pce::kSms * per_sm) n *= 2;
-    return n;
+    while (n < most && 2 * n <= units && ctas * 2 * n <= (long long)pce::kSms * per_sm) n *= 2;
+    return n >= least ? n : 1;
 }
 
 pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, bool adjoint,
@@ -1771,18 +1773,23 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
     const int fpc = pce::rows_pairs_per_cta(nx);
     const int cpc = warp && ny == 2048 ? 4 : pce::cols_columns_per_cta(ny);   // columns a CTA
     const int npairs = (ny + 1) / 2;
-    // column CTAs per SM, and the units the adjoint's column tile divides into: one in a
-    // batch's lane, where every further CTA repeats the FFT of V while other tasks could
-    // use the SM
+    // column CTAs per SM, the units a column tile divides into, and the most CTAs that
+    // share it: one in a batch's lane, where other tasks could use the SM
     const int col_ctas = !warp ? 4 : ny == 512 ? 6 : ny == 2048 ? 2 : 4;
-    const bool whole = !adjoint || scr.beside;
-    const int col_units = whole ? 1 : sepx ? p->nslots : m;
+    const int col_units = adjoint ? (sepx ? p->nslots : m) : (sepx ? p->nterms : m);
+    const int col_most = scr.beside ? 1
+                         : adjoint  ? pce::kMaxCluster
+                         : !sepx    ? pce::cols_fwd_max_split(ny)
+                         : septm && !prune ? pce::kMinSplit
+                                           : 1;
+    // two CTAs a tile don't repay the exchange: 256^2, m = 16, 8 right-hand sides 41 -> 51 us
+    const int col_least = adjoint ? 1 : pce::kMinSplit;
     for (long long b0 = 0; b0 < batch && e == cudaSuccess; b0 += bal) {
         const int nb = (int)std::min<long long>(bal, batch - b0);
         const float* src = in + b0 * P;
         float* dst = out + b0 * P;
         dim3 cgrid(nb, (nxh + cpc - 1) / cpc);
-        if (!slotwise) cgrid.z = col_split((long long)cgrid.x * cgrid.y, col_ctas, col_units);
+        if (!slotwise) cgrid.z = col_split((long long)cgrid.x * cgrid.y, col_ctas, col_units, col_least, col_most);
         if (slotwise && !adjoint) {
             for (size_t a = 0; a < active.size() && e == cudaSuccess; ++a) {
                 const int j = active[a];
@@ -1897,7 +1904,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
                 });
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_COLS_FWD, s, [&] {
-                    return pce::launch_cols_fwd(col_args(p, nb, warp, p->lowp), s, scr.Z, zb, zk, scr.A, ab);
+                    return pce::launch_cols_fwd(col_args(p, nb, warp, p->lowp, cgrid.z), s, scr.Z, zb, zk, scr.A, ab);
                 });
             if (e == cudaSuccess)
                 e = timed(p, PCE_KERNEL_ROWS_C2R, s, [&] {

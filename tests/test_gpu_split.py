@@ -106,3 +106,22 @@ def test_2d_column_splits(torch_cuda, ny, nx, gy, gx, batch, zero):
     for cv in {512: (0, 2), 1024: (0, 2)}.get(ny, ()):
         sep.set_tuning(0, cv, 2)
         check(sep, TOL)
+
+
+@pytest.mark.parametrize("ny,nx,gy,gx,zero", [(16, 32, 3, 3, ()), (64, 128, 1, 2, ()), (128, 64, 5, 1, (0, 3)),
+                                              (256, 256, 4, 4, (0, 1, 15)), (512, 128, 3, 3, ()), (1024, 64, 1, 3, ()),
+                                              (1024, 128, 5, 1, (2,))])
+def test_2d_forward_splits_keep_the_bits(torch_cuda, ny, nx, gy, gx, zero):
+    """A right-hand side alone (terms over a cluster) equals the same one in a batch
+    (fewer or no CTAs a tile) bit for bit: dense plans, both storages, and separable ones."""
+    torch = torch_cuda
+    from paper_1604_04374_gb300 import Plan, pce
+    wy, wx, h, u = problem_2d(ny, nx, gy, gx, 40, zero)
+    w = (wy[:, :, None] * wx[:, None, :]).astype(np.float32)
+    ud, hd = dev(torch, u), dev(torch, h)
+    plans = [Plan(dev(torch, w), h=hd), Plan(dev(torch, w), h=hd, flags=pce.PCE_FLAG_LOWP_STORAGE),
+             Plan(wy=dev(torch, wy), wx=dev(torch, wx), h=hd)]
+    for plan in plans:
+        y = plan.apply(ud)
+        for b in (0, 17, 39):
+            assert torch.equal(plan.apply(ud[b:b + 1].contiguous())[0], y[b])
