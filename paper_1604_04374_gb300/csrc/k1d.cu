@@ -95,13 +95,71 @@ cudaError_t launch_l1_cols(int ny, int mode, dim3 grid, cudaStream_t s, const fl
     return cudaGetLastError();
 }
 
-cudaError_t launch_l1_rows_fwd(int nx, dim3 grid, cudaStream_t s, const float2* G, int npairs,
+namespace {
+
+// The kernels for few right-hand sides: while nb right-hand sides' one-pair CTAs, at most
+// 128 registers a thread, fit the GPU at once (N = 65536: up to 9, N = 16384: up to 37;
+// forward and adjoint there still 1.1 and 1.4 times as fast).  Not for rows or columns of
+// 512: N = 262144, m = 32, one right-hand side, adjoint 111 -> 121 us.
+template <int N>
+bool l1_few(int ny, int nb) {
+    return N <= 256 && ny <= 256 && (long long)(ny / 2 + 1) * nb <= (long long)kSms * (512 / L1Few<N>::NT);
+}
+
+template <int N>
+void l1_rows_fwd(int nb, cudaStream_t s, const float2* G, int npairs, const float2* hh4, int m, int ny,
+                 const float2* twN, float2* A, const float2* tw) {
+    constexpr int IT = L1Rows<N>::ITEMS;
+    if constexpr (N <= 256) {
+        if (l1_few<N>(ny, nb)) {
+            k4_rows_fwd_few<N><<<dim3(ny / 2 + 1, nb), L1Few<N>::NT, L1Few<N>::SMEM, s>>>(G, npairs, hh4, m, ny, twN, A,
+                                                                                          tw);
+            return;
+        }
+    }
+    k4_rows_fwd<N><<<dim3((ny / 2 + IT) / IT, nb), L1Rows<N>::NT, L1Rows<N>::SMEM, s>>>(G, npairs, hh4, m, ny, twN, A,
+                                                                                        tw);
+}
+
+// alone: the pairs may go to several CTAs
+template <int N>
+void l1_rows_adj(int nb, bool alone, cudaStream_t s, const float2* V, int npairs, const float2* hh4, int m, int ny,
+                 const float2* twN, float2* Q, const float2* tw) {
+    constexpr int R = 2 * L1Rows<N>::ITEMS;
+    if constexpr (N <= 256) {
+        if (l1_few<N>(ny, nb)) {
+            int split = 1;
+            while (alone && 2 * split <= npairs && l1_few<N>(ny, 2 * split * nb)) split *= 2;
+            k4_rows_adj_few<N><<<dim3(ny / 2, nb, split), L1Few<N>::NT, L1Few<N>::SMEM, s>>>(V, npairs, hh4, m, ny, twN,
+                                                                                             Q, tw);
+            return;
+        }
+    }
+    k4_rows_adj<N><<<dim3((ny + R - 1) / R, nb), L1Rows<N>::NT, L1Rows<N>::SMEM, s>>>(V, npairs, hh4, m, ny, twN, Q,
+                                                                                      tw);
+}
+
+template <int N>
+void l1_cols_adj(dim3 grid, cudaStream_t s, const float2* Q, int npairs, const float* w, int m, int nx, float* x,
+                 float scale, const float2* tw) {
+    if constexpr (N <= 256) {
+        if (nx <= 256 && grid.x * grid.y <= 2 * kSms) {   // about two CTAs an SM
+            k4_cols_adj_few<N><<<grid, ColCfg<N>::NT, ColCfg<N>::SMEM, s>>>(Q, npairs, w, m, nx, x, scale, tw);
+            return;
+        }
+    }
+    k4_cols_adj<N><<<grid, ColCfg<N>::NT, ColCfg<N>::SMEM, s>>>(Q, npairs, w, m, nx, x, scale, tw);
+}
+
+}  // namespace
+
+cudaError_t launch_l1_rows_fwd(int nx, int nb, cudaStream_t s, const float2* G, int npairs,
                                const float2* hh4, int m, int ny, const float2* twN, float2* A,
                                const float2* tw) {
     switch (nx) {
 #define X(N)                                                                                   \
     case N:                                                                                    \
-        k4_rows_fwd<N><<<grid, L1Rows<N>::NT, L1Rows<N>::SMEM, s>>>(G, npairs, hh4, m, ny, twN, A, tw); \
+        l1_rows_fwd<N>(nb, s, G, npairs, hh4, m, ny, twN, A, tw);                              \
         break;
         PCE_L1_SIZES(X)
 #undef X
@@ -126,13 +184,13 @@ cudaError_t launch_l1_cols_inv(int ny, dim3 grid, cudaStream_t s, const float2* 
     return cudaGetLastError();
 }
 
-cudaError_t launch_l1_rows_adj(int nx, dim3 grid, cudaStream_t s, const float2* V, int npairs,
+cudaError_t launch_l1_rows_adj(int nx, int nb, bool alone, cudaStream_t s, const float2* V, int npairs,
                                const float2* hh4, int m, int ny, const float2* twN, float2* Q,
                                const float2* tw) {
     switch (nx) {
 #define X(N)                                                                                   \
     case N:                                                                                    \
-        k4_rows_adj<N><<<grid, L1Rows<N>::NT, L1Rows<N>::SMEM, s>>>(V, npairs, hh4, m, ny, twN, Q, tw); \
+        l1_rows_adj<N>(nb, alone, s, V, npairs, hh4, m, ny, twN, Q, tw);                       \
         break;
         PCE_L1_SIZES(X)
 #undef X
@@ -147,7 +205,7 @@ cudaError_t launch_l1_cols_adj(int ny, dim3 grid, cudaStream_t s, const float2* 
     switch (ny) {
 #define X(N)                                                                                   \
     case N:                                                                                    \
-        k4_cols_adj<N><<<grid, ColCfg<N>::NT, ColCfg<N>::SMEM, s>>>(Q, npairs, w, m, nx, x, scale, tw); \
+        l1_cols_adj<N>(grid, s, Q, npairs, w, m, nx, x, scale, tw);                            \
         break;
         PCE_L1_SIZES(X)
 #undef X

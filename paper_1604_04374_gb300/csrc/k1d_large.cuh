@@ -283,6 +283,182 @@ k4_cols_adj(const float2* __restrict__ Q, int npairs, const float* __restrict__ 
     }
 }
 
+// Few right-hand sides (N <= 65536): the chain of a row's term pairs is the time, and
+// CTAs of several row pairs use a few SMs (33 CTAs at N = 65536, one right-hand side).
+// The kernels below take one row pair a CTA and a pair's loads ahead of the FFT before it, in
+// registers that the packed kernels rather spend on more warps; the same operations in
+// the same order.  m = 16, one right-hand side: N = 65536 forward 30.9 -> 24.9 us (row
+// kernel 14.0 -> 8.7), adjoint 45.3 -> 25 to 27; N = 16384 forward 25 -> 23.5, adjoint 39 -> 22.5.
+template <int NX>
+struct L1Few {
+    static constexpr int T = NX / kR;
+    static constexpr int NT = 2 * T;
+    static constexpr int SMEM = 2 * fft_region(NX) * (int)sizeof(float2);
+};
+
+// K2.  Grid (NY / 2 + 1, batch).
+template <int NX>
+__global__ void __launch_bounds__(L1Few<NX>::NT)
+k4_rows_fwd_few(const float2* __restrict__ G, int npairs, const float2* __restrict__ hh4, int m, int NY,
+                const float2* __restrict__ twN, float2* __restrict__ A, const float2* __restrict__ tw) {
+    constexpr int T = L1Few<NX>::T;
+    extern __shared__ float2 smem[];
+    const int side = threadIdx.x / T;
+    const int j = threadIdx.x - side * T;
+    float2* b0 = smem + side * fft_region(NX);
+    float2* b1 = b0 + pad_len(NX);
+    const int a0 = blockIdx.x;
+    const int a = side == 0 ? a0 : (NY - a0) & (NY - 1);
+    const int b = blockIdx.y;
+    const long long N = (long long)NY * NX;
+    // partner row: the other side's, or this one for a in {0, NY/2}
+    const float2* pbuf = (a == 0 || 2 * a == NY) ? b0 : smem + (side ^ 1) * fft_region(NX);
+    const float2* G0 = G + (long long)b * npairs * N + (long long)a * NX + j;
+    const float2* H = hh4 + (long long)a * NX + j;
+    float2 acc[kR], vn[kR], tn[kR];
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+        acc[r] = make_float2(0.f, 0.f);
+        vn[r] = __ldg(&G0[r * T]);
+    }
+    for (int p = 0; p < npairs; ++p) {
+        const int k0 = 2 * p, k1 = 2 * p + 1 < m ? 2 * p + 1 : k0;
+        const float2* Gn = G0 + (p + 1 < npairs ? p + 1 : p) * N;
+        float2 v[kR], x0[kR], x1[kR];
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            v[r] = vn[r];
+            x0[r] = __ldg(&H[k0 * N + r * T]);
+            x1[r] = __ldg(&H[k1 * N + r * T]);
+            vn[r] = __ldg(&Gn[r * T]);
+        }
+        fft<NX, false>(v, j, b0, b1, tw);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kR; ++r) b0[padi(j + r * T)] = v[r];
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            float2 X0, X1;
+            split_dc_nyq(v[r], pbuf[padi(l1_partner_col(a, j + r * T, NX))], X0, X1);
+            acc[r] = cfma(x0[r], X0, acc[r]);
+            if (k1 != k0) acc[r] = cfma(x1[r], X1, acc[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kR; ++r) tn[r] = __ldg(&twN[(long long)(j + r * T) * a]);
+    fft<NX, true>(acc, j, b0, b1, tw);
+    if (side == 0 || a != a0) {
+        float2* Ar = A + (long long)b * N + (long long)a * NX;
+#pragma unroll
+        for (int r = 0; r < kR; ++r) Ar[j + r * T] = cmulc(acc[r], tn[r]);
+    }
+}
+
+// K2'.  Grid (NY / 2, batch, split): two rows a CTA; CTA z takes its share of the pairs
+// (each forms the row FFT of V itself).
+template <int NX>
+__global__ void __launch_bounds__(L1Few<NX>::NT)
+k4_rows_adj_few(const float2* __restrict__ V, int npairs, const float2* __restrict__ hh4, int m, int NY,
+                const float2* __restrict__ twN, float2* __restrict__ Q, const float2* __restrict__ tw) {
+    constexpr int T = L1Few<NX>::T;
+    extern __shared__ float2 smem[];
+    const int side = threadIdx.x / T;
+    const int j = threadIdx.x - side * T;
+    float2* b0 = smem + side * fft_region(NX);
+    float2* b1 = b0 + pad_len(NX);
+    const int a = 2 * blockIdx.x + side;
+    const int b = blockIdx.y;
+    const long long N = (long long)NY * NX;
+    const int pbeg = share_beg(npairs, blockIdx.z, gridDim.z), pend = share_beg(npairs, blockIdx.z + 1, gridDim.z);
+    const float2* Vr = V + (long long)b * N + (long long)a * NX + j;
+    const float2* H = hh4 + (long long)a * NX + j;
+    float2 vv[kR], x0[kR], x1[kR], tn[kR];
+    auto load_h = [&](int p) {
+        const int k0 = 2 * p, k1 = 2 * p + 1 < m ? 2 * p + 1 : k0;
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            x0[r] = __ldg(&H[k0 * N + r * T]);
+            x1[r] = __ldg(&H[k1 * N + r * T]);
+        }
+    };
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+        vv[r] = __ldg(&Vr[r * T]);
+        tn[r] = __ldg(&twN[(long long)(j + r * T) * a]);
+    }
+    load_h(pbeg);
+    fft<NX, false>(vv, j, b0, b1, tw);
+    for (int p = pbeg; p < pend; ++p) {
+        float2 q[kR];
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            float2 t = cmulc(vv[r], x0[r]);
+            if (2 * p + 1 < m) {
+                const float2 s = cmulc(vv[r], x1[r]);
+                t.x -= s.y;
+                t.y += s.x;
+            }
+            q[r] = t;
+        }
+        load_h(p + 1 < pend ? p + 1 : p);
+        fft<NX, true>(q, j, b0, b1, tw);
+        float2* Qr = Q + ((long long)b * npairs + p) * N + (long long)a * NX + j;
+#pragma unroll
+        for (int r = 0; r < kR; ++r) Qr[r * T] = cmulc(q[r], tn[r]);
+    }
+}
+
+// K3'.  Grid (batch, NX / C).
+template <int NY>
+__global__ void __launch_bounds__(ColCfg<NY>::NT)
+k4_cols_adj_few(const float2* __restrict__ Q, int npairs, const float* __restrict__ w, int m, int NX,
+                float* __restrict__ x, float scale, const float2* __restrict__ tw) {
+    using CC = ColCfg<NY>;
+    constexpr int T = CC::T, C = CC::C;
+    extern __shared__ float2 smem[];
+    const int c = threadIdx.x % C, j = threadIdx.x / C;
+    float2* b0 = smem + c * CC::CS;
+    float2* b1 = b0 + pad_len(NY);
+    const int b = blockIdx.x;
+    const int col = blockIdx.y * C + c;
+    const bool cv = col < NX;
+    const long long N = (long long)NY * NX;
+    const long long n0 = (cv ? col : 0) + (long long)NX * j, step = (long long)NX * T;
+    const float2* Q0 = Q + (long long)b * npairs * N + n0;
+    float2 vn[kR];
+    float acc[kR];
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+        acc[r] = 0.f;
+        vn[r] = __ldg(&Q0[r * step]);
+    }
+    for (int p = 0; p < npairs; ++p) {
+        const int k0 = 2 * p, k1 = 2 * p + 1 < m ? 2 * p + 1 : k0;
+        const float2* Qn = Q0 + (p + 1 < npairs ? p + 1 : p) * N;
+        float2 v[kR];
+        float x0[kR], x1[kR];
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            v[r] = vn[r];
+            x0[r] = __ldg(w + k0 * N + n0 + r * step);
+            x1[r] = __ldg(w + k1 * N + n0 + r * step);
+            vn[r] = __ldg(&Qn[r * step]);
+        }
+        fft<NY, true, kColLayout>(v, j, b0, b1, tw);
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            acc[r] = fmaf(x0[r], v[r].x, acc[r]);
+            if (k1 != k0) acc[r] = fmaf(x1[r], v[r].y, acc[r]);
+        }
+    }
+    if (cv) {
+        float* xb = x + (long long)b * N + n0;
+#pragma unroll
+        for (int r = 0; r < kR; ++r) xb[r * step] = acc[r] * scale;
+    }
+}
+
 // Plan: the separated spectra of h_{2p}, h_{2p+1} in the four-step order,
 // hh4[k][a][col].  Grid (ceil((NY/2 + 1) / ITEMS), npairs).
 template <int NX>

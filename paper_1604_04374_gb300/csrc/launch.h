@@ -185,12 +185,13 @@ int l1_row_items(int nx);
 cudaError_t launch_l1_cols(int ny, int mode, dim3 grid, cudaStream_t s, const float* src,
                            long long src_bstride, const float* w, int m, int nx, const float2* twN,
                            float2* G, const float2* tw);
-cudaError_t launch_l1_rows_fwd(int nx, dim3 grid, cudaStream_t s, const float2* G, int npairs,
+cudaError_t launch_l1_rows_fwd(int nx, int nb, cudaStream_t s, const float2* G, int npairs,
                                const float2* hh4, int m, int ny, const float2* twN, float2* A,
                                const float2* tw);
 cudaError_t launch_l1_cols_inv(int ny, dim3 grid, cudaStream_t s, const float2* A, int nx, float* y,
                                float scale, const float2* tw);
-cudaError_t launch_l1_rows_adj(int nx, dim3 grid, cudaStream_t s, const float2* V, int npairs,
+// alone: no other apply runs beside this one (the pairs may be split over CTAs)
+cudaError_t launch_l1_rows_adj(int nx, int nb, bool alone, cudaStream_t s, const float2* V, int npairs,
                                const float2* hh4, int m, int ny, const float2* twN, float2* Q,
                                const float2* tw);
 cudaError_t launch_l1_cols_adj(int ny, dim3 grid, cudaStream_t s, const float2* Q, int npairs,

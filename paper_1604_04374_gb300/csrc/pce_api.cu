@@ -1642,7 +1642,6 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
         const int npairs = (m + 1) / 2;
         const int cpc = pce::l1_cols_per_cta(NY);
         const int tiles = (NX + cpc - 1) / cpc;
-        const int it = pce::l1_row_items(NX);
         const int kind = adjoint ? PCE_KERNEL_ADJ_1D : PCE_KERNEL_FWD_1D;
         for (long long b0 = 0; b0 < batch && e == cudaSuccess; b0 += bal) {
             const int nb = (int)std::min<long long>(bal, batch - b0);
@@ -1655,7 +1654,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
                 });
                 if (e == cudaSuccess)
                     e = timed(p, kind, s, [&] {
-                        return pce::launch_l1_rows_fwd(NX, dim3((NY / 2 + 1 + it - 1) / it, nb), s, scr.Z, npairs,
+                        return pce::launch_l1_rows_fwd(NX, nb, s, scr.Z, npairs,
                                                        p->hh4, m, NY, p->twN, scr.A, p->twx);
                     });
                 if (e == cudaSuccess)
@@ -1669,7 +1668,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
                 });
                 if (e == cudaSuccess)
                     e = timed(p, kind, s, [&] {
-                        return pce::launch_l1_rows_adj(NX, dim3((NY + 2 * it - 1) / (2 * it), nb), s, scr.A,
+                        return pce::launch_l1_rows_adj(NX, nb, !scr.beside, s, scr.A,
                                                        npairs, p->hh4, m, NY, p->twN, scr.Z, p->twx);
                     });
                 if (e == cudaSuccess)

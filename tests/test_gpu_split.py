@@ -125,3 +125,31 @@ def test_2d_forward_splits_keep_the_bits(torch_cuda, ny, nx, gy, gx, zero):
         y = plan.apply(ud)
         for b in (0, 17, 39):
             assert torch.equal(plan.apply(ud[b:b + 1].contiguous())[0], y[b])
+
+
+TOL_LONG = 2.2e-6
+
+
+@pytest.mark.parametrize("n,batch", [(16384, 38), (65536, 10), (262144, 3)])
+@pytest.mark.parametrize("m", [1, 5, 16])
+def test_long_1d_splits_keep_the_bits(torch_cuda, n, m, batch):
+    """N > 8192: a right-hand side alone (one row pair a CTA, the adjoint's term pairs over
+    CTAs) equals the same one in the smallest batch of packed CTAs bit for bit, and the
+    FFT convolution in FP64 (bar: 18 stages each way of eps = 6e-8, 2.2e-6)."""
+    torch = torch_cuda
+    from paper_1604_04374_gb300 import Plan
+    w, h, u = problem_1d(n, m, batch)
+    wd, hd, ud = dev(torch, w), dev(torch, h), dev(torch, u)
+    plan = Plan(wd, h=hd)
+    y, x = plan.apply(ud), plan.apply_adjoint(ud)
+    hh = torch.fft.rfft(hd.double())
+    yr = torch.fft.irfft((torch.fft.rfft(wd.double() * ud[-1].double()) * hh).sum(0), n=n)
+    xr = (wd.double() * torch.fft.irfft(torch.fft.rfft(ud[-1].double()) * hh.conj(), n=n)).sum(0)
+    assert rel(y[-1:], host(yr)) <= TOL_LONG and rel(x[-1:], host(xr)) <= TOL_LONG
+    for b in (0, batch - 1):
+        assert torch.equal(plan.apply(ud[b:b + 1].contiguous())[0], y[b])
+        assert torch.equal(plan.apply_adjoint(ud[b:b + 1].contiguous())[0], x[b])
+
+
+def host(t):
+    return t.detach().cpu().numpy()[None]
