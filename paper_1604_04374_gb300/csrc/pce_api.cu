@@ -88,7 +88,12 @@ cudaMemPool_t current_pool() {
 cudaError_t mem_alloc(void** p, size_t bytes, cudaStream_t s) {
     cudaMemPool_t pool = current_pool();
     if (!pool) return cudaMalloc(p, bytes);
-    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+    // never into a graph under capture: plan memory is made at once, as by cudaMalloc
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &cs);
+    if (e != cudaSuccess) return e;
+    if (cs != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         cudaMemPoolTrimTo(pool, 0);
