@@ -227,6 +227,9 @@ pce_status pce_plan_hhat(pce_plan_t plan, float* hhat, void* stream);
  * pce_plan_destroy -- free the plan and all its device memory (synchronises the device).
  * The library keeps up to 2 GiB of freed plan memory per device for later plans;
  * pce_release_memory synchronises and returns what no plan uses to the device.
+ * Where the device cannot be synchronised (another thread captures one of its streams),
+ * both return PCE_ERR_CUDA; the handle is gone all the same, and the plan's memory is
+ * freed by the next of these calls that can wait for its work.
  */
 pce_status pce_plan_destroy(pce_plan_t plan);
 pce_status pce_release_memory(void);

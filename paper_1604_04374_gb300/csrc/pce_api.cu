@@ -51,6 +51,7 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mem_mutex;
 cudaMemPool_t g_mem_pool[kMaxDevices] = {};
 bool g_mem_asked[kMaxDevices] = {};
+pce_plan* g_parked = nullptr;   // plans whose work may still be running, linked by next_parked
 
 // The device's pool, made at the first call; null where pools are not supported.
 cudaMemPool_t mem_pool(int dev) {
@@ -108,6 +109,47 @@ void mem_free(void* p, cudaStream_t s) {
     else cudaFree(p);
 }
 
+void plan_free(pce_plan* p, cudaError_t waited) {
+    if (waited == cudaSuccess) {
+        delete p;
+        return;
+    }
+    cudaGetLastError();   // the caller has it; the thread's next launch check must not
+    std::lock_guard<std::mutex> lock(g_mem_mutex);
+    p->next_parked = g_parked;
+    g_parked = p;
+}
+
+namespace {
+
+// Waits for device dev, the current one, and frees the plans parked on it.
+cudaError_t wait_and_unpark(int dev) {
+    pce_plan* mine = nullptr;   // taken before the wait, so that it covers their work
+    {
+        std::lock_guard<std::mutex> lock(g_mem_mutex);
+        for (pce_plan** at = &g_parked; *at;) {
+            pce_plan* p = *at;
+            if (p->device != dev) {
+                at = &p->next_parked;
+                continue;
+            }
+            *at = p->next_parked;
+            p->next_parked = mine;
+            mine = p;
+        }
+    }
+    const cudaError_t e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) cudaGetLastError();   // the caller has it
+    while (mine) {
+        pce_plan* p = mine;
+        mine = p->next_parked;
+        plan_free(p, e);
+    }
+    return e;
+}
+
+}  // namespace
+
 cudaError_t mem_release() {
     int cur = 0;
     cudaError_t e = cudaGetDevice(&cur);
@@ -119,8 +161,9 @@ cudaError_t mem_release() {
             pool = g_mem_pool[d];
         }
         if (!pool) continue;
-        // only memory whose stream-ordered frees have run can go back
         e = cudaSetDevice(d);
+        if (e == cudaSuccess) e = wait_and_unpark(d);
+        // only memory whose stream-ordered frees have run can go back
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
         if (e == cudaSuccess) e = cudaMemPoolTrimTo(pool, 0);
     }
@@ -886,8 +929,7 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
     p->flags = flags;
     p->device = dev;
     auto bail = [&](pce_status e) {
-        cudaStreamSynchronize(s);
-        delete p;
+        pce_rt::plan_free(p, cudaStreamSynchronize(s));   // its work is on s alone
         return e;
     };
     if (ndims == 1 && nx > 8192) {
@@ -2067,8 +2109,8 @@ pce_status pce_plan_destroy(pce_plan_t plan) {
     cudaError_t e = cudaGetDevice(&dev);
     const bool other = e == cudaSuccess && dev != plan->device;
     if (other) e = cudaSetDevice(plan->device);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    delete plan;
+    if (e == cudaSuccess) e = pce_rt::wait_and_unpark(plan->device);
+    pce_rt::plan_free(plan, e);
     if (other) cudaSetDevice(dev);
     if (e != cudaSuccess) return fail(PCE_ERR_CUDA, "synchronise before free: %s", cudaGetErrorString(e));
     return PCE_OK;

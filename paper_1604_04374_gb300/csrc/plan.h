@@ -14,6 +14,8 @@
 using pce::Box;
 using pce::SecGeom;
 
+struct pce_plan;
+
 namespace pce_rt {
 
 // Plan memory (pce_api.cu): device memory for use after s's current work, and its
@@ -21,6 +23,11 @@ namespace pce_rt {
 cudaError_t mem_alloc(void** p, size_t bytes, cudaStream_t s);
 void mem_free(void* p, cudaStream_t s);
 cudaError_t mem_release();
+// Frees p, whose work was waited for with the result `waited`.  Where that wait failed
+// (a device synchronisation is an error while another thread captures a stream of the
+// device) the work may still be running: p is then parked, and freed by the next
+// plan_destroy or mem_release that does wait for its device.
+void plan_free(pce_plan* p, cudaError_t waited);
 
 }  // namespace pce_rt
 
@@ -149,9 +156,11 @@ struct pce_plan {
                         twN,    hh4,   wrow, wxbox, d_vbox, d_kslot, d_korder, sitems, skptr, sklist,
                         hN2,    hN2_16, tw2048l, d_geo_f, d_geo_a, sec_items_box, sec_items_win, hsT, hsN,
                         sec_twc, scrZs, scrAs, hsT16, hsN16, sec_hscale, d_kq0, hhTr, hNr, d_slot_toff, col_tab};
-        // the device is idle (or the plan never ran); the current device is the plan's
+        // the plan's work has ended (pce_rt::plan_free: the frees are ordered after nothing
+        // else); the current device is the plan's
         for (void* q : ptrs) pce_rt::mem_free(q, cudaStreamPerThread);
     }
+    pce_plan* next_parked = nullptr;
 };
 
 namespace pce_rt {

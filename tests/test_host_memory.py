@@ -1,0 +1,115 @@
+"""Plan memory on the host: what the library allocates, frees and keeps, without a GPU.
+
+A child process runs libpce.so on a CUDA runtime of host memory (fake_cudart.cpp) that counts
+work as pending until its stream or the device is synchronised.
+"""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes, sys
+fake = ctypes.CDLL(sys.argv[1], mode=ctypes.RTLD_GLOBAL)
+sys.path.insert(0, sys.argv[2])
+import paper_1604_04374_gb300.pce as pce
+lib = pce.load_library()
+P, SZ = ctypes.c_void_p, ctypes.c_size_t
+for f in ("fake_live_bytes", "fake_kept_bytes"):
+    getattr(fake, f).restype = SZ
+fake.fake_set_capacity.argtypes = [SZ]
+fake.fake_fail_alloc.argtypes = [ctypes.c_longlong]
+fake.cudaMalloc.argtypes = [ctypes.POINTER(P), SZ]
+fake.fake_launch.restype = ctypes.c_char_p
+fake.fake_launch.argtypes = [ctypes.c_int, P, P]
+S1, S2 = 0x1000, 0x2000   # streams
+
+def dmalloc(floats):
+    p = P()
+    assert fake.cudaMalloc(ctypes.byref(p), 4 * floats) == 0
+    ctypes.memset(p, 0, 4 * floats)
+    return p.value
+
+def create(shape, m, flags=0, stream=S1, sep=False):
+    \"\"\"(status, handle) of a plan of zero windows.\"\"\"
+    n = 1
+    for d in shape:
+        n *= d
+    out, shp, h = P(), (ctypes.c_int64 * len(shape))(*shape), dmalloc(m * n)
+    if sep:
+        st = lib.pce_plan_create_separable(ctypes.byref(out), shp, m, dmalloc(m * shape[0]), dmalloc(m * shape[1]), h,
+                                           flags, P(stream))
+    else:
+        st = lib.pce_plan_create(ctypes.byref(out), len(shape), shp, m, dmalloc(m * n), h, flags, P(stream))
+    return st, out.value
+
+def same(*pairs):
+    for a, b in zip(pairs[::2], pairs[1::2]):
+        if a != b:
+            raise AssertionError(f"{a} != {b} (last error: {lib.pce_last_error_string()})")
+
+def pool():
+    return fake.fake_live_bytes() - base
+
+def launches():
+    d, smem, out = (ctypes.c_uint * 6)(), SZ(), []
+    for i in range(fake.fake_launches()):
+        name = fake.fake_launch(i, d, ctypes.byref(smem)).decode()
+        out.append((name, tuple(d[:3]), tuple(d[3:])))
+    return out
+"""
+
+
+@pytest.fixture(scope="module")
+def child(tmp_path_factory):
+    from paper_1604_04374_gb300 import build
+    build.build()
+    so = str(tmp_path_factory.mktemp("fake") / "libfakecudart.so")
+    cuda = os.path.dirname(os.path.dirname(build._nvcc()))
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-I", os.path.join(cuda, "include"),
+                    os.path.join(HERE, "fake_cudart.cpp"), "-o", so], check=True)
+
+    def run(body):
+        res = subprocess.run([sys.executable, "-c", PRELUDE + textwrap.dedent(body), so, ROOT], timeout=300,
+                             stdout=subprocess.PIPE, stderr=subprocess.STDOUT)
+        assert res.returncode == 0, res.stdout.decode(errors="replace")[-4000:]
+
+    return run
+
+
+@pytest.mark.parametrize("shape", [(4096,), (16384,), (256, 256)])
+def test_a_plan_that_cannot_wait_keeps_its_memory(child, shape):
+    """A device synchronisation is an error while a stream of the device is captured.  A plan
+    destroyed then, its work pending, says so, and none of its memory goes back before a later
+    call has waited."""
+    child(f"""
+    shape = {shape}
+    n = shape[0] * (shape + (1,))[1]
+    u, y = dmalloc(n), dmalloc(n)
+    st, plan = create(shape, 4)
+    st2, other = create(shape, 4)
+    same(st, 0, st2, 0)
+    base = fake.fake_live_bytes()
+    same(lib.pce_apply(P(plan), P(u), P(y), 1, P(S2)), 0)
+    fake.fake_set_capturing(1)
+    same(lib.pce_plan_destroy(P(plan)), pce.PCE_ERR_CUDA)
+    same(fake.fake_unordered_frees(), 0, pool(), 0, fake.fake_pending(), 1)
+    fake.fake_set_capturing(0)
+    same(lib.pce_plan_destroy(P(other)), 0)   # waits: both plans' memory goes back
+    freed = -pool()
+    same(fake.fake_unordered_frees(), 0)
+    # the same when the memory is asked for
+    st, plan = create(shape, 4)
+    base = fake.fake_live_bytes()
+    same(lib.pce_apply(P(plan), P(u), P(y), 1, P(S2)), 0)
+    fake.fake_set_capturing(1)
+    same(lib.pce_plan_destroy(P(plan)), pce.PCE_ERR_CUDA, lib.pce_release_memory(), pce.PCE_ERR_CUDA, pool(), 0)
+    fake.fake_set_capturing(0)
+    same(lib.pce_release_memory(), 0)
+    same(2 * -pool(), freed, fake.fake_unordered_frees(), 0, fake.fake_kept_bytes(), 0)
+    """)
