@@ -2023,7 +2023,7 @@ pce_status create_separable(pce_plan_t* out, const int64_t* shape, int m, const 
     pce_rt::mem_free(w, s);
     if (st) return st;
     if ((st = setup_separable(*out, wy, wx, s))) {
-        delete *out;
+        pce_rt::plan_free(*out, cudaStreamSynchronize(s));   // copies into its arrays are on s
         *out = nullptr;
         return st;
     }

@@ -113,3 +113,32 @@ def test_a_plan_that_cannot_wait_keeps_its_memory(child, shape):
     same(lib.pce_release_memory(), 0)
     same(2 * -pool(), freed, fake.fake_unordered_frees(), 0, fake.fake_kept_bytes(), 0)
     """)
+
+
+@pytest.mark.parametrize("shape,m,flags,sep", [((512, 64), 3, 0, True), ((1024, 32), 2, 0, True),
+                                               ((256, 64), 2, 0, False), ((1024, 64), 2, "SECTIONED", False),
+                                               ((2048, 16), 2, "LOWP_STORAGE", False), ((2048,), 3, 0, False),
+                                               ((32768,), 3, 0, False)])
+def test_a_failed_creation_frees_in_order(child, shape, m, flags, sep):
+    """Every allocation of a plan's creation fails in turn: the creation reports it, what it
+    had allocated goes back, and only after its stream's work."""
+    child(f"""
+    shape, m, sep = {shape}, {m}, {sep}
+    flags = pce.PCE_FLAG_{flags} if {flags!r} else 0
+    base0 = fake.fake_live_bytes()
+    st, plan = create(shape, m, flags, S1, sep)
+    same(st, 0, lib.pce_plan_destroy(P(plan)), 0)
+    inputs = fake.fake_live_bytes() - base0   # create()'s own
+    for n in range(200):
+        base = fake.fake_live_bytes()
+        fake.fake_fail_alloc(n + (3 if sep else 2))
+        st, plan = create(shape, m, flags, S1, sep)
+        fake.fake_fail_alloc(-1)
+        fake.cudaGetLastError()
+        if st == 0:
+            break
+        assert st in (pce.PCE_ERR_OOM, pce.PCE_ERR_CUDA), st
+        same(plan, None, pool(), inputs, fake.fake_unordered_frees(), 0)
+    assert 3 < n < 199, n
+    same(lib.pce_plan_destroy(P(plan)), 0, fake.fake_unordered_frees(), 0)
+    """)
