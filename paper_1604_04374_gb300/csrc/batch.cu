@@ -258,7 +258,7 @@ extern "C" pce_status pce_batch_create(pce_batch_t* out, const pce_task* tasks, 
     for (int l = 0; l < lanes; ++l) off[l + 1] = off[l] + round_up(need[l], 32);
     b->scratch_bytes = off[lanes] * (long long)sizeof(float2);
     if (off[lanes] > 0) {
-        cudaError_t e = cudaMalloc(&b->lane_mem, (size_t)b->scratch_bytes);
+        cudaError_t e = pce_rt::raw_alloc(&b->lane_mem, (size_t)b->scratch_bytes);
         if (e != cudaSuccess) {
             delete b;
             return fail(e == cudaErrorMemoryAllocation ? PCE_ERR_OOM : PCE_ERR_CUDA,
@@ -529,9 +529,9 @@ extern "C" pce_status pce_plan_autotune(pce_plan_t p, int64_t batch, const char*
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
     };
-    cudaError_t e = cudaMalloc(&in, sizeof(float) * P * batch);
-    if (e == cudaSuccess) e = cudaMalloc(&out, sizeof(float) * P * batch);
-    if (e == cudaSuccess) e = cudaMalloc(&flush, flush_bytes);
+    cudaError_t e = pce_rt::raw_alloc(&in, sizeof(float) * P * batch);
+    if (e == cudaSuccess) e = pce_rt::raw_alloc(&out, sizeof(float) * P * batch);
+    if (e == cudaSuccess) e = pce_rt::raw_alloc(&flush, flush_bytes);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     if (e == cudaSuccess) {
@@ -663,7 +663,7 @@ extern "C" pce_status pce_batch_autotune(pce_batch_t b, void* stream) {
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
     };
-    cudaError_t e = cudaMalloc(&flush, flush_bytes);
+    cudaError_t e = pce_rt::raw_alloc(&flush, flush_bytes);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     if (e != cudaSuccess) {

@@ -138,8 +138,8 @@ extern "C" pce_status pce_construct_projection_bspline_1d(const float* T, int n,
         if (R) cudaFree(R);
         if (Gi) cudaFree(Gi);
     };
-    cudaError_t e = cudaMalloc(&R, sizeof(double) * (size_t)n * m);
-    if (e == cudaSuccess) e = cudaMalloc(&Gi, sizeof(double) * (size_t)m * m);
+    cudaError_t e = pce_rt::raw_alloc(&R, sizeof(double) * (size_t)n * m);
+    if (e == cudaSuccess) e = pce_rt::raw_alloc(&Gi, sizeof(double) * (size_t)m * m);
     if (e == cudaSuccess) {
         k_bsplines<<<grid_of((long long)m * n), 256, 0, s>>>(n, m, alpha, w_out);
         k_proj_rhs<<<grid_of((long long)n * m), 256, 0, s>>>(T, w_out, n, m, alpha, R);
@@ -307,8 +307,8 @@ extern "C" pce_status pce_construct_projection_2d(const float* T, int ny, int nx
         if (R) cudaFree(R);
         if (Gi) cudaFree(Gi);
     };
-    cudaError_t e = cudaMalloc(&R, sizeof(double) * (size_t)m * S);
-    if (e == cudaSuccess) e = cudaMalloc(&Gi, sizeof(double) * (size_t)m * m);
+    cudaError_t e = pce_rt::raw_alloc(&R, sizeof(double) * (size_t)m * S);
+    if (e == cudaSuccess) e = pce_rt::raw_alloc(&Gi, sizeof(double) * (size_t)m * m);
     if (e == cudaSuccess) e = cudaMemsetAsync(h_out, 0, sizeof(float) * (size_t)m * ny * nx, s);
     if (e == cudaSuccess) {
         k_hat_factors<<<grid_of((long long)m * (ny + nx)), 256, 0, s>>>(ny, nx, gy, gx, wy_out, wx_out);
@@ -574,11 +574,11 @@ extern "C" pce_status pce_construct_svd_1d(const float* T, int n, int m, int ove
             if (q) cudaFree(q);
     };
     const size_t nl = (size_t)n * l;
-    cudaError_t e = cudaMalloc(&Y, sizeof(double) * nl);
-    if (e == cudaSuccess) e = cudaMalloc(&Z, sizeof(double) * nl);
-    if (e == cudaSuccess) e = cudaMalloc(&tmp, sizeof(double) * nl);
-    if (e == cudaSuccess) e = cudaMalloc(&M, sizeof(double) * (size_t)l * l);
-    if (e == cudaSuccess) e = cudaMalloc(&sc, sizeof(double) * (size_t)std::max(l, m));
+    cudaError_t e = pce_rt::raw_alloc(&Y, sizeof(double) * nl);
+    if (e == cudaSuccess) e = pce_rt::raw_alloc(&Z, sizeof(double) * nl);
+    if (e == cudaSuccess) e = pce_rt::raw_alloc(&tmp, sizeof(double) * nl);
+    if (e == cudaSuccess) e = pce_rt::raw_alloc(&M, sizeof(double) * (size_t)l * l);
+    if (e == cudaSuccess) e = pce_rt::raw_alloc(&sc, sizeof(double) * (size_t)std::max(l, m));
     if (e != cudaSuccess) {
         cleanup();
         return fail(e == cudaErrorMemoryAllocation ? PCE_ERR_OOM : PCE_ERR_CUDA, "svd set-up: %s",

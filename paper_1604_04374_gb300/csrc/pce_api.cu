@@ -86,21 +86,44 @@ cudaMemPool_t current_pool() {
 
 }  // namespace
 
-cudaError_t mem_alloc(void** p, size_t bytes, cudaStream_t s) {
-    cudaMemPool_t pool = current_pool();
-    if (!pool) return cudaMalloc(p, bytes);
-    // never into a graph under capture: plan memory is made at once, as by cudaMalloc
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(s, &cs);
-    if (e != cudaSuccess) return e;
-    if (cs != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
-    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        cudaMemPoolTrimTo(pool, 0);
-        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+namespace {
+
+cudaError_t wait_and_unpark(int dev);
+
+// alloc(), and where memory has run out once more after the device has taken back what
+// the pool keeps: a wait, since only frees known to have run can go back, then the trim.
+// A refusal's error goes to the caller alone, not to the thread's next launch check.
+template <class F>
+cudaError_t alloc_with_room(F alloc) {
+    cudaError_t e = alloc();
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    int dev = 0;
+    cudaMemPool_t pool = nullptr;
+    if (cudaGetDevice(&dev) == cudaSuccess) pool = mem_pool(dev);
+    if (pool && wait_and_unpark(dev) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess &&
+        cudaMemPoolTrimTo(pool, 0) == cudaSuccess) {
+        e = alloc();
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();
     }
     return e;
+}
+
+}  // namespace
+
+cudaError_t mem_alloc(void** p, size_t bytes, cudaStream_t s) {
+    cudaMemPool_t pool = current_pool();
+    if (!pool) return alloc_with_room([&] { return cudaMalloc(p, bytes); });
+    // never into a graph under capture: plan memory is made at once, as by cudaMalloc
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &cs);
+    if (e != cudaSuccess) return e;
+    if (cs != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
+    return alloc_with_room([&] { return cudaMallocFromPoolAsync(p, bytes, pool, s); });
+}
+
+cudaError_t raw_alloc_bytes(void** p, size_t bytes) {
+    return alloc_with_room([&] { return cudaMalloc(p, bytes); });
 }
 
 void mem_free(void* p, cudaStream_t s) {

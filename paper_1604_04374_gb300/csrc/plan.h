@@ -22,6 +22,12 @@ namespace pce_rt {
 // return, stream-ordered on s, on the current device.
 cudaError_t mem_alloc(void** p, size_t bytes, cudaStream_t s);
 void mem_free(void* p, cudaStream_t s);
+// cudaMalloc (freed by cudaFree) that may use what the pool of plan memory keeps.
+cudaError_t raw_alloc_bytes(void** p, size_t bytes);
+template <class T>
+cudaError_t raw_alloc(T** p, size_t bytes) {
+    return raw_alloc_bytes(reinterpret_cast<void**>(p), bytes);
+}
 cudaError_t mem_release();
 // Frees p, whose work was waited for with the result `waited`.  Where that wait failed
 // (a device synchronisation is an error while another thread captures a stream of the

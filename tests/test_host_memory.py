@@ -142,3 +142,47 @@ def test_a_failed_creation_frees_in_order(child, shape, m, flags, sep):
     assert 3 < n < 199, n
     same(lib.pce_plan_destroy(P(plan)), 0, fake.fake_unordered_frees(), 0)
     """)
+
+
+@pytest.mark.parametrize("call", ["plan", "batch", "autotune", "svd", "projection_1d", "projection_2d"])
+def test_what_the_pool_keeps_serves_every_allocation(child, call):
+    """Memory of closed plans serves the library's next allocation, of whatever kind, where the
+    device has no other; where there is none at all the call is refused, and its refusal is not
+    reported again by the next one."""
+    child(f"""
+    call = {call!r}
+    st, held = create((1024, 1024), 1)
+    same(st, 0)
+    keep = [create((65536,), 2)[1] for _ in range(2)]
+    n = 1024 * 1024
+    u, y0, y1, T, h, w, w2 = (dmalloc(n) for _ in range(7))
+    task = (pce.PceTask * 2)(*(pce.PceTask(k, u, y, 1, 0, 0) for k, y in zip(keep, (y0, y1))))
+    shape, out = (ctypes.c_int64 * 1)(8192), P()
+
+    def run():
+        \"\"\"Whether memory ran out.\"\"\"
+        if call == "plan":
+            st = lib.pce_plan_create(ctypes.byref(out), 1, shape, 32, P(u), P(T), 0, P(S1))
+        elif call == "batch":
+            st = lib.pce_batch_create(ctypes.byref(out), task, 2, 2)
+        elif call == "autotune":
+            st = lib.pce_plan_autotune(P(keep[0]), 1, None, P(S1))
+        elif call == "svd":
+            st = lib.pce_construct_svd_1d(P(T), 1024, 8, 10, 2, 0, P(h), P(w), None, P(S1))
+        elif call == "projection_1d":
+            st = lib.pce_construct_projection_1d(P(T), 1024, 8, P(h), P(w), P(S1))
+        else:
+            st = lib.pce_construct_projection_2d(P(T), 32, 32, 16, 16, 2, 2, P(h), P(w), P(w2), P(S1))
+        # (the windows are zero here: a projection that got its memory ends at its Gram matrix)
+        assert st != pce.PCE_ERR_INVALID or b"singular" in lib.pce_last_error_string()
+        return st != 0 and b"out of memory" in lib.pce_last_error_string()
+
+    same(lib.pce_release_memory(), 0)
+    fake.fake_set_capacity(fake.fake_live_bytes() + 1024)   # nothing left for it
+    for _ in range(2):
+        same(run(), True, fake.cudaGetLastError(), 0)
+    kept = fake.fake_kept_bytes()
+    same(lib.pce_plan_destroy(P(held)), 0)
+    assert fake.fake_kept_bytes() > kept + (4 << 20)        # its memory stays in the pool
+    same(run(), False, fake.cudaGetLastError(), 0, fake.fake_unordered_frees(), 0)
+    """)
