@@ -230,35 +230,48 @@ cudaError_t launch_l1_rows_spec(int nx, dim3 grid, cudaStream_t s, const float2*
     return cudaGetLastError();
 }
 
+namespace {
+
+// Few right-hand sides (a batch that leaves most SMs idle) take wide CTAs, which hold more
+// slots, at 512 to 4096 points (1024: wk1d.cuh), by shares (Sum1d).  At 8192 every CTA holds
+// one slot, by shares for any batch.  Below 512 the narrow CTA's slots hold so many pairs that
+// wide CTAs add none and clusters little (N = 256, m = 40, one right-hand side, adjoint: 8.9 us
+// with clusters, 10.5 without, 12.3 before the slots had barriers of their own).
+template <int N>
+constexpr bool has_wide() { return N >= 512 && N <= 4096 && N != kWarpN; }
+template <int N>
+constexpr bool has_shares() { return has_wide<N>() || N == 8192; }
+
+template <int N, int WIDE, int MODE>
+constexpr int smem_1d() { return MODE == kShares ? Cfg1d<N, WIDE>::SMEM_SHARES : Cfg1d<N, WIDE>::SMEM; }
+
+template <int N, int WIDE, int MODE, typename WT, typename HT>
+cudaError_t prepare_1d_as() {
+    const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const cudaError_t e = cudaFuncSetAttribute(k_fwd_1d<N, WT, HT, WIDE, MODE>, at, smem_1d<N, WIDE, MODE>());
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(k_adj_1d<N, WT, HT, WIDE, MODE>, at, smem_1d<N, WIDE, MODE>());
+}
+
+template <int N, typename WT, typename HT>
+cudaError_t prepare_1d_of() {
+    cudaError_t e = cudaSuccess;
+    if constexpr (N != 8192) e = prepare_1d_as<N, 0, kOneSum, WT, HT>();
+    if constexpr (has_shares<N>()) {
+        if (e == cudaSuccess) e = prepare_1d_as<N, has_wide<N>(), kShares, WT, HT>();
+        if (e == cudaSuccess) e = prepare_1d_as<N, has_wide<N>(), kCluster, WT, HT>();
+    }
+    return e;
+}
+
+}  // namespace
+
 cudaError_t prepare_kernels() {
     cudaError_t e = prepare_cols();
     if (e == cudaSuccess) e = prepare_l1();
     if (e == cudaSuccess) e = prepare_sec();
 #define X(N)                                                                                   \
-    if (e == cudaSuccess)                                                                      \
-        e = cudaFuncSetAttribute(k_fwd_1d<N, float, float2, 1>,                                \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg1d<N, 1>::SMEM); \
-    if (e == cudaSuccess)                                                                      \
-        e = cudaFuncSetAttribute(k_adj_1d<N, float, float2, 1>,                                \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg1d<N, 1>::SMEM); \
-    if (e == cudaSuccess)                                                                      \
-        e = cudaFuncSetAttribute(k_fwd_1d<N, __nv_bfloat16, __half2, 1>,                       \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg1d<N, 1>::SMEM); \
-    if (e == cudaSuccess)                                                                      \
-        e = cudaFuncSetAttribute(k_adj_1d<N, __nv_bfloat16, __half2, 1>,                       \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg1d<N, 1>::SMEM); \
-    if (e == cudaSuccess)                                                                      \
-        e = cudaFuncSetAttribute(k_fwd_1d<N, float, float2>,                                   \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg1d<N>::SMEM); \
-    if (e == cudaSuccess)                                                                      \
-        e = cudaFuncSetAttribute(k_adj_1d<N, float, float2>,                                   \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg1d<N>::SMEM); \
-    if (e == cudaSuccess)                                                                      \
-        e = cudaFuncSetAttribute(k_fwd_1d<N, __nv_bfloat16, __half2>,                          \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg1d<N>::SMEM); \
-    if (e == cudaSuccess)                                                                      \
-        e = cudaFuncSetAttribute(k_adj_1d<N, __nv_bfloat16, __half2>,                          \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg1d<N>::SMEM); \
+    if (e == cudaSuccess) e = prepare_1d_of<N, float, float2>();                               \
+    if (e == cudaSuccess) e = prepare_1d_of<N, __nv_bfloat16, __half2>();                      \
     if (e == cudaSuccess)                                                                      \
         e = cudaFuncSetAttribute(k_spec_1d<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,    \
                                  Cfg1d<N>::SMEM);                                              \
@@ -275,47 +288,74 @@ cudaError_t prepare_kernels() {
 template <int N>
 bool wide_1d(int batch, int m) {
     const int npairs = (m + 1) / 2;
-    return Cfg1d<N, 1>::G > Cfg1d<N>::G && npairs > Cfg1d<N>::G && batch < 2 * 152;
+    return has_wide<N>() && npairs > Cfg1d<N>::G && batch < 2 * 152;
 }
 
 // CTAs per right-hand side: one cluster whose CTAs share the rounds of term pairs
-// that one CTA would run one after another (an SM each), as long as the batch
-// leaves SMs for them and no CTA goes without a round.  N = 8192, m = 32, three
-// right-hand sides, adjoint: 94.3 -> 28.7 us (three clusters of eight).
+// that one CTA would run one after another (an SM each), doubled while the batch
+// leaves SMs for them and a CTA has more than one round.  (Three rounds take four CTAs, one
+// of them idle: one round long, where two CTAs would run two.)  N = 8192, m = 32, three
+// right-hand sides, adjoint: 94.7 -> 28.9 us (three clusters of eight).
 int cluster_1d(int batch, int rounds) {
     int cl = 1;
     while (cl < kMaxCluster && cl < rounds && (long long)batch * 2 * cl <= kSms) cl *= 2;
     return cl;
 }
 
+// Shares of the rounds (Sum1d): as many as the most CTAs, whatever the batch.
+int shares_1d(int rounds) { return cluster_1d(1, rounds); }
+
 // N = 1024 with few right-hand sides: the one-warp kernels (wk1d.cuh)
 bool warp_1d(int n, int batch, const float2* tw1024) { return n == kWarpN && tw1024 && batch < 2 * 152; }
 
 namespace {
 
-template <int N, int WIDE, typename WT, typename HT>
+template <int N, int WIDE, int MODE, typename WT, typename HT>
 cudaError_t run_1d(bool adjoint, int batch, cudaStream_t s, const float* in, const WT* w, const HT* hp,
-                   const float* hscale, int m, float* out, float scale, const float2* tw) {
+                   const float* hscale, int m, float* out, float scale, const float2* tw, int cl, int shares) {
     using CF = Cfg1d<N, WIDE>;
-    const int cl = cluster_1d(batch, ((m + 1) / 2 + CF::G - 1) / CF::G);
-    return launch_cluster(adjoint ? k_adj_1d<N, WT, HT, WIDE> : k_fwd_1d<N, WT, HT, WIDE>, batch * cl, cl, CF::NT,
-                          CF::SMEM, s, in, w, hp, hscale, m, out, scale, tw, cl);
+    return launch_cluster(adjoint ? k_adj_1d<N, WT, HT, WIDE, MODE> : k_fwd_1d<N, WT, HT, WIDE, MODE>, batch * cl, cl,
+                          CF::NT, smem_1d<N, WIDE, MODE>(), s, in, w, hp, hscale, m, out, scale, tw, cl, shares);
+}
+
+template <int N, typename WT, typename HT>
+cudaError_t run_1d_of(bool adjoint, int batch, cudaStream_t s, const float* in, const WT* w, const HT* hp,
+                      const float* hscale, int m, float* out, float scale, const float2* tw) {
+    if constexpr (has_shares<N>()) {
+        constexpr int W = has_wide<N>();
+        if (!W || wide_1d<N>(batch, m)) {
+            const int rounds = ((m + 1) / 2 + Cfg1d<N, W>::G - 1) / Cfg1d<N, W>::G;
+            const int cl = cluster_1d(batch, rounds), shares = shares_1d(rounds);
+            if (cl > 1)
+                return run_1d<N, W, kCluster>(adjoint, batch, s, in, w, hp, hscale, m, out, scale, tw, cl, shares);
+            return run_1d<N, W, kShares>(adjoint, batch, s, in, w, hp, hscale, m, out, scale, tw, 1, shares);
+        }
+    }
+    if constexpr (N != 8192)
+        return run_1d<N, 0, kOneSum>(adjoint, batch, s, in, w, hp, hscale, m, out, scale, tw, 1, 1);
+    return cudaErrorInvalidValue;   // not reached
+}
+
+template <typename WT, typename HT>
+cudaError_t run_warp_1d(bool adjoint, int batch, cudaStream_t s, const float* in, const WT* w, const HT* hp,
+                        const float* hscale, int m, float* out, float scale, const float2* tw1024) {
+    const int rounds = ((m + 1) / 2 + kW1dWarps - 1) / kW1dWarps, shares = shares_1d(rounds);
+    // one share a rank, or no cluster: m = 24, 70 right-hand sides 16.6 us with two, 14.5 alone
+    const int cl = cluster_1d(batch, rounds) == shares ? shares : 1;
+    if (cl > 1)
+        return launch_cluster(adjoint ? kw_adj_1d<WT, HT, kCluster> : kw_fwd_1d<WT, HT, kCluster>, batch * cl, cl,
+                              kW1dWarps * 32, 0, s, in, w, hp, hscale, m, out, scale, tw1024, cl, shares);
+    return launch_cluster(adjoint ? kw_adj_1d<WT, HT, kShares> : kw_fwd_1d<WT, HT, kShares>, batch, 1, kW1dWarps * 32,
+                          0, s, in, w, hp, hscale, m, out, scale, tw1024, 1, shares);
 }
 
 template <typename WT, typename HT>
 cudaError_t apply_1d(bool adjoint, int n, int batch, cudaStream_t s, const float* in, const WT* w, const HT* hp,
                      const float* hscale, int m, float* out, float scale, const float2* tw, const float2* tw1024) {
-    if (warp_1d(n, batch, tw1024)) {
-        const int cl = cluster_1d(batch, ((m + 1) / 2 + kW1dWarps - 1) / kW1dWarps);
-        return launch_cluster(adjoint ? kw_adj_1d<WT, HT> : kw_fwd_1d<WT, HT>, batch * cl, cl, kW1dWarps * 32, 0, s,
-                              in, w, hp, hscale, m, out, scale, tw1024, cl);
-    }
+    if (warp_1d(n, batch, tw1024)) return run_warp_1d(adjoint, batch, s, in, w, hp, hscale, m, out, scale, tw1024);
     switch (n) {
-#define X(N)                                                                                             \
-    case N:                                                                                              \
-        return wide_1d<N>(batch, m)                                                                      \
-                   ? run_1d<N, 1>(adjoint, batch, s, in, w, hp, hscale, m, out, scale, tw)               \
-                   : run_1d<N, 0>(adjoint, batch, s, in, w, hp, hscale, m, out, scale, tw);
+#define X(N) \
+    case N: return run_1d_of<N>(adjoint, batch, s, in, w, hp, hscale, m, out, scale, tw);
         PCE_1D_SIZES(X)
 #undef X
     }

@@ -1041,6 +1041,14 @@ struct Cfg1d {
     // m = 11, 300 right-hand sides, adjoint: 26.6 -> 22.5 us
     static constexpr bool OWN = G == 1 || T == 32 || (T > 32 && WIDE);
     static constexpr int SY = OWN && G > 1 ? kNamedSync : kGroupSync;
+    // shared memory of kShares: the slots' sums so far as well
+    static constexpr int SMEM_SHARES = SMEM + G * N * (int)sizeof(float);
+    // CTAs an SM the kernels are compiled for: 1024 threads of 64 registers, in clusters one
+    // CTA.  N = 4096, m = 24, 800 right-hand sides, adjoint: 225 us with 78 registers, 176 so.
+    // Where 64 spill more, 80: N = 1024, 800 right-hand sides, adjoint 60 us with 126, 49 with 80.
+    static constexpr int min_ctas(int mode, bool lowp) {
+        return mode == 2 ? 1 : !WIDE && (N == 1024 || (lowp && (N == 512 || N == 256))) ? 3 : 1024 / NT;
+    }
 };
 
 // Ask L2 for the `bytes` at p (one 128-byte line per thread of the CTA), so that
@@ -1051,29 +1059,104 @@ __device__ __forceinline__ void prefetch_l2_block(const void* p, long long bytes
         asm volatile("prefetch.global.L2 [%0];\n" ::"l"(c + o));
 }
 
-// Rounds of term pairs one FFT slot runs: slot `first` of `stride` takes pairs
-// first, first + stride, ...  Independent slots stop at their last pair; the
-// others run as many rounds as their CTA's slot 0.
-template <bool OWN>
-__device__ __forceinline__ int rounds_1d(int npairs, int first, int stride, int slot0) {
-    const int f = OWN ? first : slot0;
-    return f < npairs ? (npairs - f + stride - 1) / stride : 0;
+// How a 1D kernel adds a right-hand side's rounds of term pairs (round i: pairs i G + g, slot
+// g): alone in its CTA, a slot's pairs in one sum; alone, by shares; or by shares in a
+// cluster of CTAs.  The shares make a result independent of how many right-hand sides share the
+// call: share v of `shares` (a power of two up to kMaxCluster, by the number of rounds
+// alone) takes rounds v, v + shares, ..., in order; a slot's shares are added in order, then
+// the slots.  A cluster of cl CTAs (cl divides shares) has on rank r the shares v = r mod cl,
+// one sum each, and the sums meet once.  N = 8192, m = 32, adjoint, 3 and 76 and 400 right-hand
+// sides: 28.9, 55.4 and 262 us; with the ranks' own sums added, which follow the batch, 28.9, 53.5 and
+// 270.  Two other orders that don't follow it were slower: one sum a slot, every round's
+// transforms exchanged through the cluster, 35.1, 87.7 and 254; a binary tree of the
+// shares, its partial sums in local memory, 28.9, 57.5 and 296.
+enum Sum1d { kOneSum = 0, kShares = 1, kCluster = 2 };
+
+__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return cadd(a, b); }
+__device__ __forceinline__ float vzero(float) { return 0.f; }
+__device__ __forceinline__ float2 vzero(float2) { return make_float2(0.f, 0.f); }
+__device__ __forceinline__ float cluster_get(const float* p, int r) { return cluster_ld(cluster_map(p, r)); }
+__device__ __forceinline__ float2 cluster_get(const float2* p, int r) { return cluster_ld2(cluster_map(p, r)); }
+
+// Runs round(i, acc) for this rank's rounds i, share by share, and leaves the shares' sums in
+// part[0 .. ) (kOneSum and kShares: the sum of all in part[0]).  kShares: the sum so far waits
+// in shared memory at tot, value r of this thread at tot[r STEP] (in registers the adjoint
+// spilled: 400 right-hand sides 314 us), and the rounds run in one loop (a loop of rounds
+// inside one of shares: 283 us).
+template <int MODE, int STEP, typename T, int K, int P, class F>
+__device__ __forceinline__ void run_shares(T (&part)[P][K], T* tot, int rounds, int shares, int rank, int cl, F round) {
+    T acc[K];
+    auto zero = [&] {
+#pragma unroll
+        for (int r = 0; r < K; ++r) acc[r] = vzero(T());
+    };
+    if constexpr (MODE == kCluster) {
+        for (int i = 0; i * cl < shares; ++i) {
+            zero();
+            for (int rd = i * cl + rank; rd < rounds; rd += shares) round(rd, acc);
+#pragma unroll
+            for (int r = 0; r < K; ++r) part[i][r] = acc[r];
+        }
+    } else {
+        zero();
+        int rd = 0, v = 0;   // round and share
+        for (int i = 0; i < rounds; ++i) {
+            round(rd, acc);
+            rd += MODE == kShares ? shares : 1;
+            if (MODE == kShares && rd >= rounds) {
+                if (v > 0) {
+#pragma unroll
+                    for (int r = 0; r < K; ++r) acc[r] = vadd(tot[r * STEP], acc[r]);
+                }
+                if (i + 1 < rounds) {
+#pragma unroll
+                    for (int r = 0; r < K; ++r) tot[r * STEP] = acc[r];
+                    zero();
+                }
+                rd = ++v;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < K; ++r) part[0][r] = acc[r];
+    }
 }
 
-// y_b = (1/N) C2R( sum_k hhat_k . R2C(w_k . u_b) ).  One cluster of cl CTAs per
-// b (cl = 1: one CTA); each FFT slot takes pairs of terms (w_k u + i w_{k+1} u in
-// one complex FFT) and accumulates the half spectrum in registers; the slots'
-// sums are reduced in shared memory, the CTAs' sums by rank 0 through the
-// cluster's shared memory, and one inverse FFT follows.  hp: [m][N/2] packed
+// The shares' sums of a cluster added in order.  base(g): where slot g's sums are on every
+// rank, its share i cl + rank at base(g)[i LEN ..].  Rank r adds elements [r LEN / cl, (r + 1)
+// LEN / cl) of every slot into its own base(g)[..], elements that no other rank reads there.
+template <int G, int LEN, int NT, class B>
+__device__ __forceinline__ void add_shares(B base, int shares, int rank, int cl) {
+    const int lg = __ffs(LEN / cl) - 1, len = 1 << lg, lc = __ffs(cl) - 1;   // all powers of two
+    cluster_sync();
+    for (int e = threadIdx.x; e < G * len; e += NT) {
+        auto* p = base(e >> lg) + rank * len + (e & (len - 1));
+        decltype(cluster_get(p, 0)) s[kMaxCluster];
+#pragma unroll
+        for (int v = 0; v < kMaxCluster; ++v)
+            if (v < shares) s[v] = cluster_get(p + (v >> lc) * LEN, v & (cl - 1));
+#pragma unroll
+        for (int v = 1; v < kMaxCluster; ++v)
+            if (v < shares) s[0] = vadd(s[0], s[v]);
+        *p = s[0];
+    }
+    cluster_sync();
+}
+
+// y_b = (1/N) C2R( sum_k hhat_k . R2C(w_k . u_b) ).  One CTA per b
+// (kCluster: one cluster of cl CTAs); each FFT slot takes pairs of terms (w_k u + i w_{k+1} u
+// in one complex FFT) and accumulates the half spectrum in registers; the shares'
+// sums of a slot meet through the cluster's shared memory, a part of the frequencies a rank,
+// the slots' in shared memory, and one inverse FFT follows (on rank 0).  hp: [m][N/2] packed
 // spectra.  The slots' FFTs use barriers of their own.
 //
 // Bound by the chain of FFTs of one slot when there are few right-hand sides:
 // the cluster shortens it to ceil(pairs / (cl G)) rounds.
-template <int N, typename WT = float, typename HT = float2, int WIDE = 0>
-__global__ void __launch_bounds__(Cfg1d<N, WIDE>::NT)
+template <int N, typename WT, typename HT, int WIDE, int MODE>
+__global__ void __launch_bounds__(Cfg1d<N, WIDE>::NT, (Cfg1d<N, WIDE>::min_ctas(MODE, sizeof(HT) == 4)))
 k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
          const HT* __restrict__ hp, const float* __restrict__ hscale, int m, float* __restrict__ y, float scale,
-         const float2* __restrict__ tw, int cl) {
+         const float2* __restrict__ tw, int cl, int shares) {
     using CF = Cfg1d<N, WIDE>;
     constexpr int T = CF::T;
     constexpr int G = CF::G;
@@ -1084,8 +1167,8 @@ k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
     const int j = threadIdx.x - slot * T;
     float2* b0 = smem + slot * fft_region(N);
     float2* b1 = b0 + pad_len(N);
-    const int b = blockIdx.x / cl;
-    const int rank = cl > 1 ? cluster_rank() : 0;
+    const int b = MODE == kCluster ? blockIdx.x / cl : blockIdx.x;
+    const int rank = MODE == kCluster ? cluster_rank() : 0;
     // the twiddles and spectra are read stage by stage and after the first FFT:
     // with few right-hand sides (a latency-bound launch) start them towards L2 now
     if (gridDim.x <= 8 * cl && rank == 0) {
@@ -1096,15 +1179,13 @@ k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
     float ureg[kR];
 #pragma unroll
     for (int r = 0; r < kR; ++r) ureg[r] = __ldg(ub + j + r * T);
-    float2 acc[kR / 2];
-#pragma unroll
-    for (int r = 0; r < kR / 2; ++r) acc[r] = make_float2(0.f, 0.f);
-
     const int npairs = (m + 1) / 2;
-    const int iters = rounds_1d<CF::OWN>(npairs, rank * G + slot, cl * G, rank * G);
-    for (int it = 0; it < iters; ++it) {
-        const int pr = (it * cl + rank) * G + slot;
+    float2 part[MODE == kCluster ? kMaxCluster / 2 : 1][kR / 2];
+    float2* tot = smem + G * fft_region(N) + slot * Nh + j;   // kShares
+    run_shares<MODE, T>(part, tot, (npairs + G - 1) / G, shares, rank, cl, [&](int rd, float2 (&acc)[kR / 2]) {
+        const int pr = rd * G + slot;
         const bool a0 = pr < npairs;
+        if (CF::OWN && !a0) return;
         const int k0 = 2 * pr, k1 = k0 + 1;
         const bool a1 = a0 && k1 < m;
         float2 v[kR];
@@ -1145,28 +1226,33 @@ k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
                 }
             }
         }
-    }
-    // the slots' sums into slot 0's second buffer (packed half spectrum), by
-    // the whole CTA; then the other CTAs' sums by rank 0
+    });
+    // the sums into slot 0's second buffer (packed half spectrum): each slot's, a cluster
+    // rank's part of the frequencies, then the slots' in order, then the parts
     __syncthreads();
-#pragma unroll
-    for (int r = 0; r < kR / 2; ++r) b0[j + r * T] = acc[r];
-    __syncthreads();
+    const int f0 = MODE == kCluster ? rank * (Nh / cl) : 0, f1 = MODE == kCluster ? f0 + Nh / cl : Nh;
     float2* red = smem + pad_len(N);
-    for (int f = threadIdx.x; f < Nh; f += CF::NT) {
+    if constexpr (MODE == kCluster) {
+        for (int i = 0; i * cl < shares; ++i)
+#pragma unroll
+            for (int r = 0; r < kR / 2; ++r) b0[i * Nh + j + r * T] = part[i][r];
+        add_shares<G, Nh, CF::NT>([&](int g) { return smem + g * fft_region(N); }, shares, rank, cl);
+        red = smem;   // in place: the second buffer holds shares
+    } else {
+#pragma unroll
+        for (int r = 0; r < kR / 2; ++r) b0[j + r * T] = part[0][r];
+        __syncthreads();
+    }
+    for (int f = f0 + threadIdx.x; f < f1; f += CF::NT) {
         float2 s = smem[f];
         for (int g = 1; g < G; ++g) s = cadd(s, smem[g * fft_region(N) + f]);
         red[f] = s;
     }
-    if (cl > 1) {
+    if constexpr (MODE == kCluster) {
         cluster_sync();
-        if (rank == 0) {
-            for (int f = threadIdx.x; f < Nh; f += CF::NT) {
-                float2 s = red[f];
-                for (int g = 1; g < cl; ++g) s = cadd(s, cluster_ld2(cluster_map(&red[f], g)));
-                red[f] = s;
-            }
-        }
+        red = smem + pad_len(N);
+        if (rank == 0)
+            for (int f = threadIdx.x; f < Nh; f += CF::NT) red[f] = cluster_get(&smem[f], f >> (__ffs(Nh / cl) - 1));
         cluster_sync();   // rank 0 has read the others' shared memory
         if (rank != 0) return;
     }
@@ -1185,17 +1271,17 @@ k_fwd_1d(const float* __restrict__ u, const WT* __restrict__ w,
     }
 }
 
-// x_b = (1/N) sum_k w_k . IFFT( conj(hhat_k) . FFT(v_b) ).  One cluster of cl
-// CTAs per b; every CTA forms FFT(v_b) (independent slots get it from slot 0 through
+// x_b = (1/N) sum_k w_k . IFFT( conj(hhat_k) . FFT(v_b) ).  One CTA per b
+// (kCluster: one cluster of cl CTAs); every CTA forms FFT(v_b) (independent slots get it from slot 0 through
 // shared memory), and its slots take pairs of terms: the two inverse FFTs of
 // a pair are real, so they share one complex inverse FFT.  The windowed sums of
-// the slots are added in shared memory, those of the CTAs through the cluster's
-// shared memory, each rank storing its part of x.
-template <int N, typename WT = float, typename HT = float2, int WIDE = 0>
-__global__ void __launch_bounds__(Cfg1d<N, WIDE>::NT)
+// the shares meet through the cluster's shared memory, those of the slots in shared memory,
+// each rank storing its part of x.
+template <int N, typename WT, typename HT, int WIDE, int MODE>
+__global__ void __launch_bounds__(Cfg1d<N, WIDE>::NT, (Cfg1d<N, WIDE>::min_ctas(MODE, sizeof(HT) == 4)))
 k_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w,
          const HT* __restrict__ hp, const float* __restrict__ hscale, int m, float* __restrict__ x, float scale,
-         const float2* __restrict__ tw, int cl) {
+         const float2* __restrict__ tw, int cl, int shares) {
     using CF = Cfg1d<N, WIDE>;
     constexpr int T = CF::T;
     constexpr int G = CF::G;
@@ -1206,8 +1292,8 @@ k_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w,
     const int j = threadIdx.x - slot * T;
     float2* b0 = smem + slot * fft_region(N);
     float2* b1 = b0 + pad_len(N);
-    const int b = blockIdx.x / cl;
-    const int rank = cl > 1 ? cluster_rank() : 0;
+    const int b = MODE == kCluster ? blockIdx.x / cl : blockIdx.x;
+    const int rank = MODE == kCluster ? cluster_rank() : 0;
     // the twiddles, spectra and windows are read stage by stage and after the
     // FFT of v: with few right-hand sides (a latency-bound launch) start them
     // towards L2 now
@@ -1236,15 +1322,13 @@ k_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w,
         }
         __syncthreads();   // read before slot 0's next FFT reuses its buffers
     }
-    float ax[kR];
-#pragma unroll
-    for (int r = 0; r < kR; ++r) ax[r] = 0.f;
-
     const int npairs = (m + 1) / 2;
-    const int iters = rounds_1d<CF::OWN>(npairs, rank * G + slot, cl * G, rank * G);
-    for (int it = 0; it < iters; ++it) {
-        const int pr = (it * cl + rank) * G + slot;
+    float part[MODE == kCluster ? kMaxCluster / 2 : 1][kR];
+    float* tot = reinterpret_cast<float*>(smem + G * fft_region(N)) + slot * N + j;   // kShares
+    run_shares<MODE, T>(part, tot, (npairs + G - 1) / G, shares, rank, cl, [&](int rd, float (&acc)[kR]) {
+        const int pr = rd * G + slot;
         const bool a0 = pr < npairs;
+        if (CF::OWN && !a0) return;
         const int k0 = 2 * pr, k1 = k0 + 1;
         const bool a1 = a0 && k1 < m;
         const HT* h0 = hp + (long long)(a0 ? k0 : 0) * Nh;
@@ -1268,32 +1352,29 @@ k_adj_1d(const float* __restrict__ vin, const WT* __restrict__ w,
 #pragma unroll
         for (int r = 0; r < kR; ++r) {
             const int n = j + r * T;
-            if (a0) ax[r] = fmaf(ldw(w + (long long)k0 * N + n), p[r].x, ax[r]);
-            if (a1) ax[r] = fmaf(ldw(w + (long long)k1 * N + n), p[r].y, ax[r]);
+            if (a0) acc[r] = fmaf(ldw(w + (long long)k0 * N + n), p[r].x, acc[r]);
+            if (a1) acc[r] = fmaf(ldw(w + (long long)k1 * N + n), p[r].y, acc[r]);
         }
-    }
+    });
     __syncthreads();
     float* fb = reinterpret_cast<float*>(b0);
+    auto at = [&](int g) { return reinterpret_cast<float*>(smem + g * fft_region(N)); };
+    const int n0 = MODE == kCluster ? rank * (N / cl) : 0, n1 = MODE == kCluster ? n0 + N / cl : N;
+    if constexpr (MODE == kCluster) {
+        for (int i = 0; i * cl < shares; ++i)
 #pragma unroll
-    for (int r = 0; r < kR; ++r) fb[j + r * T] = ax[r];
-    __syncthreads();
-    float* xb = x + (long long)b * N;
-    float* red = reinterpret_cast<float*>(smem + pad_len(N));
-    for (int n = threadIdx.x; n < N; n += CF::NT) {
-        float s = reinterpret_cast<const float*>(smem)[n];
-        for (int g = 1; g < G; ++g) s += reinterpret_cast<const float*>(smem + g * fft_region(N))[n];
-        if (cl > 1) red[n] = s;
-        else xb[n] = s * scale;
+            for (int r = 0; r < kR; ++r) fb[i * N + j + r * T] = part[i][r];
+        add_shares<G, N, CF::NT>(at, shares, rank, cl);
+    } else {
+#pragma unroll
+        for (int r = 0; r < kR; ++r) fb[j + r * T] = part[0][r];
+        __syncthreads();
     }
-    if (cl > 1) {
-        cluster_sync();
-        const int part = N / cl;   // both powers of two, cl <= 8 < N
-        for (int n = rank * part + threadIdx.x; n < (rank + 1) * part; n += CF::NT) {
-            float s = 0.f;
-            for (int g = 0; g < cl; ++g) s += cluster_ld(cluster_map(&red[n], g));
-            xb[n] = s * scale;
-        }
-        cluster_sync();   // every rank has read the others' shared memory
+    float* xb = x + (long long)b * N;
+    for (int n = n0 + threadIdx.x; n < n1; n += CF::NT) {
+        float s = at(0)[n];
+        for (int g = 1; g < G; ++g) s += at(g)[n];
+        xb[n] = s * scale;
     }
 }
 

@@ -153,3 +153,26 @@ def test_long_1d_splits_keep_the_bits(torch_cuda, n, m, batch):
 
 def host(t):
     return t.detach().cpu().numpy()[None]
+
+
+@pytest.mark.parametrize("n,ms", [(16, (257, 600)), (32, (129, 300)), (64, (65, 300)), (128, (33, 70)),
+                                  (256, (17, 40, 131)), (512, (17, 40, 131)), (1024, (9, 20, 67)), (2048, (9, 17, 67)),
+                                  (4096, (5, 11, 40)), (8192, (3, 7, 32))])
+def test_1d_results_do_not_depend_on_the_batch(torch_cuda, n, ms):
+    """N <= 8192: a right-hand side alone, in clusters of eight, four and two and in CTAs of
+    its own gives the same bits, both directions, both storages; for the lengths whose
+    CTAs do not change with the batch also beyond 304 right-hand sides."""
+    torch = torch_cuda
+    from paper_1604_04374_gb300 import Plan, pce
+    full = 310 if n <= 256 or n == 8192 else 80
+    for m in ms:
+        w, h, u = problem_1d(n, m, full)
+        ud = dev(torch, u)
+        for flags in (0, pce.PCE_FLAG_LOWP_STORAGE):
+            plan = Plan(dev(torch, w), h=dev(torch, h), flags=flags)
+            for apply in (plan.apply, plan.apply_adjoint):
+                ref = apply(ud)
+                for nb in (1, 3, 20, 39, 80):
+                    assert torch.equal(apply(ud[:nb].contiguous()), ref[:nb]), (m, flags, apply.__name__, nb)
+                assert torch.equal(apply(ud[79:80].contiguous())[0], ref[79])
+            plan.close()
