@@ -1,5 +1,7 @@
 // cols.cu -- instances of the column-pass kernels for NY = 16 .. 2048 (one-warp
 // kernels for NY = 512, 1024 and, two warps per column, 2048).
+#include <algorithm>
+
 #include "kernels.cuh"
 #include "wkernels.cuh"
 #include "wkernels2.cuh"
@@ -11,14 +13,6 @@ namespace pce {
 
 #define PCE_COL_SIZES(X) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048)
 
-int cols_threads(int ny) {
-    switch (ny) {
-#define X(N) case N: return ColCfg<N>::NT;
-        PCE_COL_SIZES(X)
-#undef X
-    }
-    return 0;
-}
 int cols_columns_per_cta(int ny) {
     switch (ny) {
 #define X(N) case N: return ColCfg<N>::C;
@@ -27,13 +21,14 @@ int cols_columns_per_cta(int ny) {
     }
     return 0;
 }
-int cols_smem(int ny) {
+int cols_ctas_per_sm(int ny) {
+    constexpr int kSmSmem = 228 * 1024, kCtaReserve = 1024;   // shared memory of an SM, taken by every CTA
     switch (ny) {
-#define X(N) case N: return ColCfg<N>::SMEM;
+#define X(N) case N: return std::min({4, 2048 / ColCfg<N>::NT, kSmSmem / (ColCfg<N>::SMEM + kCtaReserve)});
         PCE_COL_SIZES(X)
 #undef X
     }
-    return 0;
+    return 1;
 }
 
 template <int NF, int PAR, typename HT>

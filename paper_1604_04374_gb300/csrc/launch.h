@@ -11,10 +11,9 @@ struct Box;
 struct SepTerms;
 struct SecGeom;
 
-// Shared-memory bytes and threads of the column kernels for a column length.
-int cols_threads(int ny);
+// Columns of a CTA of the block column kernels, and such CTAs resident on an SM (at most 4).
 int cols_columns_per_cta(int ny);
-int cols_smem(int ny);
+int cols_ctas_per_sm(int ny);
 // Rows handled per CTA of the row kernels (two rows per FFT).
 int rows_pairs_per_cta(int nx);
 // Row pairs per CTA of the window-gradient row kernel.

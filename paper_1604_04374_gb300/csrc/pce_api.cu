@@ -1844,7 +1844,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
     const int npairs = (ny + 1) / 2;
     // column CTAs per SM, the units a column tile divides into, and the most CTAs that
     // share it: one in a batch's lane, where other tasks could use the SM
-    const int col_ctas = !warp ? 4 : ny == 512 ? 6 : ny == 2048 ? 2 : 4;
+    const int col_ctas = !warp ? pce::cols_ctas_per_sm(ny) : ny == 512 ? 6 : ny == 2048 ? 2 : 4;
     const int col_units = adjoint ? (sepx ? p->nslots : m) : (sepx ? p->nterms : m);
     const int col_most = scr.beside ? 1
                          : adjoint  ? pce::kMaxCluster

@@ -1,4 +1,4 @@
-"""Plan memory on the host: what the library allocates, frees and keeps, without a GPU.
+"""The library's host code without a GPU: what it allocates, frees and keeps, and launches.
 
 A child process runs libpce.so on a CUDA runtime of host memory (fake_cudart.cpp) that counts
 work as pending until its stream or the device is synchronised.
@@ -185,4 +185,33 @@ def test_what_the_pool_keeps_serves_every_allocation(child, call):
     same(lib.pce_plan_destroy(P(held)), 0)
     assert fake.fake_kept_bytes() > kept + (4 << 20)        # its memory stays in the pool
     same(run(), False, fake.cudaGetLastError(), 0, fake.fake_unordered_frees(), 0)
+    """)
+
+
+@pytest.mark.parametrize("shape", [(64, 1024), (256, 512), (512, 512), (1024, 512), (1024, 1024), (2048, 256)])
+def test_column_splits_stay_within_one_wave(child, shape):
+    """The CTAs that share a column tile's terms are doubled while all of them are resident at
+    once, by the threads and shared memory of the kernel that runs."""
+    child(f"""
+    shape, m = {shape}, 16
+    st, plan = create(shape, m)
+    same(st, 0)
+    u, y = (dmalloc(shape[0] * shape[1]) for _ in range(2))
+    splits = 0
+    for cv in (0, 1) if shape[0] >= 512 else (0,):
+        same(lib.pce_plan_set_tuning(P(plan), 0, cv, 0), 0)
+        fake.fake_clear_launches()
+        same(lib.pce_apply(P(plan), P(u), P(y), 1, P(S1)), 0, lib.pce_apply_adjoint(P(plan), P(u), P(y), 1, P(S1)), 0)
+        d, smem, found = (ctypes.c_uint * 6)(), SZ(), 0
+        for i in range(fake.fake_launches()):
+            name = fake.fake_launch(i, d, ctypes.byref(smem)).decode()
+            if "cols" not in name:
+                continue
+            found += 1
+            resident = min(2048 // d[3], 233472 // (smem.value + 1024))
+            ctas = d[0] * d[1] * d[2]
+            splits += d[2] > 1
+            assert d[2] == 1 or ctas <= 152 * resident, (cv, name, list(d), smem.value, resident)
+        same(found, 2)
+    assert splits > 0
     """)
