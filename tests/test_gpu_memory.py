@@ -62,3 +62,28 @@ def test_plan_memory_reuse_and_release():
     assert torch.cuda.mem_get_info()[0] >= free0 - (2 << 30) - slack
     pce.pce_release_memory()
     assert torch.cuda.mem_get_info()[0] >= free0 - slack
+
+
+def test_closed_plans_keep_at_most_two_gib():
+    """Plans of about 4 GiB together, all closed: the library keeps some of their memory, but
+    no more than 2 GiB, until it is asked for it."""
+    import torch
+    from paper_1604_04374_gb300 import Plan, build, pce
+    build.build()
+    dev = torch.device("cuda", 0)
+    big = synth.problem_2d(1024, 1024, 4, 1, 55)
+    w, h = torch.from_numpy(big.w).to(dev), torch.from_numpy(big.h).to(dev)
+    pce.pce_release_memory()
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    plans = [Plan(w, h=h) for _ in range(4)]
+    held = free0 - torch.cuda.mem_get_info()[0]
+    assert held > 3 << 30
+    for p in plans:
+        p.close()
+    torch.cuda.synchronize()
+    slack = 256 << 20
+    kept = free0 - torch.cuda.mem_get_info()[0]
+    assert kept <= (2 << 30) + slack and kept > 0
+    pce.pce_release_memory()
+    assert torch.cuda.mem_get_info()[0] >= free0 - slack

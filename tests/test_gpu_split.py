@@ -127,6 +127,42 @@ def test_2d_forward_splits_keep_the_bits(torch_cuda, ny, nx, gy, gx, zero):
             assert torch.equal(plan.apply(ud[b:b + 1].contiguous())[0], y[b])
 
 
+def forward_split(ny, nx, nb, units, sep):
+    """CTAs that share a column tile's terms in a forward launch of nb right-hand sides."""
+    cols = 4 if sep or ny >= 256 else 128 // (ny // 8)
+    ctas, per_sm, most = nb * -(-(nx // 2) // cols), 6 if ny == 512 else 4, 4 if sep else 8
+    n = 1
+    while n < most and 2 * n <= units and ctas * 2 * n <= 152 * per_sm:
+        n *= 2
+    return n if n >= 4 else 1
+
+
+@pytest.mark.parametrize("ny,nx,gy,gx,zero", [(16, 512, 3, 3, ()), (32, 256, 5, 2, (9,)), (64, 128, 4, 4, (0, 1)),
+                                              (128, 64, 3, 3, (4,)), (256, 32, 4, 4, ()), (512, 64, 3, 3, (0,)),
+                                              (1024, 64, 2, 3, ())])
+def test_2d_forward_split_and_unsplit_launches_agree(torch_cuda, ny, nx, gy, gx, zero):
+    """Launches of 64, 30 and 1 right-hand sides, which take one, four and eight CTAs a tile
+    (separable columns one and four), give the same bits."""
+    torch = torch_cuda
+    from paper_1604_04374_gb300 import Plan, pce
+    wy, wx, h, u = problem_2d(ny, nx, gy, gx, 64, zero)
+    w = (wy[:, :, None] * wx[:, None, :]).astype(np.float32)
+    ud, hd = dev(torch, u), dev(torch, h)
+    sep = ny >= 512
+    few = (1,) if sep else (30, 1)
+    terms = gy * gx - (len(zero) if sep else 0)
+    assert [forward_split(ny, nx, nb, terms, sep) for nb in (64, *few)] == ([1, 4] if sep else [1, 4, 8])
+    plans = ([Plan(wy=dev(torch, wy), wx=dev(torch, wx), h=hd)] if sep else
+             [Plan(dev(torch, w), h=hd), Plan(dev(torch, w), h=hd, flags=pce.PCE_FLAG_LOWP_STORAGE)])
+    for plan in plans:
+        assert plan.info()[2] >= 64 * ny * nx * 4   # scratch for all 64 at once
+        y = plan.apply(ud)
+        for nb in few:
+            for b in (0, 64 - nb):
+                assert torch.equal(plan.apply(ud[b:b + nb].contiguous()), y[b:b + nb])
+        plan.close()
+
+
 TOL_LONG = 2.2e-6
 
 
