@@ -55,6 +55,17 @@ cudaError_t prepare_ccols() {
     return e;
 }
 
+// Every row of Q (the window gradient): block kernels up to 256 rows, kc_cols_adj above.
+template <int N>
+constexpr bool full_block() { return N <= 256; }
+template <int N>
+cudaError_t prepare_full() {
+    if constexpr (full_block<N>())
+        return cudaFuncSetAttribute(k_cols_adj<N, true, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    ColCfg<N>::SMEM);
+    return cudaSuccess;
+}
+
 cudaError_t prepare_cols() {
     cudaError_t e = prepare_ccols();
     if (e == cudaSuccess)
@@ -70,11 +81,9 @@ cudaError_t prepare_cols() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kw2_cols_fwd<__half2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kW2Smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kw_cols_fwd<float2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kWColSmem);
+        e = cudaFuncSetAttribute(kw_cols_fwd<kWarpN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWColSmem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kw_cols_adj<false, float2, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kWColSmem);
+        e = cudaFuncSetAttribute(kw_cols_adj<kWarpN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWColSmem);
 #define X(N)                                                                                   \
     if (e == cudaSuccess)                                                                      \
         e = cudaFuncSetAttribute(k_cols_fwd<N, float2>,                                        \
@@ -88,9 +97,7 @@ cudaError_t prepare_cols() {
     if (e == cudaSuccess)                                                                      \
         e = cudaFuncSetAttribute(k_cols_adj<N, false, __half2>,                                \
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, ColCfg<N>::SMEM); \
-    if (e == cudaSuccess)                                                                      \
-        e = cudaFuncSetAttribute(k_cols_adj<N, true, float2>,                                  \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, ColCfg<N>::SMEM); \
+    if (e == cudaSuccess) e = prepare_full<N>();                                               \
     if (e == cudaSuccess)                                                                      \
         e = cudaFuncSetAttribute(k_cols_grad_h<N>,                                             \
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, ColCfg<N>::SMEM); \
@@ -179,6 +186,20 @@ cudaError_t cols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long lon
     return cudaErrorInvalidValue;
 }
 
+template <int N, bool FULL, typename HT>
+cudaError_t block_adj(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
+                      long long q_bstride, long long q_kstride) {
+    if constexpr (FULL && !full_block<N>()) {
+        return cudaErrorInvalidValue;
+    } else {
+        k_cols_adj<N, FULL, HT><<<dim3(c.nb, (c.nxh + ColCfg<N>::C - 1) / ColCfg<N>::C, c.split), ColCfg<N>::NT,
+                                  ColCfg<N>::SMEM, s>>>(V, v_bstride, static_cast<const HT*>(c.hh),
+                                                        static_cast<const HT*>(c.hN), c.hscale, c.m, c.box, c.nxh, Q,
+                                                        q_bstride, q_kstride, c.tw);
+        return cudaGetLastError();
+    }
+}
+
 template <bool FULL, typename HT>
 cudaError_t cols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
                      long long q_bstride, long long q_kstride) {
@@ -186,13 +207,8 @@ cudaError_t cols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long lon
     if (c.warp && c.ny == 1024) return ccols_adj<1024, 1, HT>(c, FULL, s, V, v_bstride, Q, q_bstride, q_kstride);
     if (c.warp && c.ny == 2048) return ccols_adj<1024, 2, HT>(c, FULL, s, V, v_bstride, Q, q_bstride, q_kstride);
     switch (c.ny) {
-#define X(N)                                                                                                     \
-    case N:                                                                                                      \
-        k_cols_adj<N, FULL, HT><<<dim3(c.nb, (c.nxh + ColCfg<N>::C - 1) / ColCfg<N>::C, c.split), ColCfg<N>::NT, \
-                                  ColCfg<N>::SMEM, s>>>(V, v_bstride, static_cast<const HT*>(c.hh),              \
-                                                        static_cast<const HT*>(c.hN), c.hscale, c.m, c.box,      \
-                                                        c.nxh, Q, q_bstride, q_kstride, c.tw);                   \
-        return cudaGetLastError();
+#define X(N) \
+    case N: return block_adj<N, FULL, HT>(c, s, V, v_bstride, Q, q_bstride, q_kstride);
         PCE_COL_SIZES(X)
 #undef X
     }
@@ -259,18 +275,18 @@ cudaError_t launch_plain_cols_inv(int ny, dim3 grid, cudaStream_t s, const float
 }
 
 cudaError_t launch_cols_fwd_sep(int ny, dim3 grid, cudaStream_t s, const float2* Z, long long z_bstride,
-                                long long z_kstride, const float2* hhT, const float2* hN, int m,
+                                long long z_kstride, const float2* hhT, const float2* hN,
                                 const Box* box, int nxh, float2* A, long long a_bstride,
                                 const float2* tw1024, int* status, long long wait_limit, int skip_copy,
                                 const SepTerms& sep) {
     if (!tw1024 || !hhT) return cudaErrorInvalidValue;
     if (ny == kWarpN)
-        kw_cols_fwd<float2, true><<<grid, kWColWarps * 32, kWColSmem, s>>>(
-            Z, z_bstride, z_kstride, hhT, hN, nullptr, m, box, nxh, A, a_bstride, tw1024, status, wait_limit,
+        kw_cols_fwd<kWarpN><<<grid, kWColWarps * 32, kWColSmem, s>>>(
+            Z, z_bstride, z_kstride, hhT, hN, box, nxh, A, a_bstride, tw1024, status, wait_limit,
             skip_copy, sep);
     else if (ny == 512)
-        kw_cols_fwd<float2, true, 512><<<grid, kWColWarps * 32, kw_col_smem<512>(), s>>>(
-            Z, z_bstride, z_kstride, hhT, hN, nullptr, m, box, nxh, A, a_bstride, tw1024, status, wait_limit,
+        kw_cols_fwd<512><<<grid, kWColWarps * 32, kw_col_smem<512>(), s>>>(
+            Z, z_bstride, z_kstride, hhT, hN, box, nxh, A, a_bstride, tw1024, status, wait_limit,
             skip_copy, sep);
     else
         return cudaErrorInvalidValue;
@@ -278,18 +294,18 @@ cudaError_t launch_cols_fwd_sep(int ny, dim3 grid, cudaStream_t s, const float2*
 }
 
 cudaError_t launch_cols_adj_sep(int ny, dim3 grid, cudaStream_t s, const float2* V, long long v_bstride,
-                                const float2* hhT, const float2* hN, int m, const Box* box, int nxh,
+                                const float2* hhT, const float2* hN, const Box* box, int nxh,
                                 float2* Q, long long q_bstride, long long q_kstride,
                                 const float2* tw1024, int* status, long long wait_limit, int skip_copy,
                                 const SepTerms& sep) {
     if (!tw1024 || !hhT) return cudaErrorInvalidValue;
     if (ny == kWarpN)
-        kw_cols_adj<false, float2, true><<<grid, kWColWarps * 32, kWColSmem, s>>>(
-            V, v_bstride, hhT, hN, nullptr, m, box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit,
+        kw_cols_adj<kWarpN><<<grid, kWColWarps * 32, kWColSmem, s>>>(
+            V, v_bstride, hhT, hN, box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit,
             skip_copy, sep);
     else if (ny == 512)
-        kw_cols_adj<false, float2, true, 512><<<grid, kWColWarps * 32, kw_col_smem<512>(), s>>>(
-            V, v_bstride, hhT, hN, nullptr, m, box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit,
+        kw_cols_adj<512><<<grid, kWColWarps * 32, kw_col_smem<512>(), s>>>(
+            V, v_bstride, hhT, hN, box, nxh, Q, q_bstride, q_kstride, tw1024, status, wait_limit,
             skip_copy, sep);
     else
         return cudaErrorInvalidValue;

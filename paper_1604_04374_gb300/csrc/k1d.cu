@@ -8,23 +8,6 @@ namespace pce {
 
 #define PCE_1D_SIZES(X) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048) X(4096) X(8192)
 
-int fft1d_threads(int n) {
-    switch (n) {
-#define X(N) case N: return Cfg1d<N>::NT;
-        PCE_1D_SIZES(X)
-#undef X
-    }
-    return 0;
-}
-int fft1d_smem(int n) {
-    switch (n) {
-#define X(N) case N: return Cfg1d<N>::SMEM;
-        PCE_1D_SIZES(X)
-#undef X
-    }
-    return 0;
-}
-
 cudaError_t prepare_cols();
 
 #define PCE_L1_SIZES(X) X(128) X(256) X(512)

@@ -20,10 +20,6 @@ int rows_pairs_per_cta(int nx);
 int rows_grad_pairs_per_cta(int nx);
 // Items (row pairs) handled per CTA of the R2C row kernel.
 int rows_r2c_items_per_cta(int nx);
-// 1D kernels.
-int fft1d_threads(int n);
-int fft1d_smem(int n);
-
 // Raise the dynamic shared-memory limit of every kernel that needs it (once per device).
 cudaError_t prepare_kernels();
 
@@ -132,12 +128,12 @@ cudaError_t launch_sec_c2r(int lc, bool win, dim3 grid, cudaStream_t s, const fl
 // Separable windows, Ny = 1024 or 512 (one-warp column kernels): Z / Q hold
 // one slot per column factor, box[] is indexed by slot.
 cudaError_t launch_cols_fwd_sep(int ny, dim3 grid, cudaStream_t s, const float2* Z, long long z_bstride,
-                                long long z_kstride, const float2* hhT, const float2* hN, int m,
+                                long long z_kstride, const float2* hhT, const float2* hN,
                                 const Box* box, int nxh, float2* A, long long a_bstride,
                                 const float2* tw1024, int* status, long long wait_limit, int skip_copy,
                                 const SepTerms& sep);
 cudaError_t launch_cols_adj_sep(int ny, dim3 grid, cudaStream_t s, const float2* V, long long v_bstride,
-                                const float2* hhT, const float2* hN, int m, const Box* box, int nxh,
+                                const float2* hhT, const float2* hN, const Box* box, int nxh,
                                 float2* Q, long long q_bstride, long long q_kstride,
                                 const float2* tw1024, int* status, long long wait_limit, int skip_copy,
                                 const SepTerms& sep);

@@ -1929,7 +1929,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
                                                            tm_hT, tm_hN, p->d_vbox, nxh, scr.A, ab, p->tw1024,
                                                            p->d_status, p->wait_limit, p->skip_copy, septp);
                     return pce::launch_cols_fwd_sep(ny, cgrid, s, scr.Z, zb, p->zk_s,
-                                                    p->hhT, p->hN, m, p->d_vbox, nxh, scr.A, ab, p->tw1024,
+                                                    p->hhT, p->hN, p->d_vbox, nxh, scr.A, ab, p->tw1024,
                                                     p->d_status, p->wait_limit, p->skip_copy, sept);
                 });
             if (e == cudaSuccess)
@@ -1952,7 +1952,7 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
                                                            tm_hN, p->d_vbox, nxh, scr.Z, zb, p->zk_s, p->tw1024,
                                                            p->d_status, p->wait_limit, p->skip_copy, septp);
                     return pce::launch_cols_adj_sep(ny, cgrid, s, scr.A, ab, p->hhT, p->hN,
-                                                    m, p->d_vbox, nxh, scr.Z, zb, p->zk_s, p->tw1024,
+                                                    p->d_vbox, nxh, scr.Z, zb, p->zk_s, p->tw1024,
                                                     p->d_status, p->wait_limit, p->skip_copy, sept);
                 });
             if (e == cudaSuccess)

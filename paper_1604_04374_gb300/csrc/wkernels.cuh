@@ -125,21 +125,20 @@ __device__ __forceinline__ void warp_split(const float2 (&v)[Q], int lane, int m
     split_dc_nyq(v[m], warp_partner(v, lane, m), A, B);
 }
 
-// F2 for Ny = NY (1024 or 512).  Grid (batch, NXh / 4), 128 threads,
-// kw_col_smem<NY>() bytes.
+// F2 of separable plans for Ny = NY (1024 or 512), column variant 0.  Grid (batch, NXh / 4),
+// 128 threads, kw_col_smem<NY>() bytes.
 // hhT: [m][NXh][NY] (column c's spectrum contiguous; c = 0: DC column),
 // hN: [m][NY] (Nyquist column).
-// SEP = false: Z holds one slot per term (box[k] rows of w_k . u's row spectra).
-// SEP = true: Z holds one slot per column factor (box[] indexed by slot), each
-// term's column is its slot's column times wy_k (row factor) on load, and a
-// slot's tile is loaded once for all of its terms.
-template <typename HT = float2, bool SEP = false, int NY = kWarpN>
+// Z holds one slot per column factor (box[] indexed by slot), each term's column is its
+// slot's column times wy_k (row factor) on load, and a slot's tile is loaded once for
+// all of its terms.
+template <int NY>
 __global__ void __launch_bounds__(kWColWarps * 32, kw_col_min_ctas<NY>())
 kw_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstride,
-            const HT* __restrict__ hhT, const HT* __restrict__ hN, const float* __restrict__ hscale, int m,
+            const float2* __restrict__ hhT, const float2* __restrict__ hN,
             const Box* __restrict__ box, int NXh, float2* __restrict__ A, long long a_bstride,
             const float2* __restrict__ tw, int* __restrict__ status, long long wait_limit, int skip_copy,
-            SepTerms sep = SepTerms{}) {
+            SepTerms sep) {
     constexpr int QN = NY / 32;   // values per lane
     extern __shared__ float2 smem[];
     float2* tile = smem;
@@ -161,56 +160,37 @@ kw_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     float2 acc[QN];
 #pragma unroll
     for (int i = 0; i < QN; ++i) acc[i] = make_float2(0.f, 0.f);
-    // the sequence of terms: general, every term with a nonempty box in index
-    // order (slot = term); separable, sep.korder (slot = sep.kslot[term])
-    const int tend = SEP ? sep.nterms : m;
-    auto next_t = [&](int t) {
-        if constexpr (!SEP) {
-            while (t < m && box[t].nr == 0) ++t;
-        }
-        return t;
-    };
-    auto kof = [&](int t) { return SEP ? __ldg(&sep.korder[t]) : t; };
-    auto slot_of = [&](int kk) { return SEP ? __ldg(&sep.kslot[kk]) : kk; };
-    // SEP: row factors of term t in buffer (t & 1), prefetched one term ahead
+    // the sequence of terms: sep.korder, term k in slot sep.kslot[k]
+    const int tend = sep.nterms;
+    auto kof = [&](int t) { return __ldg(&sep.korder[t]); };
+    auto slot_of = [&](int kk) { return __ldg(&sep.kslot[kk]); };
+    // row factors of term t in buffer (t & 1), prefetched one term ahead
     float* wys = reinterpret_cast<float*>(smem + (NY + fft_tile<NY>()) * kWColWarps);
-    int t = next_t(0);
-    int cur_slot = -1;
+    int t = 0;
     if (t < tend) {
         const int s0 = slot_of(kof(t));
-        if constexpr (SEP) wy_load<NY>(wys, sep.wrow, kof(t));
+        wy_load<NY>(wys, sep.wrow, kof(t));
         tile_load(tile, Zb + s0 * z_kstride, box[s0].nr, NXh, col0);
     }
     while (t < tend) {
         const int k = kof(t);
         const int sl = slot_of(k);
-        const int tn = next_t(t + 1);
+        const int tn = t + 1;
         const int sn = tn < tend ? slot_of(kof(tn)) : -1;
         const Box bx = box[sl];
-        if (SEP || sl != cur_slot) {   // uniform over the CTA
-            cp_async_wait_all();
-            __syncthreads();
-            cur_slot = sl;
-        }
+        cp_async_wait_all();
+        __syncthreads();
         float2 v[QN];
-        if constexpr (SEP) {
-            const float* wr = wys + (t & 1) * NY;
-            if (bx.r0 == 0 && bx.nr == NY) {   // uniform: the slot holds every row in place
-                const float2* tb = tile + 4 * lane + tix_sw(lane, warp);
+        const float* wr = wys + (t & 1) * NY;
+        if (bx.r0 == 0 && bx.nr == NY) {   // uniform: the slot holds every row in place
+            const float2* tb = tile + 4 * lane + tix_sw(lane, warp);
 #pragma unroll
-                for (int q = 0; q < QN; ++q) v[q] = cscale(tb[128 * q], wr[lane + 32 * q]);
-            } else {
-#pragma unroll
-                for (int q = 0; q < QN; ++q) {
-                    const int i = wrap(lane + 32 * q - bx.r0, NY);
-                    v[q] = (i < bx.nr) ? cscale(tile[tix(i, warp)], wr[lane + 32 * q]) : make_float2(0.f, 0.f);
-                }
-            }
+            for (int q = 0; q < QN; ++q) v[q] = cscale(tb[128 * q], wr[lane + 32 * q]);
         } else {
 #pragma unroll
             for (int q = 0; q < QN; ++q) {
                 const int i = wrap(lane + 32 * q - bx.r0, NY);
-                v[q] = (i < bx.nr) ? tile[tix(i, warp)] : make_float2(0.f, 0.f);
+                v[q] = (i < bx.nr) ? cscale(tile[tix(i, warp)], wr[lane + 32 * q]) : make_float2(0.f, 0.f);
             }
         }
         if (tn < tend && sn != sl) {   // the next term needs another slot: reload the tile
@@ -220,10 +200,9 @@ kw_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
         // this column's spectrum of term k arrives in the warp's transpose
         // tile while the FFT finishes
         const bool bulk = !dcn && cv && !failed;
-        const float sk = hscale_of<HT>(hscale, k);
         warp_fft<NY, false>(v, tr, tw, [&] {
             if (bulk && lane == 0)
-                bulk_load(tr, hhT + ((long long)k * NXh + col) * NY, NY * sizeof(HT), bar, skip_copy);
+                bulk_load(tr, hhT + ((long long)k * NXh + col) * NY, NY * sizeof(float2), bar, skip_copy);
         });
         if (bulk) {
             if (!mbar_wait(bar, parity, wait_limit)) {
@@ -237,30 +216,27 @@ kw_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
             parity ^= 1;
         }
         if (dcn) {
-            const HT* h0 = hhT + (long long)k * NXh * NY;
-            const HT* hn = hN + (long long)k * NY;
+            const float2* h0 = hhT + (long long)k * NXh * NY;
+            const float2* hn = hN + (long long)k * NY;
 #pragma unroll
             for (int mm = 0; mm < QN; ++mm) {
                 const int f = lane + 32 * mm;
                 float2 a, bb;
                 warp_split(v, lane, mm, a, bb);
-                acc[mm] = cfma(ldh(&h0[f], sk), a, acc[mm]);
-                const float2 t = cmul(ldh(&hn[f], sk), bb);
+                acc[mm] = cfma(__ldg(&h0[f]), a, acc[mm]);
+                const float2 t = cmul(__ldg(&hn[f]), bb);
                 acc[mm].x -= t.y;
                 acc[mm].y += t.x;
             }
         } else if (cv && !failed) {
-            const HT* th = reinterpret_cast<const HT*>(tr);
 #pragma unroll
-            for (int mm = 0; mm < QN; ++mm) acc[mm] = cfma(lds_h(&th[lane + 32 * mm], sk), v[mm], acc[mm]);
+            for (int mm = 0; mm < QN; ++mm) acc[mm] = cfma(tr[lane + 32 * mm], v[mm], acc[mm]);
         }
-        if constexpr (SEP) {
-            // next term's row factors into the other buffer, last read in the
-            // previous term (before this term's barrier)
-            if (tn < tend) {
-                wy_load<NY>(wys + ((t + 1) & 1) * NY, sep.wrow, kof(tn));
-                cp_async_commit();
-            }
+        // next term's row factors into the other buffer, last read in the
+        // previous term (before this term's barrier)
+        if (tn < tend) {
+            wy_load<NY>(wys + ((t + 1) & 1) * NY, sep.wrow, kof(tn));
+            cp_async_commit();
         }
         t = tn;
     }
@@ -289,21 +265,19 @@ __device__ __forceinline__ void sep_share(const SepTerms& sep, int& tbeg, int& t
     }
 }
 
-// G1b + G2 for Ny = NY (1024 or 512; FULL: every row of Q, for the window
-// gradient).
-// Grid (batch, NXh / 4, split): CTA z of a column tile takes its share of the terms
-// (SEP: of the slots) and forms the FFT of V itself.
-// SEP: Q receives one slot per column factor: S_j = sum over the slot's terms of
+// G1b + G2 of separable plans for Ny = NY (1024 or 512), column variant 0.
+// Grid (batch, NXh / 4, split): CTA z of a column tile takes its share of the slots and
+// forms the FFT of V itself.  Q receives one slot per column factor: S_j = sum over the slot's terms of
 // wy_k . IFFT_y(conj(hhat_k) V), on the slot box rows (box[] indexed by slot),
 // accumulated in the shared tile and stored once per slot.
-template <bool FULL, typename HT = float2, bool SEP = false, int NY = kWarpN>
+template <int NY>
 __global__ void __launch_bounds__(kWColWarps * 32, kw_col_min_ctas<NY>())
 kw_cols_adj(const float2* __restrict__ V, long long v_bstride,
-            const HT* __restrict__ hhT, const HT* __restrict__ hN, const float* __restrict__ hscale, int m,
+            const float2* __restrict__ hhT, const float2* __restrict__ hN,
             const Box* __restrict__ box, int NXh,
             float2* __restrict__ Q, long long q_bstride, long long q_kstride,
             const float2* __restrict__ tw, int* __restrict__ status, long long wait_limit, int skip_copy,
-            SepTerms sep = SepTerms{}) {
+            SepTerms sep) {
     constexpr int QN = NY / 32;   // values per lane
     extern __shared__ float2 smem[];
     float2* tile = smem;
@@ -323,45 +297,32 @@ kw_cols_adj(const float2* __restrict__ V, long long v_bstride,
     const bool use_bulk = !dcn && cv;
     // the sequence of terms (see kw_cols_fwd)
     int tbeg, tend;
-    if constexpr (SEP) {
-        sep_share(sep, tbeg, tend);
-    } else {
-        tbeg = share_beg(m, blockIdx.z, gridDim.z);
-        tend = share_beg(m, blockIdx.z + 1, gridDim.z);
-    }
-    auto next_t = [&](int t) {
-        if constexpr (!SEP) {
-            while (t < tend && !FULL && box[t].nr == 0) ++t;
-        }
-        return t;
-    };
-    auto kof = [&](int t) { return SEP ? __ldg(&sep.korder[t]) : t; };
-    auto slot_of = [&](int kk) { return SEP ? __ldg(&sep.kslot[kk]) : kk; };
+    sep_share(sep, tbeg, tend);
+    auto kof = [&](int t) { return __ldg(&sep.korder[t]); };
+    auto slot_of = [&](int kk) { return __ldg(&sep.kslot[kk]); };
 
-    // SEP: row factors of the t-th term in buffer (t & 1), prefetched one term ahead
+    // row factors of the t-th term in buffer (t & 1), prefetched one term ahead
     float* wys = reinterpret_cast<float*>(smem + (NY + fft_tile<NY>()) * kWColWarps);
-    if constexpr (SEP) {
-        if (tbeg < tend) wy_load<NY>(wys + (tbeg & 1) * NY, sep.wrow, __ldg(&sep.korder[tbeg]));
-    }
+    if (tbeg < tend) wy_load<NY>(wys + (tbeg & 1) * NY, sep.wrow, __ldg(&sep.korder[tbeg]));
     tile_load(tile, V + b * v_bstride, NY, NXh, col0);
     cp_async_wait_all();
     __syncthreads();
     float2 vv[QN];
 #pragma unroll
     for (int q = 0; q < QN; ++q) vv[q] = tile[4 * (lane + 32 * q) + tix_sw(lane, warp)];
-    int t = next_t(tbeg);
+    int t = tbeg;
     int prev_slot = -1;
     // the spectrum of the first term arrives while the FFT of V finishes
-    warp_fft<NY, false, SEP>(vv, tr, tw, [&] {
+    warp_fft<NY, false>(vv, tr, tw, [&] {
         if (use_bulk && t < tend && lane == 0)
-            bulk_load(tr, hhT + ((long long)kof(t) * NXh + col) * NY, NY * sizeof(HT), bar, skip_copy);
+            bulk_load(tr, hhT + ((long long)kof(t) * NXh + col) * NY, NY * sizeof(float2), bar, skip_copy);
     });
     while (t < tend) {
         const int k = kof(t);
         const int sl = slot_of(k);
         const Box bx = box[sl];
-        const int tn = next_t(t + 1);
-        const int kn = tn < tend ? kof(tn) : m;
+        const int tn = t + 1;
+        const int kn = tn < tend ? kof(tn) : -1;
         const bool first = sl != prev_slot;
         const bool last = tn >= tend || slot_of(kn) != sl;
         prev_slot = sl;
@@ -377,73 +338,56 @@ kw_cols_adj(const float2* __restrict__ V, long long v_bstride,
             parity ^= 1;
         }
         float2 p[QN];
-        const float sk = hscale_of<HT>(hscale, k);
         if (dcn) {
-            const HT* h0 = hhT + (long long)k * NXh * NY;
-            const HT* hn = hN + (long long)k * NY;
+            const float2* h0 = hhT + (long long)k * NXh * NY;
+            const float2* hn = hN + (long long)k * NY;
 #pragma unroll
             for (int mm = 0; mm < QN; ++mm) {
                 const int f = lane + 32 * mm;
                 float2 a, bb;
                 warp_split(vv, lane, mm, a, bb);
-                float2 t = cmulc(a, ldh(&h0[f], sk));
-                const float2 s = cmulc(bb, ldh(&hn[f], sk));
+                float2 t = cmulc(a, __ldg(&h0[f]));
+                const float2 s = cmulc(bb, __ldg(&hn[f]));
                 t.x -= s.y;
                 t.y += s.x;
                 p[mm] = t;
             }
         } else {
-            const HT* th = reinterpret_cast<const HT*>(tr);
 #pragma unroll
             for (int mm = 0; mm < QN; ++mm)
-                p[mm] = (use_bulk && !failed) ? cmulc(vv[mm], lds_h(&th[lane + 32 * mm], sk))
-                                              : make_float2(0.f, 0.f);
+                p[mm] = (use_bulk && !failed) ? cmulc(vv[mm], tr[lane + 32 * mm]) : make_float2(0.f, 0.f);
         }
         // the next term's spectrum arrives while this inverse FFT finishes
         const bool issue = use_bulk && !failed && tn < tend;
-        warp_fft<NY, true, SEP>(p, tr, tw, [&] {
+        warp_fft<NY, true>(p, tr, tw, [&] {
             if (issue && lane == 0)
-                bulk_load(tr, hhT + ((long long)kn * NXh + col) * NY, NY * sizeof(HT), bar, skip_copy);
+                bulk_load(tr, hhT + ((long long)kn * NXh + col) * NY, NY * sizeof(float2), bar, skip_copy);
         });
-        if constexpr (SEP) {
-            // accumulate wy_k . p into this warp's column of the tile; the previous
-            // slot's store must have finished reading the tile, and this term's
-            // row factors must have landed
-            cp_async_wait_all();
-            __syncthreads();
-            if (tn < tend) {   // the other buffer was last read in the previous term
-                wy_load<NY>(wys + ((t + 1) & 1) * NY, sep.wrow, kn);
-                cp_async_commit();
-            }
-            const float* wr = wys + (t & 1) * NY;
-            float2* col = tile + tix_sw(lane, warp) + 4 * lane;
-            if (first) {
+        // accumulate wy_k . p into this warp's column of the tile; the previous
+        // slot's store must have finished reading the tile, and this term's
+        // row factors must have landed
+        cp_async_wait_all();
+        __syncthreads();
+        if (tn < tend) {   // the other buffer was last read in the previous term
+            wy_load<NY>(wys + ((t + 1) & 1) * NY, sep.wrow, kn);
+            cp_async_commit();
+        }
+        const float* wr = wys + (t & 1) * NY;
+        float2* col = tile + tix_sw(lane, warp) + 4 * lane;
+        if (first) {
 #pragma unroll
-                for (int mm = 0; mm < QN; ++mm) col[128 * mm] = cscale(p[mm], wr[lane + 32 * mm]);
-            } else {
-#pragma unroll
-                for (int mm = 0; mm < QN; ++mm) col[128 * mm] = cadd(col[128 * mm], cscale(p[mm], wr[lane + 32 * mm]));
-            }
-            if (last) {
-                __syncthreads();
-                float2* Qs = Q + b * q_bstride + sl * q_kstride;
-                for (int e = threadIdx.x; e < bx.nr * kWColWarps; e += kWColWarps * 32) {
-                    const int i = e >> 2, c = e & 3;
-                    const int g = wrap(bx.r0 + i, NY);
-                    if (col0 + c < NXh) Qs[(long long)i * NXh + col0 + c] = tile[tix(g, c)];
-                }
-            }
+            for (int mm = 0; mm < QN; ++mm) col[128 * mm] = cscale(p[mm], wr[lane + 32 * mm]);
         } else {
-            __syncthreads();
 #pragma unroll
-            for (int mm = 0; mm < QN; ++mm) tile[4 * (lane + 32 * mm) + tix_sw(lane, warp)] = p[mm];
+            for (int mm = 0; mm < QN; ++mm) col[128 * mm] = cadd(col[128 * mm], cscale(p[mm], wr[lane + 32 * mm]));
+        }
+        if (last) {
             __syncthreads();
-            float2* Qk = Q + b * q_bstride + k * q_kstride;
-            const int rows = FULL ? NY : bx.nr;
-            for (int e = threadIdx.x; e < rows * kWColWarps; e += kWColWarps * 32) {
+            float2* Qs = Q + b * q_bstride + sl * q_kstride;
+            for (int e = threadIdx.x; e < bx.nr * kWColWarps; e += kWColWarps * 32) {
                 const int i = e >> 2, c = e & 3;
-                const int g = FULL ? i : wrap(bx.r0 + i, NY);
-                if (col0 + c < NXh) Qk[(long long)i * NXh + col0 + c] = tile[tix(g, c)];
+                const int g = wrap(bx.r0 + i, NY);
+                if (col0 + c < NXh) Qs[(long long)i * NXh + col0 + c] = tile[tix(g, c)];
             }
         }
         t = tn;
