@@ -1848,11 +1848,11 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
     const int col_units = adjoint ? (sepx ? p->nslots : m) : (sepx ? p->nterms : m);
     const int col_most = scr.beside ? 1
                          : adjoint  ? pce::kMaxCluster
-                         : !sepx    ? pce::cols_fwd_max_split(ny)
-                         : septm && !prune ? pce::kMinSplit
+                         : !sepx    ? (pce::cols_fwd_split_pays(ny, m) ? pce::kDenseSplit : 1)
+                         : septm && !prune ? pce::kSepSplit
                                            : 1;
-    // two CTAs a tile don't repay the exchange: 256^2, m = 16, 8 right-hand sides 41 -> 51 us
-    const int col_least = adjoint ? 1 : pce::kMinSplit;
+    // the forward's exchange repays the most CTAs a tile or none
+    const int col_least = adjoint ? 1 : col_most;
     for (long long b0 = 0; b0 < batch && e == cudaSuccess; b0 += bal) {
         const int nb = (int)std::min<long long>(bal, batch - b0);
         const float* src = in + b0 * P;
