@@ -204,7 +204,7 @@ kc_cols_fwd(const float2* __restrict__ Z, long long z_bstride, long long z_kstri
     const int kend = m;
     // The terms with a nonempty box in order.  512 points in reduced storage, the shortest chain
     // a term: 32 boxes looked at at a time, and the next term's box and scale read before
-    // this one's rows are waited for (512 x 64, m = 9, forward apply 47.1 -> 41.0 us).  The
+    // this one's rows are waited for (512 x 64, m = 9, forward apply 45.2 -> 41.0 us).  The
     // longer chains lose by it (2048 x 256, m = 16, 4 right-hand sides 154 -> 174 us).
     constexpr bool kAhead = NF == 512 && sizeof(HT) != sizeof(float2);
     int kb = -32;

@@ -14,9 +14,9 @@
 // collects the sums, runs the inverse transform and stores.
 // What bounds them is latency: the chain of a round's reads, FFT and exchange.  Whole
 // forward applies, m = 16, one right-hand side: 1024^2 separable 93 -> 81 us (unsplit ->
-// split); 512^2 separable 52 -> 39; 256^2 dense 33 -> 27; 64^2 dense 31 -> 23.  Eight CTAs for dense
-// plans, four for separable ones: fewer repeat the exchange (256^2 dense, 8 right-hand
-// sides, two CTAs 41 -> 51 us; 1024^2 separable, 2 right-hand sides, two CTAs 129 -> 160).
+// split); 512^2 separable 52 -> 39; 256^2 dense 33 -> 27; 64^2 dense 31 -> 23.  Four CTAs at
+// least: two repeat the exchange for half the rounds (256^2 dense, 8 right-hand sides 41 ->
+// 51 us; 1024^2 separable, 2 right-hand sides 129 -> 160).
 #include "kernels.cuh"
 #include "tkernels.cuh"
 #include "ckernels.cuh"
@@ -260,27 +260,42 @@ kt_cols_fwd_split(const float2* __restrict__ Z, long long z_bstride, long long z
 
 #define PCE_SPLIT_SIZES(X) X(16) X(32) X(64) X(128) X(256)
 
-template <int NY, typename HT>
+template <int NY, int S, typename HT>
 cudaError_t split_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride, long long z_kstride,
                       float2* A, long long a_bstride) {
-    constexpr int S = kDenseSplit;
-    if (c.split != S) return cudaErrorInvalidValue;
     return launch_cluster(k_cols_fwd_split<NY, S, HT>, dim3(c.nb, (c.nxh + ColCfg<NY>::C - 1) / ColCfg<NY>::C, S),
                           dim3(1, 1, S), ColCfg<NY>::NT, split_smem<NY>(), s, Z, z_bstride, z_kstride,
                           static_cast<const HT*>(c.hh), static_cast<const HT*>(c.hN), c.hscale, c.m, c.box, c.nxh, A,
                           a_bstride, c.tw);
 }
 
+template <int NY, typename HT>
+cudaError_t split_fwd_of(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride, long long z_kstride,
+                         float2* A, long long a_bstride) {
+    switch (c.split) {
+        case 4: return split_fwd<NY, 4, HT>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
+        case 8: return split_fwd<NY, 8, HT>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
+    }
+    return cudaErrorInvalidValue;
+}
+
 }  // namespace
 
-// A round of a cluster of eight costs what four to five terms cost one CTA after another
-// (256^2, one right-hand side: 5.3 against 1.2 us), so the rounds have to be three quarters
-// full: 8 terms 23.6 -> 21.4 us, 16 terms 32.8 -> 26.7, but 9 terms 24.6 -> 24.7.  Clusters of
-// four never repaid it (256^2: one right-hand side, 5 terms 20.5 -> 24.6 us; 4 right-hand
-// sides, 16 terms 32.8 -> 34.6, 9 terms 24.6 -> 31.8).
-bool cols_fwd_split_pays(int ny, int m) {
-    const int rounds = (m + kDenseSplit - 1) / kDenseSplit;
-    return ny <= 256 && 4 * m >= 3 * kDenseSplit * rounds;
+// Eight CTAs a tile, else four, while all are resident at once (four an SM), and only where they
+// repay the exchange: the rounds three quarters full (256^2, one right-hand side, in rounds
+// of eight: 8 terms 23.6 -> 20.6 us, 16 terms 32.8 -> 26.7, but 9 terms 24.6 -> 24.7), and four
+// CTAs where the chain is long: columns of 256 points from 28 terms on (4 right-hand sides: 16
+// terms 32.8 -> 34.6, 28 terms 47.2 -> 45.6, 64 terms 94.1 -> 85.8), of 64 points from 40 on
+// (64 x 2048, 2 right-hand sides: 32 terms 57.6 -> 59.0, 48 terms 77.0 -> 75.4), of the
+// other lengths, whose terms take longer one after another, from 8 on (128 x 256, 8 right-hand
+// sides: 8 terms 28.7 -> 25.1, 32 terms 73.7 -> 54.9).
+int cols_fwd_split(int ny, int m, long long ctas) {
+    if (ny > 256) return 1;
+    for (int n : {8, 4}) {
+        const int rounds = (m + n - 1) / n, least = n == 8 ? 8 : ny == 256 ? 28 : ny == 64 ? 40 : 8;
+        if (m >= least && 4 * m >= 3 * n * rounds && ctas * n <= 4LL * kSms) return n;
+    }
+    return 1;
 }
 
 cudaError_t launch_cols_fwd_split(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride,
@@ -288,8 +303,8 @@ cudaError_t launch_cols_fwd_split(const ColArgs& c, cudaStream_t s, const float2
     switch (c.ny) {
 #define X(N)                                                                                                    \
     case N:                                                                                                     \
-        return c.lowp ? split_fwd<N, __half2>(c, s, Z, z_bstride, z_kstride, A, a_bstride)                   \
-                      : split_fwd<N, float2>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
+        return c.lowp ? split_fwd_of<N, __half2>(c, s, Z, z_bstride, z_kstride, A, a_bstride)                   \
+                      : split_fwd_of<N, float2>(c, s, Z, z_bstride, z_kstride, A, a_bstride);
         PCE_SPLIT_SIZES(X)
 #undef X
     }

@@ -278,7 +278,9 @@ bool wide_1d(int batch, int m) {
 // that one CTA would run one after another (an SM each), doubled while the batch
 // leaves SMs for them and a CTA has more than one round.  (Three rounds take four CTAs, one
 // of them idle: one round long, where two CTAs would run two.)  N = 8192, m = 32, three
-// right-hand sides, adjoint: 94.7 -> 28.9 us (three clusters of eight).
+// right-hand sides, adjoint: 94.7 -> 28.9 us (three clusters of eight).  In the lanes of a
+// batch too, where other tasks could use the SMs: 64 tasks of N = 8192, m = 32 on 16 lanes
+// 408 -> 142 us, 256 of N = 4096 552 -> 259, 256 of all sizes 2769 -> 2800.
 int cluster_1d(int batch, int rounds) {
     int cl = 1;
     while (cl < kMaxCluster && cl < rounds && (long long)batch * 2 * cl <= kSms) cl *= 2;

@@ -287,8 +287,8 @@ k4_cols_adj(const float2* __restrict__ Q, int npairs, const float* __restrict__ 
 // CTAs of several row pairs use a few SMs (33 CTAs at N = 65536, one right-hand side).
 // The kernels below take one row pair a CTA and a pair's loads ahead of the FFT before it, in
 // registers that the packed kernels rather spend on more warps; the same operations in
-// the same order.  m = 16, one right-hand side: N = 65536 forward 30.9 -> 24.9 us (row
-// kernel 14.0 -> 8.7), adjoint 45.3 -> 25 to 27; N = 16384 forward 25 -> 23.5, adjoint 39 -> 22.5.
+// the same order.  m = 16, one right-hand side: N = 65536 forward 30.8 -> 24.6 us (row
+// kernel 14.0 -> 8.7), adjoint 45.1 -> 24.6; N = 16384 forward 24.6 -> 22.6, adjoint 39.0 -> 19.1.
 template <int NX>
 struct L1Few {
     static constexpr int T = NX / kR;

@@ -255,7 +255,8 @@ k_rows_r2c_pairs(const float* __restrict__ src, long long src_bstride, int nrows
     const bool pv = p < npairs;
     const int ga = 2 * p, gb = ga + 1;
     const bool hb = pv && gb < nrows;
-    // uniform trip count over the CTA's row pairs (the FFT has CTA barriers)
+    // uniform trip count over the CTA's row pairs (the FFT's barriers are of the whole CTA or
+    // warp)
     int nk = 0;
     for (int s2 = 0; s2 < FPC; ++s2) {
         const int ps = blockIdx.x * FPC + s2;

@@ -61,8 +61,8 @@ cudaError_t launch_wrows_c2r(int nx, int nb, cudaStream_t s, const float2* src, 
 // Nyquist column hN, hN2 split by parity for ny = 2048; half2 with hscale when lowp),
 // twiddles, the plan's status word.  warp: the one-warp column kernels where they
 // exist (ny = 512, 1024, 2048), else block Stockham.  frame_rows: col_frame_rows(), tab
-// the phased twiddles.  split: CTAs that share a column tile's terms (forward: 1 or
-// kDenseSplit).
+// the phased twiddles.  split: CTAs that share a column tile's terms (forward:
+// cols_fwd_split()).
 struct ColArgs {
     int ny = 0, nxh = 0, nb = 1, m = 0;
     unsigned split = 1;
@@ -87,10 +87,11 @@ cudaError_t launch_cols_fwd(const ColArgs& c, cudaStream_t s, const float2* Z, l
                             long long z_kstride, float2* A, long long a_bstride);
 cudaError_t launch_cols_adj(const ColArgs& c, cudaStream_t s, const float2* V, long long v_bstride, float2* Q,
                             long long q_bstride, long long q_kstride);
-// The forward over clusters of CTAs (colsplit.cu): dense plans of up to 256 rows kDenseSplit
-// (c.split) where cols_fwd_split_pays, separable ones with tensor-memory columns kSepSplit (grid.z).
-constexpr int kDenseSplit = 8, kSepSplit = 4;
-bool cols_fwd_split_pays(int ny, int m);
+// The forward over clusters of CTAs (colsplit.cu): dense plans cols_fwd_split() (c.split; 8, 4
+// or none) for a grid of ctas column CTAs, separable ones with tensor-memory columns kSepSplit
+// (grid.z).
+constexpr int kSepSplit = 4;
+int cols_fwd_split(int ny, int m, long long ctas);
 cudaError_t launch_cols_fwd_split(const ColArgs& c, cudaStream_t s, const float2* Z, long long z_bstride,
                                   long long z_kstride, float2* A, long long a_bstride);
 cudaError_t launch_cols_fwd_sep_split(int ny, dim3 grid, cudaStream_t s, const float2* Z, long long z_bstride,

@@ -1076,7 +1076,8 @@ pce_status create_common(pce_plan_t* out, int ndims, const int64_t* shape, int m
     // untuned row variant: the adjoint rows without register prefetch.  128 x 512, m = 6,
     // 24 right-hand sides 68.8 -> 65.4 us; 256-task uneven batch 3.20 -> 2.91 ms with the
     // separable default below.  Variant 2 (forward rows by row pairs) loses on small grids
-    // (256^2, one right-hand side: 20.5 -> 28.7 us) and stays the autotuner's to pick.
+    // (256^2, m = 16, one right-hand side, forward 27.0 -> 35.2 us) and stays the autotuner's
+    // to pick.
     if (ndims == 2) p->row_variant = 1;
     *out = p;
     return PCE_OK;
@@ -1225,7 +1226,7 @@ pce_status setup_separable(pce_plan* p, const float* wy, const float* wx, cudaSt
     p->sep = true;
     p->sep_prune = prune;
     // untuned column variant: the warp state in tensor memory (1024^2, m = 16, one
-    // right-hand side, both directions: 222 us with it in registers, 132 us so)
+    // right-hand side, both directions: 265 us with it in registers, 148 us so)
     p->col_variant = 2;
     return PCE_OK;
 }
@@ -1687,7 +1688,8 @@ pce::ColArgs col_args(const pce_plan* p, int nb, bool warp, bool lowp, unsigned 
 // FFT of V a CTA (adjoint), the exchange within the cluster (forward).  The same bits for
 // any split: every unit's result is formed by one CTA (adjoint), the terms are added in
 // order (forward, colsplit.cu).
-// 1024^2 separable, m = 16, one right-hand side, forward and adjoint: 223 -> 180 us.
+// 1024^2 separable, m = 16, one right-hand side: forward 93 -> 81 us; adjoint of column
+// variant 2 69 us, of which the column kernel takes 42 with eight CTAs a tile.
 int col_split(long long ctas, int per_sm, int units, int least, int most) {
     int n = 1;
     while (n < most && 2 * n <= units && ctas * 2 * n <= (long long)pce::kSms * per_sm) n *= 2;
@@ -1846,19 +1848,16 @@ pce_status apply_impl(pce_plan_t p, const float* in, float* out, int64_t batch, 
     // share it: one in a batch's lane, where other tasks could use the SM
     const int col_ctas = !warp ? pce::cols_ctas_per_sm(ny) : ny == 512 ? 6 : ny == 2048 ? 2 : 4;
     const int col_units = adjoint ? (sepx ? p->nslots : m) : (sepx ? p->nterms : m);
-    const int col_most = scr.beside ? 1
-                         : adjoint  ? pce::kMaxCluster
-                         : !sepx    ? (pce::cols_fwd_split_pays(ny, m) ? pce::kDenseSplit : 1)
-                         : septm && !prune ? pce::kSepSplit
-                                           : 1;
-    // the forward's exchange repays the most CTAs a tile or none
-    const int col_least = adjoint ? 1 : col_most;
+    const int col_most = scr.beside ? 1 : adjoint ? pce::kMaxCluster : septm && !prune ? pce::kSepSplit : 1;
+    const int col_least = adjoint ? 1 : col_most;   // fewer don't repay the forward's exchange
     for (long long b0 = 0; b0 < batch && e == cudaSuccess; b0 += bal) {
         const int nb = (int)std::min<long long>(bal, batch - b0);
         const float* src = in + b0 * P;
         float* dst = out + b0 * P;
         dim3 cgrid(nb, (nxh + cpc - 1) / cpc);
-        if (!slotwise) cgrid.z = col_split((long long)cgrid.x * cgrid.y, col_ctas, col_units, col_least, col_most);
+        const long long ctas = (long long)cgrid.x * cgrid.y;
+        if (!adjoint && !sepx) cgrid.z = scr.beside ? 1 : pce::cols_fwd_split(ny, m, ctas);
+        else if (!slotwise) cgrid.z = col_split(ctas, col_ctas, col_units, col_least, col_most);
         if (slotwise && !adjoint) {
             for (size_t a = 0; a < active.size() && e == cudaSuccess; ++a) {
                 const int j = active[a];
@@ -2334,8 +2333,8 @@ extern "C" pce_status pce_backward(pce_plan_t p, const float* u, const float* r,
 // ---------------------------------------------------------------------------
 // Forward apply without any allocation (no counterpart in the paper).
 //
-// pce_apply runs the 2D passes on intermediates that the plan allocated with
-// cudaMalloc.  pce_apply_noalloc runs the same three kernels on intermediates
+// pce_apply runs the 2D passes on intermediates that the plan allocated.
+// pce_apply_noalloc runs the same three kernels on intermediates
 // held in g_noalloc_scratch, a fixed array of device memory that exists as
 // soon as the library is loaded on a device, so the call itself never
 // allocates.  Host code may not pass g_noalloc_scratch to a kernel directly:

@@ -130,17 +130,20 @@ def test_2d_forward_splits_keep_the_bits(torch_cuda, ny, nx, gy, gx, zero):
 def forward_split(ny, nx, nb, units, sep):
     """CTAs that share a column tile's terms in a forward launch of nb right-hand sides."""
     cols = 4 if sep or ny >= 256 else 128 // (ny // 8)
-    ctas, per_sm, most = nb * -(-(nx // 2) // cols), 6 if ny == 512 else 4, 4 if sep else 8
-    if not sep and 4 * units < 3 * most * -(-units // most):
-        return 1
-    return most if most <= units and ctas * most <= 152 * per_sm else 1
+    ctas = nb * -(-(nx // 2) // cols)
+    if sep:
+        return 4 if units >= 4 and ctas * 4 <= 152 * (6 if ny == 512 else 4) else 1
+    for n, least in ((8, 8), (4, {256: 28, 64: 40}.get(ny, 8))):
+        if units >= least and 4 * units >= 3 * n * -(-units // n) and ctas * n <= 152 * 4:
+            return n
+    return 1
 
 
-@pytest.mark.parametrize("ny,nx,gy,gx,zero", [(16, 512, 2, 4, ()), (32, 256, 3, 4, (9,)), (64, 128, 4, 4, (0, 1)),
-                                              (128, 64, 5, 4, (4,)), (256, 32, 4, 4, ()), (512, 64, 3, 3, (0,)),
+@pytest.mark.parametrize("ny,nx,gy,gx,zero", [(16, 512, 2, 4, ()), (32, 256, 3, 4, (9,)), (64, 128, 8, 5, (0, 1)),
+                                              (128, 64, 5, 4, (4,)), (256, 32, 4, 8, ()), (512, 64, 3, 3, (0,)),
                                               (1024, 64, 2, 3, ())])
 def test_2d_forward_split_and_unsplit_launches_agree(torch_cuda, ny, nx, gy, gx, zero):
-    """Launches of 64, 19 and 1 right-hand sides, which take one, eight and eight CTAs a tile
+    """Launches of 64, 30 and 1 right-hand sides, which take one, four and eight CTAs a tile
     (separable columns one and four), give the same bits."""
     torch = torch_cuda
     from paper_1604_04374_gb300 import Plan, pce
@@ -148,9 +151,9 @@ def test_2d_forward_split_and_unsplit_launches_agree(torch_cuda, ny, nx, gy, gx,
     w = (wy[:, :, None] * wx[:, None, :]).astype(np.float32)
     ud, hd = dev(torch, u), dev(torch, h)
     sep = ny >= 512
-    few = (1,) if sep else (19, 1)
+    few = (1,) if sep else (30, 1)
     terms = gy * gx - (len(zero) if sep else 0)
-    assert [forward_split(ny, nx, nb, terms, sep) for nb in (64, *few)] == ([1, 4] if sep else [1, 8, 8])
+    assert [forward_split(ny, nx, nb, terms, sep) for nb in (64, *few)] == ([1, 4] if sep else [1, 4, 8])
     plans = ([Plan(wy=dev(torch, wy), wx=dev(torch, wx), h=hd)] if sep else
              [Plan(dev(torch, w), h=hd), Plan(dev(torch, w), h=hd, flags=pce.PCE_FLAG_LOWP_STORAGE)])
     for plan in plans:

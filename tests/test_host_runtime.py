@@ -218,16 +218,19 @@ def test_column_splits_stay_within_one_wave(child, shape):
 
 
 def test_dense_forward_splits_where_its_rounds_are_full(child):
-    """256 x 256: eight CTAs share a column tile's terms where the rounds of eight are three
-    quarters full and all CTAs are resident at once, none otherwise."""
+    """Eight or four CTAs share a column tile's terms where the rounds are three quarters full,
+    the chain is long enough for the length and all CTAs are resident at once, none otherwise."""
     child("""
-    for m, batch, split in ((4, 1, 1), (5, 1, 1), (7, 1, 1), (8, 1, 8), (8, 2, 8), (8, 4, 1), (9, 1, 1), (11, 2, 1),
-                            (12, 2, 8), (16, 1, 8), (16, 8, 1), (17, 1, 1), (24, 1, 8)):
-        st, plan = create((256, 256), m)
-        same(st, 0)
-        u, y = (dmalloc(65536 * batch) for _ in range(2))
-        fake.fake_clear_launches()
-        same(lib.pce_apply(P(plan), P(u), P(y), batch, P(S1)), 0)
-        same((m, batch, [grid[2] for name, grid, block in launches() if "k_cols_fwd" in name]), (m, batch, [split]))
-        same(lib.pce_plan_destroy(P(plan)), 0)
+    for ny, cases in ((256, ((4, 1, 1), (5, 1, 1), (7, 1, 1), (8, 1, 8), (8, 2, 8), (8, 4, 1), (9, 1, 1), (11, 2, 1),
+                             (12, 2, 8), (16, 1, 8), (16, 4, 1), (17, 1, 1), (24, 1, 8), (28, 4, 4), (32, 8, 1))),
+                      (128, ((4, 1, 1), (8, 8, 8), (8, 16, 4), (9, 1, 4), (10, 1, 4), (12, 4, 8), (16, 24, 1)))):
+        for m, batch, split in cases:
+            st, plan = create((ny, ny), m)
+            same(st, 0)
+            u, y = (dmalloc(ny * ny * batch) for _ in range(2))
+            fake.fake_clear_launches()
+            same(lib.pce_apply(P(plan), P(u), P(y), batch, P(S1)), 0)
+            got = [grid[2] for name, grid, block in launches() if "k_cols_fwd" in name]
+            same((ny, m, batch, got), (ny, m, batch, [split]))
+            same(lib.pce_plan_destroy(P(plan)), 0)
     """)
