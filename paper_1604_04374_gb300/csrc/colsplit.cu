@@ -282,19 +282,20 @@ cudaError_t split_fwd_of(const ColArgs& c, cudaStream_t s, const float2* Z, long
 }  // namespace
 
 // Eight CTAs a tile, else four, while all are resident at once (four an SM), and only where they
-// repay the exchange: the rounds three quarters full (256^2, one right-hand side, in rounds
-// of eight: 8 terms 23.6 -> 20.6 us, 16 terms 32.8 -> 26.7, but 9 terms 24.6 -> 24.7), and four
-// CTAs where the chain is long: columns of 256 points from 28 terms on (4 right-hand sides: 16
-// terms 32.8 -> 34.6, 28 terms 47.2 -> 45.6, 64 terms 94.1 -> 85.8), of 64 points from 40 on
-// (64 x 2048, 2 right-hand sides: 32 terms 57.6 -> 59.0, 48 terms 77.0 -> 75.4), of the
-// other lengths, whose terms take longer one after another, from 8 on (128 x 256, 8 right-hand
-// sides: 8 terms 28.7 -> 25.1, 32 terms 73.7 -> 54.9).
+// repay the exchange.  Eight: from 8 terms on, at 256 points with five terms a round (256^2, one
+// right-hand side: 8 terms 23.6 -> 20.6 us, 16 terms 32.8 -> 26.7; two: 9 terms 24.6 -> 27.5;
+// fewer terms, so of four CTAs: 5 terms 20.5 -> 24.6; 64 x 128, reduced storage, 10 terms, 18
+// right-hand sides, both directions 61.4 -> 57.4).  Four: where the rounds are three quarters full and
+// the chain is long, at 256 points from 28 terms on (4 right-hand sides: 16 terms 32.8 ->
+// 34.6, 28 terms 47.2 -> 45.6, 64 terms 94.1 -> 85.8), at 64 from 40 on (64 x 2048, 2
+// right-hand sides: 32 terms 57.6 -> 59.0, 48 terms 77.0 -> 75.4), at the other lengths,
+// whose terms take longer one after another, from 8 on (128 x 256, 8 right-hand sides:
+// 8 terms 28.7 -> 25.1, 32 terms 73.7 -> 54.9).
 int cols_fwd_split(int ny, int m, long long ctas) {
     if (ny > 256) return 1;
-    for (int n : {8, 4}) {
-        const int rounds = (m + n - 1) / n, least = n == 8 ? 8 : ny == 256 ? 28 : ny == 64 ? 40 : 8;
-        if (m >= least && 4 * m >= 3 * n * rounds && ctas * n <= 4LL * kSms) return n;
-    }
+    const int r8 = (m + 7) / 8, r4 = (m + 3) / 4;   // rounds
+    if (m >= 8 && (ny < 256 || m >= 5 * r8) && ctas * 8 <= 4LL * kSms) return 8;
+    if (m >= (ny == 256 ? 28 : ny == 64 ? 40 : 8) && m >= 3 * r4 && ctas * 4 <= 4LL * kSms) return 4;
     return 1;
 }
 

@@ -133,9 +133,10 @@ def forward_split(ny, nx, nb, units, sep):
     ctas = nb * -(-(nx // 2) // cols)
     if sep:
         return 4 if units >= 4 and ctas * 4 <= 152 * (6 if ny == 512 else 4) else 1
-    for n, least in ((8, 8), (4, {256: 28, 64: 40}.get(ny, 8))):
-        if units >= least and 4 * units >= 3 * n * -(-units // n) and ctas * n <= 152 * 4:
-            return n
+    if units >= 8 and (ny < 256 or units >= 5 * -(-units // 8)) and ctas * 8 <= 152 * 4:
+        return 8
+    if units >= {256: 28, 64: 40}.get(ny, 8) and units >= 3 * -(-units // 4) and ctas * 4 <= 152 * 4:
+        return 4
     return 1
 
 

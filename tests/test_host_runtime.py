@@ -218,12 +218,12 @@ def test_column_splits_stay_within_one_wave(child, shape):
 
 
 def test_dense_forward_splits_where_its_rounds_are_full(child):
-    """Eight or four CTAs share a column tile's terms where the rounds are three quarters full,
-    the chain is long enough for the length and all CTAs are resident at once, none otherwise."""
+    """Eight or four CTAs share a column tile's terms where the rounds are full enough and the
+    chain is long enough for the length, and all CTAs are resident at once; none otherwise."""
     child("""
-    for ny, cases in ((256, ((4, 1, 1), (5, 1, 1), (7, 1, 1), (8, 1, 8), (8, 2, 8), (8, 4, 1), (9, 1, 1), (11, 2, 1),
-                             (12, 2, 8), (16, 1, 8), (16, 4, 1), (17, 1, 1), (24, 1, 8), (28, 4, 4), (32, 8, 1))),
-                      (128, ((4, 1, 1), (8, 8, 8), (8, 16, 4), (9, 1, 4), (10, 1, 4), (12, 4, 8), (16, 24, 1)))):
+    for ny, cases in ((256, ((4, 1, 1), (5, 1, 1), (7, 1, 1), (8, 1, 8), (8, 2, 8), (8, 4, 1), (9, 1, 1), (11, 2, 8),
+                             (12, 2, 8), (16, 1, 8), (16, 4, 1), (17, 1, 8), (24, 1, 8), (28, 4, 4), (32, 8, 1))),
+                      (128, ((4, 1, 1), (8, 8, 8), (8, 16, 4), (9, 1, 8), (9, 16, 4), (10, 16, 4), (12, 4, 8), (16, 24, 1)))):
         for m, batch, split in cases:
             st, plan = create((ny, ny), m)
             same(st, 0)
