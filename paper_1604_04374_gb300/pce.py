@@ -597,9 +597,9 @@ class Plan:
         return out
 
     def close(self):
-        if getattr(self, "handle", None):
-            pce_plan_destroy(self.handle)
-            self.handle = None
+        handle, self.handle = getattr(self, "handle", None), None   # gone even where the call fails
+        if handle:
+            pce_plan_destroy(handle)
 
     def __del__(self):
         try:
@@ -645,9 +645,9 @@ class Batch:
         _check(load_library().pce_batch_set_tuning(self.handle, col_policy, row_policy))
 
     def close(self):
-        if getattr(self, "handle", None):
-            pce_batch_destroy(self.handle)
-            self.handle = None
+        handle, self.handle = getattr(self, "handle", None), None   # gone even where the call fails
+        if handle:
+            pce_batch_destroy(handle)
         self._keep = []
 
     def __del__(self):

@@ -115,6 +115,43 @@ def test_a_plan_that_cannot_wait_keeps_its_memory(child, shape):
     """)
 
 
+def test_a_handle_is_destroyed_once(child):
+    """Plan.close() and Batch.close() give their handle up also where the call fails: a second
+    close, and the object's end, leave it alone."""
+    child("""
+    st, plan = create((256, 256), 4)
+    same(st, 0)
+    u, y = dmalloc(65536), dmalloc(65536)
+    obj = object.__new__(pce.Plan)
+    obj.handle = plan
+    same(lib.pce_apply(P(plan), P(u), P(y), 1, P(S2)), 0)
+    base = fake.fake_live_bytes()
+    fake.fake_set_capturing(1)
+    try:
+        obj.close()
+    except pce.PceError as e:
+        same(e.status, pce.PCE_ERR_CUDA)
+    else:
+        raise AssertionError("the destroy did not fail")
+    same(obj.handle, None)
+    fake.fake_set_capturing(0)
+    obj.close()
+    same(pool(), 0)
+    same(lib.pce_release_memory(), 0, fake.fake_unordered_frees(), 0)
+    assert pool() < 0
+    del obj
+    batch = object.__new__(pce.Batch)
+    batch.handle, batch._keep = 1, []
+    pce.pce_batch_destroy = lambda handle: (_ for _ in ()).throw(pce.PceError(4, "fails"))
+    try:
+        batch.close()
+    except pce.PceError:
+        pass
+    same(batch.handle, None)
+    batch.close()
+    """)
+
+
 @pytest.mark.parametrize("shape,m,flags,sep", [((512, 64), 3, 0, True), ((1024, 32), 2, 0, True),
                                                ((256, 64), 2, 0, False), ((1024, 64), 2, "SECTIONED", False),
                                                ((2048, 16), 2, "LOWP_STORAGE", False), ((2048,), 3, 0, False),
